@@ -51,7 +51,7 @@ WORKLOADS = {
     "rmat20-directed": ("directed R-MAT scale 20, edge factor 16, a=.57 b=.19 c=.19, weights U[1,255], "
                         "4096 uniform sources, ordered pairs, scale n/k", gen.workload_rmat20_directed),
     "grid1024-delta": ("perturbed 1024x1024 4-neighbour grid, 5% edges removed, weights U[1,10000], 1024 sources, "
-                       "delta-stepping schedule with DAG hop-depth levels", gen.workload_grid1024),
+                       "sweep schedule pinned", gen.workload_grid1024),
 }
 
 # per-workload options: edge output, directed graph, per-source schedule
@@ -105,7 +105,8 @@ def edge_units(g, opts):
 # per reached vertex 80 B.
 BYTES_PER_ENTRY = 64
 BYTES_PER_VERTEX = 80
-KERNEL_SRC = os.path.join(ROOT, "paper_1701_05975_gb300", "csrc", "bc_batched.cuh")
+# the kernel the benchmark workloads run and the primitives it is built from
+KERNEL_SRC = [os.path.join(ROOT, "paper_1701_05975_gb300", "csrc", f) for f in ("bc_sweep.cuh", "bc_team.cuh")]
 
 
 def reach_model(g, sources, directed=False, sample=32):
@@ -137,7 +138,7 @@ def reach_model(g, sources, directed=False, sample=32):
 
 
 def kernel_digest():
-    return hashlib.sha256(open(KERNEL_SRC, "rb").read()).hexdigest()[:16]
+    return hashlib.sha256(b"".join(open(f, "rb").read() for f in KERNEL_SRC)).hexdigest()[:16]
 
 
 def load_traffic(workload):
@@ -556,7 +557,7 @@ def main():
     ap.add_argument("--team", type=int, default=0, help="threads per source (0 = automatic / autotuned)")
     ap.add_argument("--width", type=int, default=0, help="near/far split width (0 = automatic / autotuned)")
     ap.add_argument("--algorithm", type=int, default=0, help="per-source schedule: 0 = automatic / autotuned, "
-                    "1 = strict, 2 = delta-stepping")
+                    "1 = strict, 2 = sweep")
     ap.add_argument("--warp-degree", type=int, default=0, help="rows with at least this many entries get a warp "
                     "(0 = automatic / autotuned)")
     ap.add_argument("--team-degree", type=int, default=0, help="rows with at least this many entries get the whole "
@@ -728,7 +729,7 @@ def main():
                    "graph_prep_s": round(prep_s, 3),
                    "launch": "CUDA graph (bc_step_launch)" if use_graph else (
                        "bc_edge_compute_async per step" if edge else "bc_compute_async per step"),
-                   "algorithm": "delta-stepping" if int(st.algorithm) == 2 else "strict",
+                   "algorithm": "sweep" if int(st.algorithm) == 2 else "strict",
                    "relabeled_by_degree": bool(G.info().relabeled), "dist_bits": int(G.info().dist_bits)},
         "e2e": {"value": whole_job_gteps(ws, k, m, e2e_s), "unit": "GTEPS", "h2d_bytes_per_step": 4 * k,
                 "d2h_bytes_per_step": 8 * g.n + (8 * g.nnz if edge else 0)},
@@ -738,7 +739,7 @@ def main():
                      "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
                      # ncu-measured DRAM bytes per launch over the same launch time
                      "frac_measured": (traffic / launch_avg_s / 1e9 / peak) if traffic else None,
-                     "alg_bytes_per_launch": alg_bytes, "kernel": "bc_batched_kernel"},
+                     "alg_bytes_per_launch": alg_bytes, "kernel": "bc_sweep_kernel" if int(st.algorithm) == 2 else "bc_batched_kernel"},
         "clocks": clk,
         "run_stats": {"phases_per_source": st.phases / max(st.sources, 1),
                       "refills_per_source": st.refills / max(st.sources, 1),

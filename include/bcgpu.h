@@ -67,13 +67,16 @@ extern "C" {
 #define BC_MODE_PLAIN 1u   /* one source at a time over the whole GPU, host-driven phase loop */
 
 /* ---- per-source schedules of the batched mode --------------------------- */
-#define BC_ALGO_AUTO 0u   /* the graph's tuned schedule, else BC_ALGO_STRICT */
+#define BC_ALGO_AUTO 0u   /* the graph's tuned schedule, else BC_ALGO_DELTA; BC_ALGO_STRICT while the configuration
+                             sets a knob that only that schedule has (settle_in, bucket_width, warp_degree,
+                             team_degree, hot_vertices) */
 #define BC_ALGO_STRICT 1u /* the paper's phases: settle every vertex that meets the strict OUT (Eq. 2 + Eq. 4) or
                              IN criterion, sigma pulled as each batch settles (Sec. 3.2, Algorithm 2) */
-#define BC_ALGO_DELTA 2u  /* distances by delta-stepping rounds (bucket width = bucket_width), then predecessor
-                             counts, sigma pushed down the shortest-path DAG in hop-depth levels, and the
-                             dependency pull of Algorithm 3 over those levels in reverse.  Same results; far
-                             fewer synchronised steps on high-diameter graphs. */
+#define BC_ALGO_DELTA 2u  /* sweep schedule: distances by rounds of frontier relaxation (bucket width =
+                             bucket_width), started from landmark bounds on graphs where those help; then the
+                             shortest-path DAG as compact lists, sigma pushed down it in hop-depth levels, and
+                             the dependency pull of Algorithm 3 over those levels in reverse.  Same results; far
+                             fewer synchronised steps, and only the entries that the landmark bounds leave. */
 
 /* ---- request states (bc_request_poll) ---------------------------------- */
 #define BC_REQ_QUEUED 0
@@ -93,7 +96,7 @@ typedef struct bc_config {
   uint32_t mode;          /* BC_MODE_BATCHED or BC_MODE_PLAIN */
   uint32_t team_threads;  /* threads that share one source: 32 (warp team) or 128/256/512/1024 (CTA team);
                              1024 needs 32-bit distances and falls back to 512 otherwise.  0 = tuned value,
-                             else by entries walked per vertex (>= 20: 1024 or 512, >= 6: 256, else 128) */
+                             else by average degree and vertex count */
   uint32_t max_slots;     /* cap on sources in flight at once (per-source slabs held in device memory) */
   uint32_t settle_in;     /* 1: settle by the strict OUT criterion (Eq. 2 + Eq. 4) OR the strict IN
                              criterion, each with Delta_node raised to the second smallest incident
@@ -102,7 +105,9 @@ typedef struct bc_config {
                              Delta_node (the paper's criterion alone); 3: OUT or IN with Delta_node;
                              0 = automatic (tuned, else 3) */
   uint64_t bucket_width;  /* near/far split width, in distance units (>= 1); 0 = tuned value, else the
-                             mean over non-empty rows of the row's smallest weight (Delta_node) */
+                             mean over non-empty rows of the row's smallest weight (Delta_node).  With
+                             BC_ALGO_DELTA the width of a distance bucket; 0 = tuned value, else one bucket
+                             under landmark bounds and 4 max_weight / (average degree) without */
   uint64_t phase_cap;     /* device cap on phases + queue refills per source; hitting it returns BC_ERR_TIMEOUT.
                              0 = automatic: 4n + 64, above what any valid input needs (phases <= n,
                              refills <= 3n + 2) */
@@ -271,8 +276,9 @@ int bc_serving_reset(void);
 
 /*
  * Test hook: distances (UINT64_MAX = unreachable), shortest-path counts and
- * the settle batch (level) of every vertex from one source, as the batched
- * path computes them (Algorithm 2 semantics, strict criterion).  HOST outputs
+ * the settle batch (level) of every vertex from one source, as the strict
+ * schedule computes them (Algorithm 2 semantics, strict criterion); with
+ * bc_config.algorithm = BC_ALGO_DELTA, the sweep schedule's hop-depth levels.  HOST outputs
  * of n entries each; any may be NULL.  Unreached vertices get level
  * UINT32_MAX.  Within a source, every shortest-path DAG edge (p -> v)
  * satisfies level[p] < level[v].
@@ -286,19 +292,19 @@ int bc_sssp_debug(bc_graph_t g, uint32_t s, uint64_t *out_dist, double *out_sigm
  */
 typedef struct bc_run_stats {
   uint64_t sources;
-  uint64_t phases;
-  uint64_t refills;
+  uint64_t phases;          /* settle batches (BC_ALGO_DELTA: relaxation rounds) */
+  uint64_t refills;         /* near-queue refills (BC_ALGO_DELTA: bucket advances) */
   uint64_t reached;
   uint64_t relax_atomics;
   uint64_t entries_scanned;
   uint32_t team_threads;
   uint32_t slots;
   uint64_t bucket_width;
-  uint64_t dag_edges;       /* shortest-path DAG edges recorded by the forward pass */
+  uint64_t dag_edges;       /* shortest-path DAG edges recorded by the forward pass (BC_ALGO_DELTA: list words) */
   uint64_t pair_overflows;  /* sources whose DAG edge list overflowed (backward fell back to a CSR scan) */
   uint64_t cycles_expand;   /* SM cycles summed over sources: frontier expansion (sigma pull + relax) */
-  uint64_t cycles_refill;   /* near-queue refills from the far queue */
-  uint64_t cycles_settle;   /* threshold + settle of the near queue */
+  uint64_t cycles_refill;   /* near-queue refills from the far queue (BC_ALGO_DELTA: landmark bounds, DAG lists) */
+  uint64_t cycles_settle;   /* threshold + settle of the near queue (BC_ALGO_DELTA: sigma levels) */
   uint64_t cycles_backward; /* dependency accumulation */
   uint64_t near_scanned;    /* near-queue entries read by threshold and settle */
   uint64_t far_scanned;     /* far-queue entries read by refills */
@@ -315,12 +321,12 @@ int bc_last_run_stats(bc_graph_t g, bc_run_stats *out);
  * Autotuner: times candidate settings on a probe sample of `sources`
  * (k_probe of them, HOST array) and stores the fastest as the graph's tuned
  * configuration, used whenever the process-wide config leaves a field at 0:
- * team size x bucket width (and the delta-stepping schedule where the strict
- * one needs 1000 or more phases per source), then the degree thresholds of
- * the forward expansion (warp_degree in {8, 16, 32, 64}, then team_degree in
- * {2, 8, 32} x team size; Sec. 3.4 studies the same trade-off as its
- * WARP_SIZE), then sources in flight (full or half capacity).  Results are
- * cached per graph fingerprint.
+ * the sweep schedule's team size x bucket width, then its sources in flight
+ * (full or half capacity); the strict schedule's team size x split width, and
+ * where that one is the faster its degree thresholds (warp_degree in {8, 16,
+ * 32, 64}, then team_degree in {2, 8, 32} x team size; Sec. 3.4 studies the
+ * same trade-off as its WARP_SIZE), settle test and sources in flight.
+ * Results are cached per graph fingerprint.
  */
 int bc_autotune(bc_graph_t g, const uint32_t *sources, uint32_t k_probe);
 

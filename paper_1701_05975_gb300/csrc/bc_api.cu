@@ -27,6 +27,15 @@ using namespace bcgpu;
 
 namespace {
 
+// Graphs of up to this many vertices run the sweep schedule from shared memory.
+#ifndef BCGPU_SWEEP_SMEM_N
+#define BCGPU_SWEEP_SMEM_N 2048u
+#endif
+constexpr uint32_t SWEEP_SMEM_N = BCGPU_SWEEP_SMEM_N;
+// The vertex bits are in shared memory while 1024 threads' worth of teams
+// keep theirs within this many bytes of an SM's 227 KB.
+constexpr uint32_t SWEEP_BITS_MAX = 212u << 10;
+
 thread_local std::string g_last_error;
 
 int fail(int code, const char* fmt, ...) {
@@ -63,39 +72,74 @@ bc_config config_snapshot() {
 
 uint64_t align256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
 
-SlabLayout make_layout(uint32_t n, int dist_bits) {
+// What a workspace's slabs hold: the layouts and the values their arrays keep
+// between sources differ by schedule.
+enum SlabKind : int { SLAB_STRICT = 0, SLAB_SWEEP = 1, SLAB_NONE = 2 };
+
+SlabLayout make_layout(uint32_t n, int dist_bits, SlabKind kind) {
   SlabLayout L{};
+  if (kind == SLAB_NONE) {  // every per-source array is in shared memory
+    L.stride = 256;
+    return L;
+  }
   uint64_t off = 0;
-  L.off_d = off;
-  off += align256((uint64_t)n * (dist_bits / 8));
-  L.off_sig = off;
-  off += align256((uint64_t)n * 8);
-  L.off_S = off;
-  off += align256((uint64_t)n * 4);
-  L.off_ends = off;
-  off += align256(((uint64_t)n + 2) * 4);
-  L.off_near = off;
-  off += align256((uint64_t)n * 4);
-  L.off_far = off;
-  off += align256((uint64_t)n * 4);
-  L.off_far2 = off;
-  off += align256((uint64_t)n * 4);
-  L.off_acc = off;
-  off += align256((uint64_t)n * 8);
-  L.off_pend = off;
-  off += align256(((uint64_t)n + 2) * 4);
+  auto take = [&](uint64_t bytes) {
+    const uint64_t at = off;
+    off += align256(bytes);
+    return at;
+  };
+  const uint64_t w = (uint64_t)n * 4, w2 = ((uint64_t)n + 2) * 4;
+  L.off_d = take((uint64_t)n * (dist_bits / 8));
+  if (kind == SLAB_SWEEP) {
+    L.off_sig = take((uint64_t)n * 16);
+    L.off_near = take(w2);
+    L.off_far = take(w2);
+    L.off_far2 = take(w);
+    L.off_ends = take(w);
+    L.off_S = take(w);
+    L.off_acc = take(w);
+    L.off_pend = take((((uint64_t)n + 31) / 32) * 12);
+    // DAG lists (two words per vertex with successors, then the successors):
+    // 8 n words cover six DAG edges per vertex; a source beyond that walks
+    // the rows again instead
+    L.pair_cap = (uint32_t)std::min<uint64_t>(8ull * n + 64, 0xffffffffull);
+    L.off_pairs = take(((uint64_t)L.pair_cap + 8) * 4);
+    L.stride = off;
+    return L;
+  }
+  L.off_sig = take((uint64_t)n * 8);
+  L.off_S = take(w);
+  L.off_ends = take(w2);
+  L.off_near = take(w);
+  L.off_far = take(w);
+  L.off_far2 = take(w);
+  L.off_acc = take((uint64_t)n * 8);
+  L.off_pend = take(w2);
   // DAG edge list: 2 n pairs covers every graph whose shortest-path DAG has at
   // most two in-edges per vertex on average (sources beyond it fall back to
   // the per-entry backward scan)
   L.pair_cap = (uint32_t)std::min<uint64_t>(2ull * n + 64, 0xffffffffull);
-  L.off_pairs = off;
-  off += align256((uint64_t)L.pair_cap * 8);
-  L.off_pc = off;
-  off += align256((uint64_t)n * 4);
-  L.off_pair_e = off;
-  off += align256((uint64_t)L.pair_cap * 4);
+  L.off_pairs = take((uint64_t)L.pair_cap * 8);
+  L.off_pair_e = take((uint64_t)L.pair_cap * 4);
   L.stride = off;
   return L;
+}
+
+// The values every slab holds between sources: distances INF, backward
+// accumulators (strict) or vertex records and bits (sweep) zero; other arrays are
+// written before they are read.
+cudaError_t init_slabs(char* slabs, const SlabLayout& lay, SlabKind kind, uint32_t slots, uint32_t n, int dist_bits,
+                       cudaStream_t st) {
+  if (kind == SLAB_NONE) return cudaSuccess;
+  cudaError_t e = launch_fill_slabs(slabs, lay.stride, slots, lay.off_d, align256((uint64_t)n * (dist_bits / 8)),
+                                    0xffffffffu, st);
+  if (e != cudaSuccess) return e;
+  if (kind == SLAB_SWEEP) {
+    e = launch_fill_slabs(slabs, lay.stride, slots, lay.off_sig, align256((uint64_t)n * 16), 0u, st);
+    if (e != cudaSuccess) return e;
+    return launch_fill_slabs(slabs, lay.stride, slots, lay.off_pend, align256((((uint64_t)n + 31) / 32) * 8), 0u, st);
+  }
+  return launch_fill_slabs(slabs, lay.stride, slots, lay.off_acc, align256((uint64_t)n * 8), 0u, st);
 }
 
 // Control block of one launch: source counter, status word, counters, debug.
@@ -109,6 +153,7 @@ struct Ctl {
 // Device memory for `slots` sources in flight plus per-call buffers.
 struct Workspace {
   uint32_t slots = 0;
+  SlabKind kind = SLAB_STRICT;
   SlabLayout lay{};
   char* slabs = nullptr;
   Ctl* ctl = nullptr;
@@ -124,13 +169,18 @@ struct Workspace {
 };
 
 struct TuneCfg {
+  // sweep schedule
+  uint32_t sweep_team = 0;
+  uint64_t sweep_width = 0;
+  uint32_t sweep_slots = 0;
+  // strict schedule
   uint32_t team = 0;
   uint64_t width = 0;
   uint32_t settle_in = 0;
   uint32_t max_slots = 0;  // 0: the full resident capacity
   uint32_t warp_deg = 0;
   uint32_t team_deg = 0;
-  uint32_t algo = 0;
+  uint32_t algo = 0;  // the faster schedule
 };
 
 std::mutex g_tune_mu;
@@ -163,6 +213,14 @@ struct bc_graph {
   uint32_t* o2n = nullptr;  // device maps (relabeled graphs only)
   uint32_t* n2o = nullptr;
   uint32_t* e2o = nullptr;
+  uint2* kadj = nullptr;        // landmark order of the rows (GraphDev)
+  uint32_t* kw = nullptr;
+  uint32_t* k2o = nullptr;
+  void* land_out = nullptr;
+  void* land_in = nullptr;      // undirected graphs: land_out
+  uint64_t land_stride = 0;
+  uint32_t land_bits = 0, nland = 0, land_n = 0;
+  uint32_t act_n = 0;           // vertices from this id on have no entries
   uint32_t* esm = nullptr;  // edge output: walked entry -> caller's output entry (built on first use)
   int esm_state = 0;        // 0 not built, 1 ready, 2 unavailable (an entry without a twin)
   std::vector<uint32_t> h_o2n;  // host copy of old -> new
@@ -200,6 +258,16 @@ GraphDev view(const bc_graph* g) {
   v.in_adj = g->in_adj;
   v.in_adjp = g->in_adjp;
   v.dnode_in = g->dnode_in;
+  v.kadj = g->kadj;
+  v.kw = g->kw;
+  v.k2o = g->k2o;
+  v.land_out = g->land_out;
+  v.land_in = g->land_in;
+  v.land_stride = g->land_stride;
+  v.land_bits = g->land_bits;
+  v.nland = g->nland;
+  v.land_n = g->land_n;
+  v.act_n = g->act_n;
   return v;
 }
 
@@ -235,10 +303,52 @@ struct RunCfg {
   uint32_t team_deg;
   uint32_t algo;  // ALGO_STRICT or ALGO_DELTA
   uint32_t hot_n;
+  SweepPlan sweep;  // ALGO_DELTA
 };
 
-RunCfg resolve(const bc_graph* g) {
+SlabKind slab_kind(const RunCfg& r) {
+  return r.algo != ALGO_DELTA ? SLAB_STRICT : (r.sweep.mem == 2 ? SLAB_NONE : SLAB_SWEEP);
+}
+
+// Kernel variant of the sweep schedule for `team` threads per source.
+void plan_sweep(const bc_graph* g, RunCfg& r, bool allow_smem) {
+  SweepPlan p;
+  p.dist_bits = g->dist_bits;
+  p.team = (int)r.team;
+  p.prune = g->kadj != nullptr;
+  const double avg_deg = g->n ? (double)g->nnz / g->n : 0.0;
+  p.group = (!p.prune && avg_deg >= 12.0) ? 8 : 1;
+  if (r.team >= 128) {
+    if (allow_smem && g->n <= SWEEP_SMEM_N) {
+      p.mem = 2;
+      p.group = 1;
+      p.succ_cap = 3 * g->n + 64;
+    } else if (sweep_smem(1, 32, g->act_n, 0) <= SWEEP_BITS_MAX * r.team / 1024) {
+      p.mem = 1;
+    }
+    p.smem_bytes = sweep_smem(p.mem, g->dist_bits, p.mem == 2 ? g->n : g->act_n, p.succ_cap);
+  }
+  r.sweep = p;
+}
+
+// Threads per source of the sweep schedule.
+uint32_t sweep_team_default(const bc_graph* g) {
+  const double avg_deg = g->n ? (double)g->nnz / g->n : 0.0;
+  if (avg_deg < 6.0 || g->n < 32768) return 256u;
+  return g->n < 131072 ? 512u : 1024u;
+}
+
+// Bucket width of the sweep schedule: one bucket where the landmark bounds
+// leave few vertices to relax; else 4 max_w / (average degree).
+uint64_t sweep_width_default(const bc_graph* g) {
+  if (g->kadj) return ~0ull;
+  const double avg_deg = g->n ? (double)g->nnz / g->n : 0.0;
+  return (uint64_t)std::max(1.0, 4.0 * g->max_w / std::max(avg_deg, 1.0));
+}
+
+RunCfg resolve(const bc_graph* g, uint32_t force_algo = BC_ALGO_AUTO) {
   bc_config c = config_snapshot();
+  if (force_algo) c.algorithm = force_algo;
   RunCfg r;
   r.mode = c.mode;
   // entries walked per vertex: a directed graph's batches walk in- and out-edges
@@ -249,10 +359,22 @@ RunCfg resolve(const bc_graph* g) {
   // graphs
   const uint32_t wide = g->dist_bits == 32 ? 1024u : 512u;
   const uint32_t team_default = avg_deg >= 20.0 ? wide : (avg_deg >= 6.0 ? 256u : 128u);
-  r.team = c.team_threads ? c.team_threads : (g->tuned.team ? g->tuned.team : team_default);
+  // the sweep schedule unless the configuration asks for the strict one or
+  // sets a knob that only the strict one has
+  const bool strict_knob = c.settle_in || c.bucket_width || c.warp_degree || c.team_degree || c.hot_vertices;
+  const uint32_t al = c.algorithm ? c.algorithm
+                                  : (strict_knob || g->n >= 0x80000000u || g->nnz + g->n >= (1ull << 32)
+                                     ? (uint32_t)BC_ALGO_STRICT
+                                     : (g->tuned.algo ? g->tuned.algo : (uint32_t)BC_ALGO_DELTA));
+  r.algo = (al == BC_ALGO_DELTA) ? ALGO_DELTA : ALGO_STRICT;
+  const bool sweep = r.algo == ALGO_DELTA;
+  const uint32_t tuned_team = sweep ? g->tuned.sweep_team : g->tuned.team;
+  r.team = c.team_threads ? c.team_threads
+                          : (tuned_team ? tuned_team : (sweep ? sweep_team_default(g) : team_default));
   if (r.team == 1024 && g->dist_bits != 32) r.team = 512;  // 1024-thread teams hold 32-bit distances only
+  const uint64_t tuned_width = sweep ? g->tuned.sweep_width : g->tuned.width;
   r.width = c.bucket_width ? c.bucket_width
-                           : (g->tuned.width ? g->tuned.width : g->width_default);
+                           : (tuned_width ? tuned_width : (sweep ? sweep_width_default(g) : g->width_default));
   // 1: OUT or IN with the settled-neighbour refinement; 2: OUT alone with
   // Delta_node (the paper's test); 3: OUT or IN with Delta_node (the default
   // until the autotuner has timed the refinement for this graph)
@@ -263,28 +385,37 @@ RunCfg resolve(const bc_graph* g) {
   // move entries <= n per queue level, empty refills <= second-level refills + 2:
   // phases + refills <= 4n + 2 (delta-stepping rounds + advances <= 3n)
   r.phase_cap = c.phase_cap ? c.phase_cap : 4ull * g->n + 64;
-  r.max_slots = c.max_slots ? c.max_slots : g->tuned.max_slots;
+  r.max_slots = c.max_slots ? c.max_slots : (sweep ? g->tuned.sweep_slots : g->tuned.max_slots);
   r.mem_fraction = c.mem_fraction > 0 ? c.mem_fraction : 0.6;
   r.warp_deg = c.warp_degree ? c.warp_degree : (g->tuned.warp_deg ? g->tuned.warp_deg : 32u);
   r.team_deg = c.team_degree ? c.team_degree : (g->tuned.team_deg ? g->tuned.team_deg : 8u * r.team);
   r.team_deg = std::max(r.team_deg, r.warp_deg);
-  const uint32_t al = c.algorithm ? c.algorithm : (g->tuned.algo ? g->tuned.algo : (uint32_t)BC_ALGO_STRICT);
-  r.algo = (al == BC_ALGO_DELTA) ? ALGO_DELTA : ALGO_STRICT;
   const uint32_t hot = c.hot_vertices ? c.hot_vertices : BCGPU_HOT_VERTICES;
   r.hot_n = g->relabeled ? std::min<uint32_t>(g->n, hot) : 0u;
+  plan_sweep(g, r, true);
   return r;
+}
+
+// Resident CTAs per SM of the run's kernel.
+cudaError_t run_occupancy(const bc_graph* g, const RunCfg& r, int* bps) {
+  return r.algo == ALGO_DELTA ? sweep_occupancy(r.sweep, bps) : batched_occupancy(g->dist_bits, (int)r.team, bps);
+}
+
+cudaError_t launch_run(const BatchArgs& a, const bc_graph* g, const RunCfg& r, int grid, cudaStream_t st) {
+  return r.algo == ALGO_DELTA ? launch_sweep(a, r.sweep, grid, st)
+                              : launch_batched(a, g->dist_bits, (int)r.team, grid, st);
 }
 
 // Number of sources in flight for a run of k sources.
 int plan_slots(const bc_graph* g, const RunCfg& r, uint32_t k, uint32_t* slots_out) {
   int bps = 0;
-  cudaError_t e = batched_occupancy(g->dist_bits, (int)r.team, (int)r.algo, &bps);
+  cudaError_t e = run_occupancy(g, r, &bps);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
   const uint32_t per_block = (uint32_t)(batched_block_threads((int)r.team) / (int)r.team);
   uint64_t slots = (uint64_t)std::max(bps, 1) * g->sm_count * per_block;
   size_t free_b = 0, total_b = 0;
   CK(cudaMemGetInfo(&free_b, &total_b));
-  const uint64_t stride = make_layout(g->n, g->dist_bits).stride;
+  const uint64_t stride = make_layout(g->n, g->dist_bits, slab_kind(r)).stride;
   const uint64_t by_mem = (uint64_t)((double)free_b * r.mem_fraction) / std::max<uint64_t>(stride, 1);
   slots = std::min<uint64_t>(slots, by_mem);
   if (r.max_slots) slots = std::min<uint64_t>(slots, r.max_slots);
@@ -297,33 +428,26 @@ int plan_slots(const bc_graph* g, const RunCfg& r, uint32_t k, uint32_t* slots_o
 
 // Acquire a free workspace with >= slots slabs and a source buffer >= k.
 // The caller's stream waits for the workspace's previous use.
-int ws_acquire(bc_graph* g, uint32_t slots, uint32_t k, cudaStream_t st, Workspace** out) {
+int ws_acquire(bc_graph* g, SlabKind kind, uint32_t slots, uint32_t k, cudaStream_t st, Workspace** out) {
   Workspace* w = nullptr;
   {
     std::lock_guard<std::mutex> lk(g->mu);
     for (auto& p : g->pool)
-      if (!p->busy && p->slots >= slots && (!w || p->slots < w->slots)) w = p.get();
+      if (!p->busy && p->kind == kind && p->slots >= slots && (!w || p->slots < w->slots)) w = p.get();
     if (w) w->busy = true;
   }
   if (!w) {
     auto nw = std::make_unique<Workspace>();
     nw->slots = slots;
-    nw->lay = make_layout(g->n, g->dist_bits);
+    nw->kind = kind;
+    nw->lay = make_layout(g->n, g->dist_bits, kind);
     const uint64_t bytes = nw->lay.stride * slots;
     cudaError_t e = cudaMalloc(&nw->slabs, bytes);
     if (e == cudaSuccess) e = cudaMalloc(&nw->ctl, sizeof(Ctl));
     if (e == cudaSuccess) e = cudaMalloc(&nw->bc, (size_t)g->n * 8);
     if (e == cudaSuccess) e = cudaMallocHost(&nw->host_ctl, sizeof(Ctl));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&nw->done, cudaEventDisableTiming);
-    // the slab invariant: every distance word is INF between sources
-    // and the backward accumulators are zero; other arrays are written before read
-    if (e == cudaSuccess)
-      e = launch_fill_slabs(nw->slabs, nw->lay.stride, slots, nw->lay.off_d,
-                            align256((uint64_t)g->n * (g->dist_bits / 8)), 0xffffffffu, st);
-    if (e == cudaSuccess)
-      e = launch_fill_slabs(nw->slabs, nw->lay.stride, slots, nw->lay.off_acc, align256((uint64_t)g->n * 8), 0u, st);
-    if (e == cudaSuccess)
-      e = launch_fill_slabs(nw->slabs, nw->lay.stride, slots, nw->lay.off_pc, align256((uint64_t)g->n * 4), 0u, st);
+    if (e == cudaSuccess) e = init_slabs(nw->slabs, nw->lay, kind, slots, g->n, g->dist_bits, st);
     if (e != cudaSuccess) {
       ws_free(nw.get());
       return cuda_fail(e, "workspace allocation");
@@ -489,7 +613,7 @@ BatchArgs make_args(bc_graph* g, Workspace* w, const RunCfg& r, const uint32_t* 
   a.debug_out = w->ctl->debug;
   a.warp_deg = r.warp_deg;
   a.team_deg = r.team_deg;
-  a.algo = r.algo;
+  a.sm_succ_cap = r.sweep.succ_cap;
   a.esm = (d_ebc && g->esm_state == 1) ? g->esm : nullptr;
   // the highest-degree vertices after relabeling: 128 KiB of 32-bit distance
   // words per source (the whole L2 holds this prefix for ~1000 sources)
@@ -510,7 +634,7 @@ int enqueue_batched(bc_graph* g, Workspace* w, const RunCfg& r, const uint32_t* 
   if (d_ebc) CK(cudaMemsetAsync(d_ebc, 0, (size_t)g->nnz * 8, st));
   if (check_src) CK(launch_check_sources(d_src, k, g->n, &w->ctl->err, st));
   BatchArgs a = make_args(g, w, r, d_src, k, d_bc, d_ebc, slots, flags);
-  CK(launch_batched(a, g->dist_bits, (int)r.team, grid_for_slots(r.team, slots), st));
+  CK(launch_run(a, g, r, grid_for_slots(r.team, slots), st));
   if (d_bc && scale != 1.0) CK(launch_scale(d_bc, g->n, scale, st));
   if (d_ebc && scale != 1.0) CK(launch_scale(d_ebc, g->nnz, scale, st));
   return BC_OK;
@@ -560,14 +684,14 @@ int compute_sync(bc_graph* g, const uint32_t* sources, uint32_t k, double scale,
                  const RunCfg& r) {
   for (uint32_t i = 0; i < k; ++i)
     if (sources[i] >= g->n) return fail(BC_ERR_INVALID, "source %u out of range (n = %u)", sources[i], g->n);
-  if (out_ebc)
+  if (out_ebc && r.algo == ALGO_STRICT)
     if (int rc = ensure_edge_map(g)) return rc;
   cudaStream_t st = g->stream;
   uint32_t slots = 0;
   int rc = plan_slots(g, r, k, &slots);
   if (rc) return rc;
   Workspace* w = nullptr;
-  if ((rc = ws_acquire(g, slots, k, st, &w))) return rc;
+  if ((rc = ws_acquire(g, slab_kind(r), slots, k, st, &w))) return rc;
   if (k) {
     memcpy(w->host_src, sources, (size_t)k * 4);
     cudaError_t e = cudaMemcpyAsync(w->src, w->host_src, (size_t)k * 4, cudaMemcpyHostToDevice, st);
@@ -718,6 +842,157 @@ std::string fingerprint(uint32_t n, uint64_t nnz, const uint64_t* rp, const uint
   return buf;
 }
 
+void free_landmarks(bc_graph* g) {
+  if (g->land_in != g->land_out) cudaFree(g->land_in);
+  cudaFree(g->land_out);
+  cudaFree(g->kadj);
+  cudaFree(g->kw);
+  cudaFree(g->k2o);
+  g->land_in = g->land_out = nullptr;
+  g->kadj = nullptr;
+  g->kw = g->k2o = nullptr;
+}
+
+// Landmarks of the sweep schedule: the highest-degree vertices.  Their exact
+// distances come from the schedule's own distance rounds (one launch over all
+// of them, unpruned).  A few probe sources then tell how many entries the main
+// landmark's prefix test would keep; above LAND_KEEP_MAX the graph keeps its
+// plain rows (random graphs keep 62%, grids all of them; R-MAT scale 20 keeps
+// 3%, Barabasi-Albert 65k 21%).  Undirected graphs must be symmetric for the
+// triangle inequality to hold in both directions.  Running out of device
+// memory here only means no landmarks.
+constexpr double LAND_KEEP_MAX = 0.5;
+constexpr uint32_t LAND_PROBES = 4;
+constexpr uint32_t LAND_MIN_N = 256;
+
+cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<uint64_t>& tdeg) {
+  const uint32_t n = g->n;
+  if (g->dist_bits != 32 || n < LAND_MIN_N || g->nnz == 0) return cudaSuccess;
+  const uint32_t L = std::min<uint32_t>(SWEEP_MAX_LAND, n / 16);
+  std::vector<uint32_t> ids(n);
+  for (uint32_t v = 0; v < n; ++v) ids[v] = v;
+  if (!g->relabeled)  // relabeled graphs number their vertices by decreasing degree already
+    std::partial_sort(ids.begin(), ids.begin() + L, ids.end(), [&](uint32_t a, uint32_t b) {
+      return tdeg[a] != tdeg[b] ? tdeg[a] > tdeg[b] : a < b;
+    });
+  ids.resize(L);
+  const uint32_t h = ids[0];
+  uint32_t probes = 0;
+  for (uint64_t i = 0, x = 12345; i < 64 && probes < LAND_PROBES; ++i) {
+    x = mix64(x + 0x9e3779b97f4a7c15ull);
+    const uint32_t v = (uint32_t)(x % n);
+    if (rp[v + 1] == rp[v]) continue;
+    ids.push_back(v);
+    ++probes;
+  }
+  if (probes == 0) return cudaSuccess;
+
+  std::vector<void*> temp;
+  auto alloc = [&](uint64_t bytes) -> void* {
+    void* p = nullptr;
+    if (cudaMalloc(&p, std::max<uint64_t>(bytes, 256)) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    temp.push_back(p);
+    return p;
+  };
+  cudaStream_t st = g->stream;
+  RunCfg r = resolve(g, BC_ALGO_DELTA);
+  r.team = n >= 16384 ? 1024u : 256u;
+  r.width = sweep_width_default(g);
+  r.phase_cap = 4ull * n + 64;
+  plan_sweep(g, r, true);
+  const uint32_t k = (uint32_t)ids.size();
+  int bps = 0;
+  cudaError_t e = run_occupancy(g, r, &bps);
+  if (e != cudaSuccess) return e;
+  const SlabKind kind = slab_kind(r);
+  const SlabLayout lay = make_layout(n, 32, kind);
+  size_t free_b = 0, total_b = 0;
+  if ((e = cudaMemGetInfo(&free_b, &total_b)) != cudaSuccess) return e;
+  const uint64_t dist_bytes = (uint64_t)k * n * 4;
+  uint64_t slots = std::min<uint64_t>(k, (uint64_t)std::max(bps, 1) * g->sm_count);
+  if (slots * lay.stride + 2 * dist_bytes + 28 * g->nnz > free_b / 2) return cudaSuccess;
+  char* slabs = static_cast<char*>(alloc(slots * lay.stride));
+  uint32_t* d_ids = static_cast<uint32_t*>(alloc(k * 4ull));
+  uint32_t* tab = static_cast<uint32_t*>(alloc(dist_bytes));
+  uint32_t* tab_in = g->directed ? static_cast<uint32_t*>(alloc((uint64_t)L * n * 4)) : tab;
+  // one control block per launch, then the symmetry sums, the judge's sums and the largest distance
+  Ctl* ctl = static_cast<Ctl*>(alloc(2 * sizeof(Ctl) + 8 * 8));
+  auto done = [&](cudaError_t err) {
+    for (void* p : temp) cudaFree(p);
+    if (err == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      free_landmarks(g);
+      return cudaSuccess;
+    }
+    return err;
+  };
+  if (!slabs || !d_ids || !tab || !tab_in || !ctl) return done(cudaErrorMemoryAllocation);
+  unsigned long long* sums = reinterpret_cast<unsigned long long*>(ctl + 2);
+  e = cudaMemsetAsync(ctl, 0, 2 * sizeof(Ctl) + 8 * 8, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(d_ids, ids.data(), k * 4ull, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = init_slabs(slabs, lay, kind, (uint32_t)slots, n, 32, st);
+  auto distances = [&](const GraphDev& gd, uint32_t count, uint32_t* out, Ctl* c) {
+    Workspace w;
+    w.lay = lay;
+    w.kind = kind;
+    w.slabs = slabs;
+    w.ctl = c;
+    BatchArgs a = make_args(g, &w, r, d_ids, count, nullptr, nullptr, (uint32_t)slots, RUN_DIST_ONLY);
+    a.g = gd;
+    a.g.o2n = nullptr;  // internal ids
+    a.dist_out = out;
+    a.stats = nullptr;
+    return launch_run(a, g, r, grid_for_slots(r.team, (uint32_t)slots), st);
+  };
+  const GraphDev fwd = view(g);
+  if (e == cudaSuccess) e = distances(fwd, k, tab, ctl);
+  if (e == cudaSuccess && g->directed) {
+    GraphDev rev = fwd;
+    rev.row_ptr = g->in_row_ptr;
+    rev.adj = g->in_adj;
+    e = distances(rev, L, tab_in, ctl + 1);
+  }
+  if (e == cudaSuccess && !g->directed) e = land_symmetry(fwd, sums, st);
+  if (e == cudaSuccess) e = land_judge(fwd, tab, tab + (uint64_t)L * n, h, probes, sums + 2, st);
+  if (e == cudaSuccess) e = land_max((uint64_t)L * n, tab, reinterpret_cast<uint32_t*>(sums + 6), st);
+  if (e == cudaSuccess && g->directed)
+    e = land_max((uint64_t)L * n, tab_in, reinterpret_cast<uint32_t*>(sums + 6), st);
+  std::vector<unsigned char> host(2 * sizeof(Ctl) + 8 * 8);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(host.data(), ctl, host.size(), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return done(e);
+  unsigned long long hs[7];
+  memcpy(hs, host.data() + 2 * sizeof(Ctl), sizeof hs);
+  const Ctl* hc = reinterpret_cast<const Ctl*>(host.data());
+  const uint32_t max_d = (uint32_t)hs[6];
+  if (hc[0].err != DEV_OK || hc[1].err != DEV_OK || hs[0] != hs[1]) return done(cudaSuccess);
+  if (hs[2] == 0 || (double)hs[3] > LAND_KEEP_MAX * (double)hs[2]) return done(cudaSuccess);
+
+  g->land_bits = max_d < 0x3fffu ? 16 : 32;  // every sum of two distances below 0x7fff
+  g->land_stride = ((uint64_t)n + 7) & ~7ull;
+  g->nland = L;
+  g->land_n = g->directed ? g->act_n : (uint32_t)hs[5];
+  const uint64_t tab_bytes = g->land_stride * L * (g->land_bits / 8);
+  unsigned long long* key = static_cast<unsigned long long*>(alloc(g->nnz * 8));
+  if (!key) return done(cudaErrorMemoryAllocation);
+  e = cudaMalloc(&g->land_out, tab_bytes);
+  if (e == cudaSuccess && g->directed) e = cudaMalloc(&g->land_in, tab_bytes);
+  if (!g->directed) g->land_in = g->land_out;
+  if (e == cudaSuccess) e = cudaMalloc(&g->kadj, g->nnz * 8);
+  if (e == cudaSuccess && !g->adjp) e = cudaMalloc(&g->kw, g->nnz * 4);
+  if (e == cudaSuccess) e = cudaMalloc(&g->k2o, g->nnz * 4);
+  if (e == cudaSuccess) e = land_pack(n, g->land_stride, L, tab, (int)g->land_bits, g->land_out, st);
+  if (e == cudaSuccess && g->directed)
+    e = land_pack(n, g->land_stride, L, tab_in, (int)g->land_bits, g->land_in, st);
+  if (e == cudaSuccess)
+    e = land_rows(fwd, tab, key, g->adjp ? g->col_bits : 0u, g->kadj, g->kw, g->k2o, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  return done(e);
+}
+
 }  // namespace
 
 int bcgpu::set_error(int code, const char* msg) { return fail(code, "%s", msg); }
@@ -731,6 +1006,7 @@ struct bcgpu::ServeLease {
   cudaEvent_t ev;    // recorded after each source batch
   uint32_t k;
   uint32_t slot_cap;  // slabs the lease holds
+  RunCfg r;           // settings at admission: the slabs belong to its schedule
 };
 
 int bcgpu::graph_device(const bc_graph* g) { return g->device; }
@@ -741,12 +1017,12 @@ void bcgpu::graph_serving_ref(bc_graph* g, int delta) { g->serving_refs += delta
 int bcgpu::serve_plan(bc_graph* g, ServePlan* out) {
   RunCfg r = resolve(g);
   int bps = 0;
-  cudaError_t e = batched_occupancy(g->dist_bits, (int)r.team, (int)r.algo, &bps);
+  cudaError_t e = run_occupancy(g, r, &bps);
   if (e != cudaSuccess) return cuda_fail(e, "occupancy");
   const uint32_t per_block = (uint32_t)(batched_block_threads((int)r.team) / (int)r.team);
   out->team = r.team;
   out->max_slots = (uint32_t)std::max(bps, 1) * (uint32_t)g->sm_count * per_block;
-  out->slot_bytes = make_layout(g->n, g->dist_bits).stride;
+  out->slot_bytes = make_layout(g->n, g->dist_bits, slab_kind(r)).stride;
   out->fixed_bytes = (uint64_t)g->n * 16 + 4096;
   return BC_OK;
 }
@@ -755,7 +1031,9 @@ int bcgpu::serve_open(bc_graph* g, const uint32_t* sources, uint32_t k, uint32_t
                       ServeLease** out) {
   Workspace* w = nullptr;
   const uint32_t cap = std::max<uint32_t>(slot_cap, 1);
-  int rc = ws_acquire(g, cap, k, st, &w);
+  RunCfg r = resolve(g);
+  r.mode = BC_MODE_BATCHED;
+  int rc = ws_acquire(g, slab_kind(r), cap, k, st, &w);
   if (rc) return rc;
   cudaError_t e = cudaSuccess;
   if (!w->host_bc) e = cudaMallocHost(&w->host_bc, (size_t)g->n * 8);
@@ -771,7 +1049,7 @@ int bcgpu::serve_open(bc_graph* g, const uint32_t* sources, uint32_t k, uint32_t
     ws_release(g, w, st);
     return cuda_fail(e, "serve_open");
   }
-  *out = new ServeLease{g, w, st, w->done, k, std::min(cap, w->slots)};
+  *out = new ServeLease{g, w, st, w->done, k, std::min(cap, w->slots), r};
   return BC_OK;
 }
 
@@ -781,8 +1059,7 @@ int bcgpu::serve_batch(ServeLease* l, uint32_t first, uint32_t count, uint32_t s
                        cudaStream_t st) {
   bc_graph* g = l->g;
   Workspace* w = l->w;
-  RunCfg r = resolve(g);
-  r.mode = BC_MODE_BATCHED;
+  const RunCfg& r = l->r;
   l->st = st;
   // the previous batch of this request (possibly on another stream) comes first
   cudaError_t e = cudaStreamWaitEvent(st, w->done, 0);
@@ -790,7 +1067,7 @@ int bcgpu::serve_batch(ServeLease* l, uint32_t first, uint32_t count, uint32_t s
   const uint32_t sl = std::max<uint32_t>(1, std::min<uint32_t>(slots, l->slot_cap));
   if (e == cudaSuccess) {
     BatchArgs a = make_args(g, w, r, w->src + first, count, w->bc, nullptr, sl, 0);
-    e = launch_batched(a, g->dist_bits, (int)r.team, grid_for_slots(r.team, sl), st);
+    e = launch_run(a, g, r, grid_for_slots(r.team, sl), st);
   }
   if (e == cudaSuccess && last && scale != 1.0) e = launch_scale(w->bc, g->n, scale, st);
   if (e == cudaSuccess && last)
@@ -984,6 +1261,10 @@ int bc_graph_create(const uint64_t* row_ptr, const uint32_t* col_idx, const uint
     }
     g->width_default = rows ? std::max<uint64_t>(1, (uint64_t)(sum / (double)rows + 0.5)) : 1;
   }
+  for (g->act_n = n; g->act_n > 0; --g->act_n) {
+    const uint32_t v = g->act_n - 1;
+    if (row_ptr[v + 1] > row_ptr[v] || (directed && irp[v + 1] > irp[v])) break;
+  }
   g->dist_bits = distance_bits(n, row_ptr, col_idx, w, max_w, directed);
   g->fingerprint = fingerprint(n, nnz, row_ptr, col_idx, w);
   {
@@ -1003,9 +1284,10 @@ int bc_graph_create(const uint64_t* row_ptr, const uint32_t* col_idx, const uint
   if (packed) {
     g->col_bits = col_bits;
     if (e == cudaSuccess) e = cudaMalloc(&g->adjp, std::max<size_t>(nnz, 1) * 4);
-  } else {
-    if (e == cudaSuccess) e = cudaMalloc(&g->adj, std::max<size_t>(nnz, 1) * 8);
   }
+  // {col, w} records: the strict schedule's entries where they do not pack,
+  // and the sweep schedule's rows unless they go into landmark order
+  if (e == cudaSuccess) e = cudaMalloc(&g->adj, std::max<size_t>(nnz, 1) * 8);
   if (e == cudaSuccess) e = cudaMalloc(&g->dnode, (size_t)n * 4);
   if (!directed) {
     if (e == cudaSuccess) e = cudaMalloc(&g->dnode2, (size_t)n * 4);
@@ -1037,7 +1319,7 @@ int bc_graph_create(const uint64_t* row_ptr, const uint32_t* col_idx, const uint
     if (e == cudaSuccess) e = cudaMalloc(&g->dnode_in, (size_t)n * 4);
     if (e == cudaSuccess) {
       if (packed) e = cudaMalloc(&g->in_adjp, std::max<size_t>(nnz, 1) * 4);
-      else e = cudaMalloc(&g->in_adj, std::max<size_t>(nnz, 1) * 8);
+      if (e == cudaSuccess) e = cudaMalloc(&g->in_adj, std::max<size_t>(nnz, 1) * 8);
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(g->in_row_ptr, irp.data(), ((size_t)n + 1) * 8, cudaMemcpyHostToDevice, g->stream);
     if (e == cudaSuccess && nnz) e = cudaMemcpyAsync(d_col, icol.data(), nnz * 4, cudaMemcpyHostToDevice, g->stream);
@@ -1049,7 +1331,17 @@ int bc_graph_create(const uint64_t* row_ptr, const uint32_t* col_idx, const uint
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
   cudaFree(d_col);
   cudaFree(d_w);
+  if (e == cudaSuccess) e = build_landmarks(g.get(), row_ptr, tdeg);
+  if (e == cudaSuccess && packed) {
+    if (g->kadj) {
+      cudaFree(g->adj);
+      g->adj = nullptr;
+    }
+    cudaFree(g->in_adj);
+    g->in_adj = nullptr;
+  }
   if (e != cudaSuccess) {
+    free_landmarks(g.get());
     cudaFree(g->row_ptr);
     cudaFree(g->adj);
     cudaFree(g->adjp);
@@ -1067,7 +1359,10 @@ int bc_graph_create(const uint64_t* row_ptr, const uint32_t* col_idx, const uint
     return cuda_fail(e, "bc_graph_create upload");
   }
   g->device_bytes = (((uint64_t)n + 1) * 8 + nnz * (packed ? 4 : 8) + (uint64_t)n * 4) * (directed ? 2 : 1) +
-                    (directed ? 0 : 8ull * n) + (relabel ? 8ull * n + 4ull * nnz : 0);
+                    (directed ? 0 : 8ull * n) + (relabel ? 8ull * n + 4ull * nnz : 0) +
+                    (packed && g->adj ? 8ull * nnz : 0) +
+                    (g->kadj ? (g->kw ? 16ull : 12ull) * nnz +
+                                   g->land_stride * g->nland * (g->land_bits / 8) * (directed ? 2 : 1) : 0);
   *out = g.release();
   return BC_OK;
 }
@@ -1085,6 +1380,7 @@ int bc_graph_destroy(bc_graph_t g) {
   g->pool.clear();
   plain_destroy(g->plain);
   paper_destroy(g->paper);
+  free_landmarks(g);
   cudaFree(g->row_ptr);
   cudaFree(g->adj);
   cudaFree(g->adjp);
@@ -1113,7 +1409,7 @@ int bc_graph_get_info(bc_graph_t g, bc_graph_info* out) {
   out->max_weight = g->max_w;
   out->dist_bits = (uint32_t)g->dist_bits;
   out->device_bytes = g->device_bytes;
-  out->slab_bytes = make_layout(g->n, g->dist_bits).stride;
+  out->slab_bytes = make_layout(g->n, g->dist_bits, slab_kind(resolve(g))).stride;
   out->relabeled = g->relabeled ? 1u : 0u;
   out->directed = g->directed ? 1u : 0u;
   return BC_OK;
@@ -1142,7 +1438,7 @@ int compute_async(bc_graph* g, const uint32_t* d_sources, uint32_t k, double sca
   CK(cudaSetDevice(g->device));
   RunCfg r = resolve(g);
   if (r.mode != BC_MODE_BATCHED) return fail(BC_ERR_INVALID, "the async entry points run the batched mode only");
-  if (d_out_ebc)
+  if (d_out_ebc && r.algo == ALGO_STRICT)
     if (int rc = ensure_edge_map(g)) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the workspace this stream kept from its previous async call: that run
@@ -1161,7 +1457,7 @@ int compute_async(bc_graph* g, const uint32_t* d_sources, uint32_t k, double sca
   int rc = plan_slots(g, r, k, &slots);
   if (rc) return rc;
   Workspace* w = nullptr;
-  if ((rc = ws_acquire(g, slots, 0, st, &w))) return rc;
+  if ((rc = ws_acquire(g, slab_kind(r), slots, 0, st, &w))) return rc;
   rc = enqueue_batched(g, w, r, d_sources, k, scale, d_out_bc, d_out_ebc, slots, 0, st, true);
   if (!rc) {
     cudaError_t e = cudaMemcpyAsync(w->host_ctl, w->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st);
@@ -1262,15 +1558,21 @@ int bc_sssp_debug(bc_graph_t g, uint32_t s, uint64_t* out_dist, double* out_sigm
   if (int rc = check_graph(g)) return rc;
   if (s >= g->n) return fail(BC_ERR_INVALID, "source out of range");
   CK(cudaSetDevice(g->device));
-  RunCfg r = resolve(g);
+  // the strict schedule's levels unless the sweep schedule is asked for by name
+  const bool sweep = config_snapshot().algorithm == BC_ALGO_DELTA;
+  RunCfg r = resolve(g, sweep ? BC_ALGO_DELTA : BC_ALGO_STRICT);
+  plan_sweep(g, r, false);  // the arrays are read back from a slab
   cudaStream_t st = g->stream;
   Workspace* w = nullptr;
-  int rc = ws_acquire(g, 1, 1, st, &w);
+  int rc = ws_acquire(g, slab_kind(r), 1, 1, st, &w);
   if (rc) return rc;
   w->host_src[0] = s;  // the kernel maps caller ids to internal ids
   const uint32_t n = g->n;
   std::vector<uint8_t> dbuf((size_t)n * (g->dist_bits / 8));
-  std::vector<double> sig(n);
+  const uint32_t sig_step = sweep ? 2 : 1;  // sigma leads a 16-byte record in the sweep schedule's slab
+  const uint64_t off_S = sweep ? w->lay.off_near : w->lay.off_S;
+  const uint64_t off_ends = sweep ? w->lay.off_far : w->lay.off_ends;
+  std::vector<double> sig((size_t)n * sig_step);
   std::vector<uint32_t> S(n), ends((size_t)n + 2);
   cudaError_t e = cudaMemcpyAsync(w->src, w->host_src, 4, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) {
@@ -1285,12 +1587,13 @@ int bc_sssp_debug(bc_graph_t g, uint32_t s, uint64_t* out_dist, double* out_sigm
   char* base = w->slabs;
   e = cudaMemcpyAsync(w->host_ctl, w->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dbuf.data(), base + w->lay.off_d, dbuf.size(), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(sig.data(), base + w->lay.off_sig, (size_t)n * 8, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(S.data(), base + w->lay.off_S, (size_t)n * 4, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(sig.data(), base + w->lay.off_sig, sig.size() * 8, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(S.data(), base + off_S, (size_t)n * 4, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(ends.data(), base + w->lay.off_ends, ((size_t)n + 2) * 4, cudaMemcpyDeviceToHost, st);
-  // restore the slab invariant (forward-only runs leave distances behind)
+    e = cudaMemcpyAsync(ends.data(), base + off_ends, ((size_t)n + 2) * 4, cudaMemcpyDeviceToHost, st);
+  // restore the slab invariant (forward-only runs leave distances and records behind)
   if (e == cudaSuccess) e = cudaMemsetAsync(base + w->lay.off_d, 0xff, dbuf.size(), st);
+  if (e == cudaSuccess && sweep) e = cudaMemsetAsync(base + w->lay.off_sig, 0, (size_t)n * 16, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   const Ctl c = *w->host_ctl;  // read before the workspace goes back to the pool
   ws_release(g, w, st);
@@ -1309,7 +1612,7 @@ int bc_sssp_debug(bc_graph_t g, uint32_t s, uint64_t* out_dist, double* out_sigm
       else if (g->dist_bits == 32) out_dist[ov] = reinterpret_cast<const uint32_t*>(dbuf.data())[v];
       else out_dist[ov] = reinterpret_cast<const uint64_t*>(dbuf.data())[v];
     }
-    if (out_sigma) out_sigma[ov] = reached_v ? sig[v] : 0.0;
+    if (out_sigma) out_sigma[ov] = reached_v ? sig[(size_t)v * sig_step] : 0.0;
     if (out_level) out_level[ov] = level[v];
   }
   return BC_OK;
@@ -1379,56 +1682,77 @@ int bc_autotune(bc_graph_t g, const uint32_t* sources, uint32_t k_probe) {
     *ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     return rc;
   };
-  RunCfg base = resolve(g);
-  base.mode = BC_MODE_BATCHED;
-  base.settle_in = 1;
-  base.refine = (g->dnode2 && user.settle_in == 1) ? 1u : 0u;
-  base.algo = (user.algorithm == BC_ALGO_DELTA) ? ALGO_DELTA : ALGO_STRICT;
-  // every candidate starts from the built-in thresholds (not a previous tuning)
-  base.warp_deg = user.warp_degree ? user.warp_degree : 32u;
-  auto team_deg_of = [&](uint32_t team, uint32_t warp_deg) {
-    return std::max(user.team_degree ? user.team_degree : 8u * team, warp_deg);
-  };
-  base.team_deg = team_deg_of(base.team, base.warp_deg);
-  double ms = 0;
-  if (int rc = timed(base, &ms)) return rc;  // warm-up: workspace allocation
-  double best_ms = 1e300;
-  double best_phases = 0;  // settle phases per source of the fastest strict candidate
   TuneCfg best;
-  for (uint32_t team : teams) {
-    if (user.team_threads && user.team_threads != team) continue;
-    if (user.algorithm == BC_ALGO_DELTA) break;
-    for (uint64_t width : widths) {
-      if (user.bucket_width && user.bucket_width != width) continue;
-      RunCfg r = base;
-      r.team = team;
-      r.width = width;
-      r.team_deg = team_deg_of(team, r.warp_deg);
-      if (int rc = timed(r, &ms)) return rc;
-      if (ms < best_ms) {
-        best_ms = ms;
-        best.team = team;
-        best.width = width;
-        best.settle_in = 3;
-        best.algo = BC_ALGO_STRICT;
-        std::lock_guard<std::mutex> lk(g->mu);
-        best_phases = g->last.sources ? (double)g->last.phases / (double)g->last.sources : 0.0;
-      }
-    }
-  }
-  // the delta-stepping schedule, buckets one to sixteen maximum weights wide:
-  // it walks every reached row about four times (rounds, predecessor count,
-  // sigma push, backward) against about once, so it is only a candidate where
-  // the strict schedule needs many settle phases per source (high diameter)
-  if (user.algorithm == BC_ALGO_DELTA || (user.algorithm == BC_ALGO_AUTO && best_phases >= 1000.0)) {
+  double ms = 0;
+  // a pinned schedule, or a knob that only the strict one has, leaves one schedule
+  const bool strict_knob = user.settle_in || user.warp_degree || user.team_degree || user.hot_vertices ||
+                           (user.bucket_width && user.algorithm != BC_ALGO_DELTA);
+  const bool try_sweep = user.algorithm == BC_ALGO_DELTA || (user.algorithm == BC_ALGO_AUTO && !strict_knob);
+  const bool try_strict = user.algorithm != BC_ALGO_DELTA;
+  // sweep schedule: team size x bucket width (one bucket under landmark
+  // bounds), then sources in flight
+  double sweep_ms = 1e300;
+  if (try_sweep) {
+    RunCfg base = resolve(g, BC_ALGO_DELTA);
+    base.mode = BC_MODE_BATCHED;
+    base.max_slots = user.max_slots;
+    if (int rc = timed(base, &ms)) return rc;  // warm-up: workspace allocation
+    const uint64_t w0 = sweep_width_default(g);
+    std::vector<uint64_t> sw = {w0};
+    if (!g->kadj) sw = {std::max<uint64_t>(1, w0 / 2), w0, 2 * w0, 4 * w0};
+    if (user.bucket_width) sw = {user.bucket_width};
     for (uint32_t team : teams) {
       if (user.team_threads && user.team_threads != team) continue;
-      if (!user.team_threads && best.team && team != best.team) continue;
-      for (uint64_t m : {1ull, 4ull, 16ull}) {
-        const uint64_t width = std::max<uint64_t>(1, g->max_w) * m;
+      for (uint64_t width : sw) {
+        RunCfg r = base;
+        r.team = team;
+        r.width = width;
+        plan_sweep(g, r, true);
+        if (int rc = timed(r, &ms)) return rc;
+        if (ms < sweep_ms) {
+          sweep_ms = ms;
+          best.sweep_team = team;
+          best.sweep_width = width;
+        }
+      }
+    }
+    if (best.sweep_team == 0 && !try_strict)
+      return fail(BC_ERR_INVALID, "autotune: the configuration pins every candidate out");
+    if (best.sweep_team && !user.max_slots) {
+      RunCfg r = base;
+      r.team = best.sweep_team;
+      r.width = best.sweep_width;
+      plan_sweep(g, r, true);
+      uint32_t full = 0;
+      if (int rc = plan_slots(g, r, k_probe, &full)) return rc;
+      r.max_slots = std::max<uint32_t>(1, full / 2);
+      if (int rc = timed(r, &ms)) return rc;
+      if (ms < sweep_ms) {
+        sweep_ms = ms;
+        best.sweep_slots = r.max_slots;
+      }
+    }
+    best.algo = BC_ALGO_DELTA;
+  }
+  if (try_strict) {
+    RunCfg base = resolve(g, BC_ALGO_STRICT);
+    base.mode = BC_MODE_BATCHED;
+    base.settle_in = 1;
+    base.refine = (g->dnode2 && user.settle_in == 1) ? 1u : 0u;
+    // every candidate starts from the built-in thresholds (not a previous tuning)
+    base.warp_deg = user.warp_degree ? user.warp_degree : 32u;
+    auto team_deg_of = [&](uint32_t team, uint32_t warp_deg) {
+      return std::max(user.team_degree ? user.team_degree : 8u * team, warp_deg);
+    };
+    base.team_deg = team_deg_of(base.team, base.warp_deg);
+    base.max_slots = user.max_slots;
+    if (int rc = timed(base, &ms)) return rc;  // warm-up: workspace allocation
+    double best_ms = 1e300;
+    for (uint32_t team : teams) {
+      if (user.team_threads && user.team_threads != team) continue;
+      for (uint64_t width : widths) {
         if (user.bucket_width && user.bucket_width != width) continue;
         RunCfg r = base;
-        r.algo = ALGO_DELTA;
         r.team = team;
         r.width = width;
         r.team_deg = team_deg_of(team, r.warp_deg);
@@ -1437,81 +1761,68 @@ int bc_autotune(bc_graph_t g, const uint32_t* sources, uint32_t k_probe) {
           best_ms = ms;
           best.team = team;
           best.width = width;
-          best.settle_in = 3;
-          best.algo = BC_ALGO_DELTA;
         }
       }
     }
-  }
-  if (best.team == 0) return fail(BC_ERR_INVALID, "autotune: the configuration pins every candidate out");
-  // degree thresholds of the strict schedule's expansion tiers: first the
-  // warp threshold, then the team threshold (as a multiple of the team size)
-  if (best.algo == BC_ALGO_STRICT) {
-    RunCfg r = base;
-    r.team = best.team;
-    r.width = best.width;
-    if (!user.warp_degree) {
-      uint32_t best_wd = r.warp_deg;
-      for (uint32_t wd : {8u, 16u, 32u, 64u}) {
-        if (wd == r.warp_deg) continue;  // the built-in value was timed with the team and width above
-        r.warp_deg = wd;
-        r.team_deg = team_deg_of(r.team, wd);
+    if (best.team == 0 && best.sweep_team == 0)
+      return fail(BC_ERR_INVALID, "autotune: the configuration pins every candidate out");
+    if (best_ms < sweep_ms || !try_sweep) best.algo = BC_ALGO_STRICT;
+    best.settle_in = 3;
+    // the strict schedule's finer settings matter only where it is the one that runs
+    if (best.team && best.algo == BC_ALGO_STRICT) {
+      RunCfg r = base;
+      r.team = best.team;
+      r.width = best.width;
+      // degree thresholds of the expansion tiers: first the warp threshold,
+      // then the team threshold (as a multiple of the team size)
+      best.warp_deg = r.warp_deg;
+      if (!user.warp_degree)
+        for (uint32_t wd : {8u, 16u, 64u}) {  // the built-in 32 was timed with the team and width above
+          r.warp_deg = wd;
+          r.team_deg = team_deg_of(r.team, wd);
+          if (int rc = timed(r, &ms)) return rc;
+          if (ms < best_ms) {
+            best_ms = ms;
+            best.warp_deg = wd;
+          }
+        }
+      r.warp_deg = best.warp_deg;
+      const uint32_t td0 = team_deg_of(r.team, r.warp_deg);
+      uint32_t best_td = td0;
+      if (!user.team_degree)
+        for (uint32_t mult : {2u, 32u}) {
+          r.team_deg = std::max(mult * r.team, r.warp_deg);
+          if (int rc = timed(r, &ms)) return rc;
+          if (ms < best_ms) {
+            best_ms = ms;
+            best_td = r.team_deg;
+          }
+        }
+      r.team_deg = best_td;
+      if (best_td != td0) best.team_deg = best_td;
+      // the settle test with the settled-neighbour refinement of Delta_node:
+      // fewer, larger batches (high-diameter graphs) against one more gather
+      // per candidate and settle pass (dense graphs)
+      if (!user.settle_in && g->dnode2) {
+        r.refine = 1;
         if (int rc = timed(r, &ms)) return rc;
         if (ms < best_ms) {
           best_ms = ms;
-          best_wd = wd;
+          best.settle_in = 1;
         }
+        r.refine = best.settle_in == 1 ? 1u : 0u;
       }
-      r.warp_deg = best_wd;
-      r.team_deg = team_deg_of(r.team, best_wd);
-      best.warp_deg = best_wd;
-    }
-    if (!user.team_degree) {
-      uint32_t best_td = 0;
-      for (uint32_t mult : {2u, 32u}) {
-        r.team_deg = std::max(mult * r.team, r.warp_deg);
+      // sources in flight: the full resident capacity, or half of it
+      if (!user.max_slots) {
+        uint32_t full = 0;
+        if (int rc = plan_slots(g, r, k_probe, &full)) return rc;
+        r.max_slots = std::max<uint32_t>(1, full / 2);
         if (int rc = timed(r, &ms)) return rc;
         if (ms < best_ms) {
           best_ms = ms;
-          best_td = r.team_deg;
+          best.max_slots = r.max_slots;
         }
       }
-      if (best_td) best.team_deg = best_td;
-    }
-  }
-  // the settle test with the settled-neighbour refinement of Delta_node:
-  // fewer, larger batches (high-diameter graphs) against one more gather per
-  // candidate and settle pass (dense graphs)
-  if (best.algo == BC_ALGO_STRICT && !user.settle_in) best.settle_in = 3;
-  if (!user.settle_in && g->dnode2 && best.algo == BC_ALGO_STRICT) {
-    RunCfg r = base;
-    r.team = best.team;
-    r.width = best.width;
-    if (best.warp_deg) r.warp_deg = best.warp_deg;
-    r.team_deg = best.team_deg ? best.team_deg : team_deg_of(r.team, r.warp_deg);
-    r.refine = 1;
-    if (int rc = timed(r, &ms)) return rc;
-    if (ms < best_ms) {
-      best_ms = ms;
-      best.settle_in = 1;
-    }
-  }
-  // sources in flight: the full resident capacity, or half of it
-  if (!user.max_slots) {
-    RunCfg r = base;
-    r.team = best.team;
-    r.width = best.width;
-    r.algo = best.algo == BC_ALGO_DELTA ? ALGO_DELTA : ALGO_STRICT;
-    if (best.warp_deg) r.warp_deg = best.warp_deg;
-    r.team_deg = best.team_deg ? best.team_deg : team_deg_of(r.team, r.warp_deg);
-    r.refine = best.settle_in == 1 ? 1u : 0u;
-    uint32_t full = 0;
-    if (int rc = plan_slots(g, r, k_probe, &full)) return rc;
-    r.max_slots = std::max<uint32_t>(1, full / 2);
-    if (int rc = timed(r, &ms)) return rc;
-    if (ms < best_ms) {
-      best_ms = ms;
-      best.max_slots = r.max_slots;
     }
   }
   g->tuned = best;
@@ -1561,7 +1872,8 @@ int bc_step_create(bc_graph_t g, const uint32_t* d_sources, uint32_t k, double s
   if (int rc = plan_slots(g, r, k, &s->slots)) return rc;
   Workspace& w = s->ws;
   w.slots = s->slots;
-  w.lay = make_layout(g->n, g->dist_bits);
+  w.kind = slab_kind(r);
+  w.lay = make_layout(g->n, g->dist_bits, w.kind);
   w.bytes = w.lay.stride * s->slots;
   cudaStream_t cap = nullptr;
   cudaError_t e = cudaMalloc(&w.slabs, w.bytes);
@@ -1569,13 +1881,7 @@ int bc_step_create(bc_graph_t g, const uint32_t* d_sources, uint32_t k, double s
   if (e == cudaSuccess) e = cudaMallocHost(&w.host_ctl, sizeof(Ctl));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
   // the slab invariant, established once: later runs restore it themselves
-  if (e == cudaSuccess)
-    e = launch_fill_slabs(w.slabs, w.lay.stride, s->slots, w.lay.off_d,
-                          align256((uint64_t)g->n * (g->dist_bits / 8)), 0xffffffffu, cap);
-  if (e == cudaSuccess)
-    e = launch_fill_slabs(w.slabs, w.lay.stride, s->slots, w.lay.off_acc, align256((uint64_t)g->n * 8), 0u, cap);
-  if (e == cudaSuccess)
-    e = launch_fill_slabs(w.slabs, w.lay.stride, s->slots, w.lay.off_pc, align256((uint64_t)g->n * 4), 0u, cap);
+  if (e == cudaSuccess) e = init_slabs(w.slabs, w.lay, w.kind, s->slots, g->n, g->dist_bits, cap);
   if (e == cudaSuccess) e = cudaStreamSynchronize(cap);
   if (e != cudaSuccess) {
     if (cap) cudaStreamDestroy(cap);

@@ -23,10 +23,9 @@
 // Every CSR walk uses a load-balanced edge-parallel chunk: the team takes up
 // to TEAM frontier vertices, scans their degrees and spreads the chunk's edges
 // evenly over its threads, so hubs never serialise one thread or warp.
-// This header holds the device code; bc_batched.cu instantiates the strict
-// schedule and bc_batched_delta.cu the delta-stepping one, so the two compile
-// in parallel.  Everything is in an anonymous namespace: each translation unit
-// owns its instantiations.
+// This header holds the device code of the strict schedule (bc_batched.cu
+// instantiates it); the sweep schedule is in bc_sweep.cuh.  Everything is in an
+// anonymous namespace: each translation unit owns its instantiations.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -34,12 +33,11 @@
 #include <type_traits>
 
 #include "bc_common.h"
+#include "bc_team.cuh"
 
 namespace bcgpu {
 namespace {
 
-constexpr unsigned FULL = 0xffffffffu;
-constexpr uint32_t NONE = 0xffffffffu;
 #ifndef BCGPU_UNROLL
 #define BCGPU_UNROLL 4
 #endif
@@ -63,17 +61,6 @@ constexpr int NEAR_MID = 8;
 #endif
 constexpr uint64_t FAR_LEVELS = BCGPU_FAR_LEVELS;   // the second far level starts FAR_LEVELS split widths out
 
-template <typename D>
-__device__ __forceinline__ D dinf() {
-  return ~D(0);
-}
-
-__device__ __forceinline__ uint32_t ldcg(const uint32_t* p) { return __ldcg(p); }
-__device__ __forceinline__ uint64_t ldcg(const uint64_t* p) {
-  return (uint64_t)__ldcg(reinterpret_cast<const unsigned long long*>(p));
-}
-__device__ __forceinline__ double ldcg(const double* p) { return __ldcg(p); }
-
 // Gathers of a team's own slab (distances, sigma).  A slab is private to one
 // CTA and every read is ordered after the writes it must see by the team's
 // barrier, so L1-cacheable loads are valid; BCGPU_GATHER_L1=0 keeps them in L2.
@@ -89,36 +76,9 @@ __device__ __forceinline__ T ldg_slab(const T* p) {
 #endif
 }
 
-__device__ __forceinline__ uint32_t atomic_min_d(uint32_t* p, uint32_t v) { return atomicMin(p, v); }
-__device__ __forceinline__ uint64_t atomic_min_d(uint64_t* p, uint64_t v) {
-  return (uint64_t)atomicMin(reinterpret_cast<unsigned long long*>(p), (unsigned long long)v);
-}
-
 // FAR_LEVELS split widths, saturating (a caller may set any width)
 __device__ __forceinline__ uint64_t far_span(uint64_t width) {
   return width > ~0ull / FAR_LEVELS ? ~0ull : FAR_LEVELS * width;
-}
-
-template <typename D>
-__device__ __forceinline__ D sat_add(D a, uint64_t b) {
-  uint64_t lim = (uint64_t)dinf<D>() - 1;
-  uint64_t aa = (uint64_t)a;
-  if (aa >= lim || b >= lim - aa) return (D)lim;
-  return (D)(aa + b);
-}
-
-template <typename D>
-__device__ __forceinline__ D shfl_xor_d(D x, int o) {
-  return __shfl_xor_sync(FULL, x, o);
-}
-
-template <typename D>
-__device__ __forceinline__ D dmin(D a, D b) {
-  return a < b ? a : b;
-}
-template <typename D>
-__device__ __forceinline__ D dmax(D a, D b) {
-  return a < b ? b : a;
 }
 
 // d + Delta_node for the OUT threshold (Eq. 2); a vertex without out-edges
@@ -155,134 +115,9 @@ struct TeamShared {
   Idx tlist[TEAM];
   uint32_t wnext, nwl, ntl;
   uint32_t staged;  // leading entries of the next batch already in vtx / rs / dg / dv
-  // delta-stepping schedule
-  uint32_t front_len, def_len, lvl_len, round;
-  uint32_t* front_out;
-  D bound;
   D red[2 * (TEAM / 32) + 2];
   uint32_t scan[2 * (TEAM / 32 + 1)];
 };
-
-template <int TEAM>
-__device__ __forceinline__ void team_sync() {
-  if constexpr (TEAM == 32) {
-    __syncwarp();
-  } else {
-    __syncthreads();
-  }
-}
-
-__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t y = __shfl_up_sync(FULL, x, o);
-    if (lane >= o) x += y;
-  }
-  return x;
-}
-
-// Exclusive prefix sum over the team; *total receives the team-wide sum.
-// Every thread of the team must call it.
-template <int TEAM>
-__device__ __forceinline__ uint32_t team_excl_scan(uint32_t x, uint32_t* total, uint32_t* scratch) {
-  uint32_t inc = warp_incl_scan(x);
-  if constexpr (TEAM == 32) {
-    *total = __shfl_sync(FULL, inc, 31);
-    return inc - x;
-  } else {
-    constexpr int NW = TEAM / 32;
-    const int w = (threadIdx.x % TEAM) >> 5, lane = threadIdx.x & 31;
-    if (lane == 31) scratch[w] = inc;
-    __syncthreads();
-    if (w == 0) {
-      uint32_t v = lane < NW ? scratch[lane] : 0u;
-      uint32_t vi = warp_incl_scan(v);
-      if (lane < NW) scratch[lane] = vi - v;
-      if (lane == NW - 1) scratch[NW] = vi;
-    }
-    __syncthreads();
-    *total = scratch[NW];
-    uint32_t r = scratch[w] + inc - x;
-    __syncthreads();
-    return r;
-  }
-}
-
-// Two exclusive prefix sums at once (shares the barriers).
-template <int TEAM>
-__device__ __forceinline__ void team_excl_scan2(uint32_t x, uint32_t y, uint32_t* ex, uint32_t* ey, uint32_t* tx,
-                                                uint32_t* ty, uint32_t* scratch) {
-  const uint32_t ix = warp_incl_scan(x), iy = warp_incl_scan(y);
-  if constexpr (TEAM == 32) {
-    *tx = __shfl_sync(FULL, ix, 31);
-    *ty = __shfl_sync(FULL, iy, 31);
-    *ex = ix - x;
-    *ey = iy - y;
-  } else {
-    constexpr int NW = TEAM / 32;
-    const int w = (threadIdx.x % TEAM) >> 5, lane = threadIdx.x & 31;
-    if (lane == 31) {
-      scratch[w] = ix;
-      scratch[NW + 1 + w] = iy;
-    }
-    __syncthreads();
-    if (w == 0) {
-      const uint32_t vx = lane < NW ? scratch[lane] : 0u, vy = lane < NW ? scratch[NW + 1 + lane] : 0u;
-      const uint32_t sx = warp_incl_scan(vx), sy = warp_incl_scan(vy);
-      if (lane < NW) {
-        scratch[lane] = sx - vx;
-        scratch[NW + 1 + lane] = sy - vy;
-      }
-      if (lane == NW - 1) {
-        scratch[NW] = sx;
-        scratch[2 * NW + 1] = sy;
-      }
-    }
-    __syncthreads();
-    *tx = scratch[NW];
-    *ty = scratch[2 * NW + 1];
-    *ex = scratch[w] + ix - x;
-    *ey = scratch[NW + 1 + w] + iy - y;
-    __syncthreads();
-  }
-}
-
-// Team-wide minimum of two values at once.
-template <typename D, int TEAM>
-__device__ __forceinline__ void team_min2(D& a, D& b, D* scratch) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a = dmin(a, shfl_xor_d(a, o));
-    b = dmin(b, shfl_xor_d(b, o));
-  }
-  if constexpr (TEAM > 32) {
-    constexpr int NW = TEAM / 32;
-    const int w = (threadIdx.x % TEAM) >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) {
-      scratch[w] = a;
-      scratch[NW + w] = b;
-    }
-    __syncthreads();
-    if (w == 0) {
-      D x = lane < NW ? scratch[lane] : dinf<D>();
-      D y = lane < NW ? scratch[NW + lane] : dinf<D>();
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        x = dmin(x, shfl_xor_d(x, o));
-        y = dmin(y, shfl_xor_d(y, o));
-      }
-      if (lane == 0) {
-        scratch[2 * NW] = x;
-        scratch[2 * NW + 1] = y;
-      }
-    }
-    __syncthreads();
-    a = scratch[2 * NW];
-    b = scratch[2 * NW + 1];
-    __syncthreads();
-  }
-}
 
 // L2 residency hints.  The distance words of the highest-degree vertices (a
 // prefix of the ids after relabeling) are gathered by most edges and are
@@ -391,7 +226,6 @@ struct Slab {
   uint32_t* pend;   // pend[l] = end of level l's DAG edges in pairs
   uint2* pairs;     // DAG edges {predecessor u, vertex v}
   uint32_t pair_cap;
-  uint32_t* pc;     // delta-stepping: round stamps, then predecessor counts (zero between sources)
   uint32_t* pair_e; // edge output: the walked entry of each DAG edge, else nullptr
 };
 
@@ -410,7 +244,6 @@ __device__ __forceinline__ Slab<D> slab_at(const BatchArgs& a, uint32_t slot) {
   s.pend = reinterpret_cast<uint32_t*>(base + a.lay.off_pend);
   s.pairs = reinterpret_cast<uint2*>(base + a.lay.off_pairs);
   s.pair_cap = a.lay.pair_cap;
-  s.pc = reinterpret_cast<uint32_t*>(base + a.lay.off_pc);
   s.pair_e = (a.ebc && a.esm && a.lay.off_pair_e) ? reinterpret_cast<uint32_t*>(base + a.lay.off_pair_e) : nullptr;
   return s;
 }
@@ -458,11 +291,7 @@ __device__ __forceinline__ uint32_t owner_of(const uint32_t* off, uint32_t cnt, 
 // Walk modes: an undirected row serves both the sigma pull and the
 // relaxation; a directed graph pulls over its in-edges and relaxes over its
 // out-edges in two walks.
-// The delta-stepping schedule adds three walks: relaxation into the next
-// round's frontier (WALK_DS), counting each vertex's predecessors once the
-// distances are final (WALK_COUNT), and pushing sigma down the DAG level by
-// level (WALK_KAHN).
-enum : int { WALK_BOTH = 0, WALK_PULL = 1, WALK_RELAX = 2, WALK_DS = 3, WALK_COUNT = 4, WALK_KAHN = 5 };
+enum : int { WALK_BOTH = 0, WALK_PULL = 1, WALK_RELAX = 2 };
 
 template <typename D, int TEAM, int MODE>
 __device__ __forceinline__ void visit_entry(const Slab<D>& sl, TeamShared<D, TEAM>& sh, uint32_t i, uint2 ent, D du,
@@ -474,33 +303,6 @@ __device__ __forceinline__ void visit_entry(const Slab<D>& sl, TeamShared<D, TEA
   const uint32_t u = ent.x;
   const D w = (D)ent.y;
   const D dvi = sh.dv[i];
-  if constexpr (MODE == WALK_DS) {
-    const D nd = dvi + w;
-    if (nd < du) {
-      ++relax;
-      const D old = atomic_min_d(&sl.d[u], nd);
-      if (nd < old) {
-        if (old == INF) sl.S[atomicAdd(&sh.S_len, 1u)] = u;  // reached list
-        if (nd < sh.bound) {
-          // once per round in the next frontier (stamp = that round)
-          if (atomicExch(&sl.pc[u], sh.round) != sh.round) sh.front_out[atomicAdd(&sh.front_len, 1u)] = u;
-        } else if (old == INF) {
-          sl.farq2[atomicAdd(&sh.def_len, 1u)] = u;  // deferred to a later bucket
-        }
-      }
-    }
-    return;
-  } else if constexpr (MODE == WALK_COUNT) {
-    if (du != INF && du + w == dvi) atomicAdd(&sh.acc[i], 1.0);
-    return;
-  } else if constexpr (MODE == WALK_KAHN) {
-    if (du != INF && du == dvi + w) {
-      // u is a successor: push sigma; the last predecessor releases u
-      atomicAdd(&sl.sig[u], sh.sv[i]);
-      if (atomicSub(&sl.pc[u], 1u) == 1u) sl.ends[atomicAdd(&sh.lvl_len, 1u)] = u;
-    }
-    return;
-  }
   if (MODE != WALK_RELAX && du != INF && du + w == dvi) {
 #if BCGPU_HOT_SIG
     atomicAdd(&sh.acc[i], gather_sig(sl.sig, u, hot_n, pol_last));
@@ -596,7 +398,6 @@ __device__ void expand_forward(const BatchArgs& a, const Rows& rows, const Slab<
         sh.dv[t] = ldcg(&sl.d[v]);
       }
       sh.acc[t] = 0.0;
-      if (MODE == WALK_KAHN) sh.sv[t] = ldcg(&sl.sig[sh.vtx[t]]);
       if (deg >= team_deg) is_t = 1;
       else if (deg >= warp_deg) is_w = 1;
       else small = deg;
@@ -662,11 +463,6 @@ __device__ void expand_forward(const BatchArgs& a, const Rows& rows, const Slab<
     team_sync<TEAM>();
     if ((MODE == WALK_BOTH || MODE == WALK_PULL) && (uint32_t)t < cnt && sh.vtx[t] != s)
       sl.sig[sh.vtx[t]] = sh.acc[t];
-    if (MODE == WALK_COUNT && (uint32_t)t < cnt) {
-      const uint32_t v = sh.vtx[t];
-      sl.pc[v] = (uint32_t)sh.acc[t];
-      sl.sig[v] = (v == s) ? 1.0 : 0.0;
-    }
     team_sync<TEAM>();
   }
 }
@@ -1232,201 +1028,6 @@ __device__ bool run_source(const BatchArgs& a, const Slab<D>& sl, TeamShared<D, 
 }
 
 
-// Delta-stepping schedule (ALGO_DELTA), for graphs whose strict settle batches
-// are many and small (high diameter):
-//   1. exact distances by delta-stepping rounds: the frontier relaxes its
-//      out-edges; improved vertices below the bucket bound form the next
-//      round's frontier (each at most once per round), the rest wait in a
-//      deferred list until the bound advances;
-//   2. one walk counts each reached vertex's shortest-path predecessors;
-//   3. sigma is pushed down the shortest-path DAG level by level (Kahn's
-//      order): a vertex joins the next level when its last predecessor has
-//      pushed to it, so a level holds vertices of equal DAG hop depth and no
-//      DAG edge lies inside a level (FP64 atomic sums of integer counts are
-//      exact below 2^53);
-//   4. Algorithm 3 over those levels in reverse (pull from successors).
-// Returns false on a cap hit or a failed consistency check (slab restored).
-template <typename D, int TEAM, bool PACKED>
-__device__ bool run_source_ds(const BatchArgs& a, const Slab<D>& sl, TeamShared<D, TEAM>& sh, uint32_t s, int t) {
-  const D INF = dinf<D>();
-  unsigned long long relax = 0, scanned = 0;
-  uint64_t rounds = 0, advances = 0;
-  unsigned long long cyc_expand = 0, cyc_refill = 0, cyc_settle = 0, cyc_back = 0, far_sc = 0;
-  long long c0 = clock64();
-  uint32_t* qa = sl.nearq;  // current frontier (stamp = sh.round)
-  uint32_t* qb = sl.farq;   // next frontier
-  if (t == 0) {
-    sl.d[s] = 0;
-    sl.S[0] = s;
-    sh.S_len = 1;
-    qa[0] = s;
-    sl.pc[s] = 1;
-    sh.round = 1;
-    sh.def_len = 0;
-    sh.bound = sat_add<D>((D)0, a.width);
-    sh.stop = 0;
-  }
-  team_sync<TEAM>();
-  uint32_t alen = 1;
-  int err = DEV_OK;
-  for (;;) {
-    c0 = clock64();
-    team_sync<TEAM>();  // every thread has read the last frontier length
-    if (t == 0) {
-      sh.front_out = qb;
-      sh.front_len = 0;
-      sh.round += 1;
-    }
-    team_sync<TEAM>();
-    expand_forward<D, TEAM, PACKED, WALK_DS>(a, out_rows(a.g), sl, sh, qa, 0, alen, s, t, INF, relax, scanned);
-    cyc_expand += clock64() - c0;
-    ++rounds;
-    alen = sh.front_len;
-    uint32_t* tmp = qa;
-    qa = qb;
-    qb = tmp;
-    if (alen == 0) {
-      c0 = clock64();
-      // next bucket: the deferred vertices within one width of the smallest
-      while (alen == 0 && sh.def_len > 0) {
-        const D old = sh.bound;
-        const uint32_t dl = sh.def_len;
-        far_sc += 2ull * dl;
-        D lo = INF, dummy = INF;
-        for (uint32_t base = 0; base < dl; base += TEAM) {
-          const uint32_t j = base + t;
-          if (j < dl) {
-            const D du = ldcg(&sl.d[ldcg(&sl.farq2[j])]);
-            if (du >= old) lo = dmin(lo, du);
-          }
-        }
-        team_min2<D, TEAM>(lo, dummy, sh.red);
-        const D nb = (lo == INF) ? old : sat_add<D>(lo, a.width);
-        if (t == 0) sh.front_len = 0;
-        team_sync<TEAM>();
-        uint32_t kept = 0;
-        for (uint32_t base = 0; base < dl; base += TEAM) {
-          const uint32_t j = base + t;
-          uint32_t u = 0, keep = 0;
-          if (j < dl) {
-            u = ldcg(&sl.farq2[j]);
-            const D du = ldcg(&sl.d[u]);
-            if (du >= old) {  // below old: already relaxed in an earlier bucket
-              if (du < nb) {
-                if (atomicExch(&sl.pc[u], sh.round) != sh.round) qa[atomicAdd(&sh.front_len, 1u)] = u;
-              } else {
-                keep = 1;
-              }
-            }
-          }
-          uint32_t ktot;
-          const uint32_t kx = team_excl_scan<TEAM>(keep, &ktot, sh.scan);
-          if (TEAM == 32) __syncwarp();
-          if (keep) sl.farq2[kept + kx] = u;
-          kept += ktot;
-        }
-        team_sync<TEAM>();
-        if (t == 0) {
-          sh.def_len = kept;
-          sh.bound = nb;
-        }
-        ++advances;
-        team_sync<TEAM>();
-        alen = sh.front_len;
-      }
-      cyc_refill += clock64() - c0;
-      if (alen == 0) break;
-    }
-    if (rounds + advances > a.phase_cap) {
-      err = DEV_ERR_TIMEOUT;
-      break;
-    }
-  }
-  uint32_t nlev = 0;
-  const uint32_t nr = sh.S_len;
-  if (err == DEV_OK) {
-    // distances are final: count predecessors (in-edges for directed graphs)
-    c0 = clock64();
-    const Rows prow = a.g.in_row_ptr ? in_rows(a.g) : out_rows(a.g);
-    expand_forward<D, TEAM, PACKED, WALK_COUNT>(a, prow, sl, sh, sl.S, 0, nr, s, t, INF, relax, scanned);
-    // sigma down the DAG, one hop-depth level at a time
-    if (t == 0) {
-      sl.ends[0] = s;
-      sh.lvl_len = 1;
-      sl.pend[0] = 0;
-      sl.pend[1] = 1;
-    }
-    team_sync<TEAM>();
-    nlev = 1;
-    uint32_t l0 = 0, l1 = 1;
-    for (;;) {
-      expand_forward<D, TEAM, PACKED, WALK_KAHN>(a, out_rows(a.g), sl, sh, sl.ends, l0, l1, s, t, INF, relax,
-                                                 scanned);
-      const uint32_t l2 = sh.lvl_len;
-      if (l2 == l1) break;
-      if (t == 0) sl.pend[nlev + 1] = l2;
-      ++nlev;
-      l0 = l1;
-      l1 = l2;
-    }
-    team_sync<TEAM>();
-    cyc_settle += clock64() - c0;
-    if (l1 != nr) err = DEV_ERR_INTERNAL;  // every reached vertex must be released exactly once
-  }
-  if (err != DEV_OK) {
-    if (t == 0) atomicCAS(a.err, DEV_OK, err);
-    for (uint32_t j = t; j < nr; j += TEAM) {
-      const uint32_t v = ldcg(&sl.S[j]);
-      sl.d[v] = INF;
-      sl.pc[v] = 0;
-    }
-  } else if (a.flags & RUN_FORWARD_ONLY) {
-    // test hook: present the levels in the S / ends layout of the strict schedule
-    for (uint32_t j = t; j < nr; j += TEAM) sl.S[j] = ldcg(&sl.ends[j]);
-    team_sync<TEAM>();
-    for (uint32_t l = t; l <= nlev; l += TEAM) sl.ends[l] = ldcg(&sl.pend[l]);
-    if (t == 0 && a.debug_out) {
-      a.debug_out[0] = nlev;
-      a.debug_out[1] = nr;
-    }
-  } else {
-    c0 = clock64();
-    const int last = a.ebc ? 0 : 1;
-    for (int lev = (int)nlev - 1; lev >= last; --lev) {
-      const uint32_t b0 = ldcg(&sl.pend[lev]);
-      const uint32_t b1 = ldcg(&sl.pend[lev + 1]);
-      accumulate_level<D, TEAM, PACKED>(a, sl, sh, sl.ends, b0, b1, s, t, scanned);
-    }
-    cyc_back += clock64() - c0;
-    for (uint32_t j = t; j < nr; j += TEAM) sl.d[ldcg(&sl.S[j])] = INF;
-  }
-  if (a.stats) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      relax += __shfl_xor_sync(FULL, relax, o);
-      scanned += __shfl_xor_sync(FULL, scanned, o);
-    }
-    if ((t & 31) == 0) {
-      atomicAdd(&a.stats[STAT_RELAX], relax);
-      atomicAdd(&a.stats[STAT_ENTRIES], scanned);
-    }
-    if (t == 0) {
-      atomicAdd(&a.stats[STAT_SOURCES], 1ull);
-      atomicAdd(&a.stats[STAT_PHASES], (unsigned long long)rounds);
-      atomicAdd(&a.stats[STAT_REFILLS], (unsigned long long)advances);
-      atomicAdd(&a.stats[STAT_REACHED], (unsigned long long)nr);
-      atomicAdd(&a.stats[STAT_LEVELS], (unsigned long long)nlev);
-      atomicAdd(&a.stats[STAT_CYC_EXPAND], cyc_expand);
-      atomicAdd(&a.stats[STAT_CYC_REFILL], cyc_refill);
-      atomicAdd(&a.stats[STAT_CYC_SETTLE], cyc_settle);
-      atomicAdd(&a.stats[STAT_CYC_BACKWARD], cyc_back);
-      atomicAdd(&a.stats[STAT_FAR_SCANNED], far_sc);
-    }
-  }
-  team_sync<TEAM>();
-  return err == DEV_OK;
-}
-
 // Resident CTAs per SM that a CTA team's register budget is compiled for:
 // 64 registers per thread (2048 threads per SM for 32-bit distances; 7/8 of
 // that for 64-bit ones, where 64 registers would spill).  Measured with
@@ -1439,9 +1040,7 @@ __host__ __device__ constexpr int min_blocks_of() {
   return TEAM == 32 ? 1 : (sizeof(D) == 4 ? 1024 / BLOCK : (BLOCK <= 256 ? 896 / BLOCK : 1024 / BLOCK));
 }
 
-// One instantiation per schedule, so the strict schedule's register allocation
-// does not pay for the delta-stepping code.
-template <typename D, int TEAM, int BLOCK, bool PACKED, int ALGO>
+template <typename D, int TEAM, int BLOCK, bool PACKED>
 __global__ void __launch_bounds__(BLOCK, (min_blocks_of<D, TEAM, BLOCK>())) bc_batched_kernel(const BatchArgs a) {
   static_assert(TEAM == 32 || TEAM == BLOCK, "a CTA holds either warp teams or one team");
   constexpr int NTEAMS = BLOCK / TEAM;
@@ -1464,70 +1063,64 @@ __global__ void __launch_bounds__(BLOCK, (min_blocks_of<D, TEAM, BLOCK>())) bc_b
       continue;
     }
     if (a.g.o2n) s = __ldg(&a.g.o2n[s]);
-    bool ok;
-    if constexpr (ALGO == ALGO_DELTA)
-      ok = run_source_ds<D, TEAM, PACKED>(a, sl, sh, s, t);
-    else
-      ok = run_source<D, TEAM, PACKED>(a, sl, sh, s, t);
+    const bool ok = run_source<D, TEAM, PACKED>(a, sl, sh, s, t);
     if (!ok || (a.flags & RUN_FORWARD_ONLY)) break;
   }
 }
 
-template <typename D, int TEAM, int BLOCK, bool PACKED, int ALGO>
+template <typename D, int TEAM, int BLOCK, bool PACKED>
 cudaError_t launch_t(const BatchArgs& a, int grid, cudaStream_t st) {
-  bc_batched_kernel<D, TEAM, BLOCK, PACKED, ALGO><<<grid, BLOCK, 0, st>>>(a);
+  bc_batched_kernel<D, TEAM, BLOCK, PACKED><<<grid, BLOCK, 0, st>>>(a);
   return cudaGetLastError();
 }
 
 // 1024-thread teams exist for 32-bit distances only (their shared state fits
 // the 48 KB of static shared memory; 64-bit distance words do not).
-template <typename D, bool PACKED, int ALGO>
+template <typename D, bool PACKED>
 cudaError_t launch_d(const BatchArgs& a, int team, int grid, cudaStream_t st) {
   switch (team) {
-    case 32: return launch_t<D, 32, 256, PACKED, ALGO>(a, grid, st);
-    case 128: return launch_t<D, 128, 128, PACKED, ALGO>(a, grid, st);
-    case 256: return launch_t<D, 256, 256, PACKED, ALGO>(a, grid, st);
-    case 512: return launch_t<D, 512, 512, PACKED, ALGO>(a, grid, st);
+    case 32: return launch_t<D, 32, 256, PACKED>(a, grid, st);
+    case 128: return launch_t<D, 128, 128, PACKED>(a, grid, st);
+    case 256: return launch_t<D, 256, 256, PACKED>(a, grid, st);
+    case 512: return launch_t<D, 512, 512, PACKED>(a, grid, st);
     case 1024:
-      if constexpr (sizeof(D) == 4) return launch_t<D, 1024, 1024, PACKED, ALGO>(a, grid, st);
+      if constexpr (sizeof(D) == 4) return launch_t<D, 1024, 1024, PACKED>(a, grid, st);
       return cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
   }
 }
 
-template <typename D, bool PACKED, int ALGO>
+template <typename D, bool PACKED>
 cudaError_t occ_d(int team, int* out) {
   switch (team) {
-    case 32: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bc_batched_kernel<D, 32, 256, PACKED, ALGO>, 256, 0);
-    case 128: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bc_batched_kernel<D, 128, 128, PACKED, ALGO>, 128, 0);
-    case 256: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bc_batched_kernel<D, 256, 256, PACKED, ALGO>, 256, 0);
-    case 512: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bc_batched_kernel<D, 512, 512, PACKED, ALGO>, 512, 0);
+    case 32: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bc_batched_kernel<D, 32, 256, PACKED>, 256, 0);
+    case 128: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bc_batched_kernel<D, 128, 128, PACKED>, 128, 0);
+    case 256: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bc_batched_kernel<D, 256, 256, PACKED>, 256, 0);
+    case 512: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bc_batched_kernel<D, 512, 512, PACKED>, 512, 0);
     case 1024:
       if constexpr (sizeof(D) == 4)
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bc_batched_kernel<D, 1024, 1024, PACKED, ALGO>, 1024, 0);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bc_batched_kernel<D, 1024, 1024, PACKED>, 1024, 0);
       return cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
   }
 }
 
 // Packed adjacency is only generated for graphs with 32-bit distances.
-template <int ALGO>
-cudaError_t launch_algo(const BatchArgs& a, int dist_bits, int team, int grid, cudaStream_t st) {
+inline cudaError_t launch_strict(const BatchArgs& a, int dist_bits, int team, int grid, cudaStream_t st) {
   if (grid <= 0) return cudaSuccess;
   if (dist_bits == 32)
-    return a.g.adjp ? launch_d<uint32_t, true, ALGO>(a, team, grid, st)
-                    : launch_d<uint32_t, false, ALGO>(a, team, grid, st);
+    return a.g.adjp ? launch_d<uint32_t, true>(a, team, grid, st)
+                    : launch_d<uint32_t, false>(a, team, grid, st);
   if (a.g.adjp) return cudaErrorInvalidValue;
-  return launch_d<uint64_t, false, ALGO>(a, team, grid, st);
+  return launch_d<uint64_t, false>(a, team, grid, st);
 }
 
 // Resident CTAs per SM; for 32-bit distances the smaller of the two adjacency forms.
-template <int ALGO>
-cudaError_t occupancy_algo(int dist_bits, int team, int* blocks_per_sm) {
-  if (dist_bits != 32) return occ_d<uint64_t, false, ALGO>(team, blocks_per_sm);
+inline cudaError_t occupancy_strict(int dist_bits, int team, int* blocks_per_sm) {
+  if (dist_bits != 32) return occ_d<uint64_t, false>(team, blocks_per_sm);
   int a = 0, b = 0;
-  cudaError_t e = occ_d<uint32_t, false, ALGO>(team, &a);
-  if (e == cudaSuccess) e = occ_d<uint32_t, true, ALGO>(team, &b);
+  cudaError_t e = occ_d<uint32_t, false>(team, &a);
+  if (e == cudaSuccess) e = occ_d<uint32_t, true>(team, &b);
   *blocks_per_sm = a < b ? a : b;
   return e;
 }

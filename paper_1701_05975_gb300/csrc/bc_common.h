@@ -37,35 +37,57 @@ struct GraphDev {
   const uint32_t* o2n;      // [n] old id -> new id (applied to sources)
   const uint32_t* n2o;      // [n] new id -> old id (applied to BC output)
   const uint32_t* e2o;      // [nnz] new CSR entry -> old CSR entry (edge BC output)
+  // Landmarks of the sweep schedule (kadj == nullptr: none).  h is the main
+  // landmark; land_out[l][v] = D(landmark l, v) and land_in[l][v] =
+  // D(v, landmark l) in 16- or 32-bit words (the same table for undirected
+  // graphs); kadj holds every row in ascending order of its second word.
+  const uint2* kadj;        // [nnz] {neighbour | weight << col_bits, w - D(h, neighbour)}; {neighbour, ...} with kw
+  const uint32_t* kw;       // [nnz] weights, where neighbour and weight do not fit one word
+  const uint32_t* k2o;      // [nnz] kadj entry -> caller's entry
+  const void* land_out;
+  const void* land_in;
+  uint64_t land_stride;     // words per table row (a multiple of 8)
+  uint32_t land_bits;       // 16 (0x7fff: unreachable) or 32 (0xffffffff: unreachable)
+  uint32_t nland;
+  uint32_t land_n;          // vertices from this id on are unreachable from and to h
+  uint32_t act_n;           // vertices from this id on have no entries (sweep schedule)
 };
 
+constexpr uint32_t SWEEP_MAX_LAND = 64;
+
 // Byte offsets of the per-source arrays inside one slab (one slab per source
-// in flight).  d: distances (all INF between sources), sig: sigma during the
-// forward pass and the coefficient c = (1 + delta) / sigma during the backward
-// pass, S: settle order (the level lists of Algorithm 1's S/ends), ends: level
-// boundaries, nearq / farq / farq2: candidate queues (reached, unsettled
-// vertices below the split, between the split and split2, above split2).
-// acc: per-vertex sum of successor coefficients during the backward pass
-// (zero between sources); pend: end of each level's range in the DAG edge
+// in flight).
+// Strict schedule.  d: distances (all INF between sources), sig: sigma during
+// the forward pass and the coefficient c = (1 + delta) / sigma during the
+// backward pass, S: settle order (the level lists of Algorithm 1's S/ends),
+// ends: level boundaries, nearq / farq / farq2: candidate queues (reached,
+// unsettled vertices below the split, between the split and split2, above
+// split2), acc: per-vertex sum of successor coefficients during the backward
+// pass (zero between sources); pend: end of each level's range in the DAG edge
 // list; pairs: the shortest-path DAG edges (u -> v) found while pulling sigma,
 // in level order of v (capacity pair_cap; on overflow the backward pass falls
-// back to scanning every CSR entry); pc: per-vertex round stamps, then
-// predecessor counts, of the delta-stepping schedule (zero between sources).
+// back to scanning every CSR entry).
+// Sweep schedule.  d: distances (INF between sources), sig: 16-byte vertex
+// records (zero between sources), near / far: frontiers, then the level lists
+// and their bounds, far2: deferred vertices, ends: rows left to whole warps,
+// S: reached vertices, acc: DAG list offsets, pend: three bits per vertex (two
+// of them zero between sources), pairs: compact DAG lists (capacity pair_cap words).
 struct SlabLayout {
   uint64_t stride;
-  uint64_t off_d, off_sig, off_S, off_ends, off_near, off_far, off_far2, off_acc, off_pend, off_pairs, off_pc;
+  uint64_t off_d, off_sig, off_S, off_ends, off_near, off_far, off_far2, off_acc, off_pend, off_pairs;
   uint64_t off_pair_e;  // entry walked by each DAG edge (edge output); 0 = not in this layout
   uint32_t pair_cap;
 };
 
 enum : uint32_t {
   RUN_FORWARD_ONLY = 1u,  // stop after distances / sigma / levels (test hook)
+  RUN_DIST_ONLY = 2u,     // sweep schedule: write distances to dist_out and stop there
 };
 
 // Per-source schedules of the batched kernel.
 enum : uint32_t {
   ALGO_STRICT = 1,  // strict settle batches (Sec. 3.2), sigma pulled per batch
-  ALGO_DELTA = 2,   // delta-stepping distances, then sigma and delta over DAG hop levels
+  ALGO_DELTA = 2,   // sweep schedule: distances first, then sigma and delta over DAG hop levels
 };
 
 enum : int {
@@ -106,7 +128,7 @@ struct BatchArgs {
   char* slabs;
   SlabLayout lay;
   uint32_t nslots;
-  uint64_t width;      // near/far split width
+  uint64_t width;      // near/far split width (sweep schedule: bucket width, all ones = one bucket)
   uint32_t settle_in;  // apply the strict IN criterion too
   uint32_t refine;     // bound each candidate's edges to unsettled vertices by dnode2 once dnode_arg is settled
   uint64_t phase_cap;  // cap on phases + refills per source
@@ -115,18 +137,55 @@ struct BatchArgs {
   uint32_t warp_deg;   // forward expansion: rows with >= warp_deg entries get a warp each
   uint32_t team_deg;   // ... and rows with >= team_deg entries the whole team
   uint32_t hot_n;      // ids below hot_n are gathered with an L2 evict-last hint
-  uint32_t algo;       // ALGO_*
   uint32_t flags;      // RUN_*
   uint32_t* debug_out; // RUN_FORWARD_ONLY: [0] = levels, [1] = reached
+  uint32_t* dist_out;  // RUN_DIST_ONLY: [k][n] distances
+  uint32_t sm_succ_cap;  // sweep schedule, shared-memory form: DAG list words
 };
 
-// Launchers (bc_batched.cu).  team: 32, 128, 256 or 512 threads per source.
+// Strict schedule (bc_batched.cu).  team: 32, 128, 256, 512 or (32-bit
+// distances) 1024 threads per source.
 cudaError_t launch_batched(const BatchArgs& a, int dist_bits, int team, int grid, cudaStream_t st);
 int batched_block_threads(int team);
-cudaError_t batched_occupancy(int dist_bits, int team, int* blocks_per_sm);  // strict schedule
-cudaError_t batched_occupancy(int dist_bits, int team, int algo, int* blocks_per_sm);
-cudaError_t launch_batched_delta(const BatchArgs& a, int dist_bits, int team, int grid, cudaStream_t st);
-cudaError_t batched_occupancy_delta(int dist_bits, int team, int* blocks_per_sm);
+cudaError_t batched_occupancy(int dist_bits, int team, int* blocks_per_sm);
+
+// Sweep schedule (bc_sweep*.cu): the kernel variant and its dynamic shared memory.
+struct SweepPlan {
+  int dist_bits = 32;
+  int team = 256;
+  bool prune = false;   // rows in landmark order (kadj)
+  int mem = 0;          // 0: slab, 1: slab with the vertex bits in shared memory, 2: all in shared memory
+  int group = 1;        // threads per row: 1 or 8
+  uint32_t smem_bytes = 0;
+  uint32_t succ_cap = 0;  // shared-memory form: DAG list words
+};
+cudaError_t launch_sweep(const BatchArgs& a, const SweepPlan& p, int grid, cudaStream_t st);
+cudaError_t sweep_occupancy(const SweepPlan& p, int* blocks_per_sm);
+uint32_t sweep_smem(int mem, int dist_bits, uint32_t n, uint32_t cap);  // dynamic shared memory of a team
+// One instantiation set each (a == nullptr: occupancy into *occ).
+cudaError_t sweep32_prune_global(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep32_prune_bits(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep32_prune_all(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep32_full1_global(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep32_full8_global(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep32_full1_bits(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep32_full8_bits(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep32_full1_all(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep64_full1_global(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep64_full8_global(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep64_full1_bits(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep64_full8_bits(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep64_full1_all(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+
+// Landmark preparation (bc_land.cu); g.adj holds the rows walked.
+cudaError_t land_symmetry(const GraphDev& g, unsigned long long* out, cudaStream_t st);
+cudaError_t land_judge(const GraphDev& g, const uint32_t* from_h, const uint32_t* probe, uint32_t h,
+                       uint32_t nprobe, unsigned long long* out, cudaStream_t st);
+cudaError_t land_max(uint64_t count, const uint32_t* tab, uint32_t* out, cudaStream_t st);
+cudaError_t land_pack(uint32_t n, uint64_t stride, uint32_t rows, const uint32_t* tab, int bits, void* out,
+                      cudaStream_t st);
+cudaError_t land_rows(const GraphDev& g, const uint32_t* from_h, unsigned long long* key, uint32_t col_bits,
+                      uint2* kadj, uint32_t* kw, uint32_t* k2o, cudaStream_t st);
 
 // Graph preparation and small helpers (bc_prep.cu).
 // dnode2 / dnode_arg may be nullptr (not computed).
