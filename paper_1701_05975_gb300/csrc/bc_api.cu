@@ -78,16 +78,26 @@ enum SlabKind : int { SLAB_STRICT = 0, SLAB_SWEEP = 1, SLAB_NONE = 2 };
 
 SlabLayout make_layout(uint32_t n, int dist_bits, SlabKind kind) {
   SlabLayout L{};
-  if (kind == SLAB_NONE) {  // every per-source array is in shared memory
-    L.stride = 256;
-    return L;
-  }
   uint64_t off = 0;
+  const uint64_t grain = kind == SLAB_NONE ? 16 : 256;
   auto take = [&](uint64_t bytes) {
     const uint64_t at = off;
-    off += align256(bytes);
+    off += (bytes + grain - 1) & ~(grain - 1);
     return at;
   };
+  if (kind == SLAB_NONE) {
+    // every per-source array in a CTA's shared memory, queue entries in 16 bits
+    L.off_sig = take((uint64_t)n * 16);
+    L.off_d = take((uint64_t)n * (dist_bits / 8));
+    L.off_acc = take((uint64_t)n * 4);
+    L.pair_cap = 3 * n + 64;
+    L.off_pairs = take(((uint64_t)L.pair_cap + 8) * 4);
+    L.off_pend = take((((uint64_t)n + 31) / 32) * 12);
+    for (uint64_t* q : {&L.off_near, &L.off_far, &L.off_far2, &L.off_ends, &L.off_S}) *q = take(((uint64_t)n + 2) * 2);
+    L.smem = (uint32_t)off;
+    L.stride = 256;  // nothing of it is in the slab
+    return L;
+  }
   const uint64_t w = (uint64_t)n * 4, w2 = ((uint64_t)n + 2) * 4;
   L.off_d = take((uint64_t)n * (dist_bits / 8));
   if (kind == SLAB_SWEEP) {
@@ -322,11 +332,14 @@ void plan_sweep(const bc_graph* g, RunCfg& r, bool allow_smem) {
     if (allow_smem && g->n <= SWEEP_SMEM_N) {
       p.mem = 2;
       p.group = 1;
-      p.succ_cap = 3 * g->n + 64;
-    } else if (sweep_smem(1, 32, g->act_n, 0) <= SWEEP_BITS_MAX * r.team / 1024) {
-      p.mem = 1;
+      p.smem_bytes = make_layout(g->n, g->dist_bits, SLAB_NONE).smem;
+    } else {
+      const uint32_t bits = ((g->act_n + 31) / 32) * 8;
+      if (bits <= SWEEP_BITS_MAX * r.team / 1024) {
+        p.mem = 1;
+        p.smem_bytes = bits;
+      }
     }
-    p.smem_bytes = sweep_smem(p.mem, g->dist_bits, p.mem == 2 ? g->n : g->act_n, p.succ_cap);
   }
   r.sweep = p;
 }
@@ -613,7 +626,6 @@ BatchArgs make_args(bc_graph* g, Workspace* w, const RunCfg& r, const uint32_t* 
   a.debug_out = w->ctl->debug;
   a.warp_deg = r.warp_deg;
   a.team_deg = r.team_deg;
-  a.sm_succ_cap = r.sweep.succ_cap;
   a.esm = (d_ebc && g->esm_state == 1) ? g->esm : nullptr;
   // the highest-degree vertices after relabeling: 128 KiB of 32-bit distance
   // words per source (the whole L2 holds this prefix for ~1000 sources)

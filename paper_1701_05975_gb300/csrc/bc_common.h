@@ -70,13 +70,14 @@ constexpr uint32_t SWEEP_MAX_LAND = 64;
 // Sweep schedule.  d: distances (INF between sources), sig: 16-byte vertex
 // records (zero between sources), near / far: frontiers, then the level lists
 // and their bounds, far2: deferred vertices, ends: rows left to whole warps,
-// S: reached vertices, acc: DAG list offsets, pend: three bits per vertex (two
-// of them zero between sources), pairs: compact DAG lists (capacity pair_cap words).
+// S: reached vertices, acc: DAG list offsets, pend: three bits per vertex (two of
+// them zero between sources), pairs: compact DAG lists (capacity pair_cap words).
 struct SlabLayout {
   uint64_t stride;
   uint64_t off_d, off_sig, off_S, off_ends, off_near, off_far, off_far2, off_acc, off_pend, off_pairs;
   uint64_t off_pair_e;  // entry walked by each DAG edge (edge output); 0 = not in this layout
   uint32_t pair_cap;
+  uint32_t smem;  // sweep schedule in shared memory: the offsets are into it, and this many bytes
 };
 
 enum : uint32_t {
@@ -140,7 +141,6 @@ struct BatchArgs {
   uint32_t flags;      // RUN_*
   uint32_t* debug_out; // RUN_FORWARD_ONLY: [0] = levels, [1] = reached
   uint32_t* dist_out;  // RUN_DIST_ONLY: [k][n] distances
-  uint32_t sm_succ_cap;  // sweep schedule, shared-memory form: DAG list words
 };
 
 // Strict schedule (bc_batched.cu).  team: 32, 128, 256, 512 or (32-bit
@@ -157,11 +157,9 @@ struct SweepPlan {
   int mem = 0;          // 0: slab, 1: slab with the vertex bits in shared memory, 2: all in shared memory
   int group = 1;        // threads per row: 1 or 8
   uint32_t smem_bytes = 0;
-  uint32_t succ_cap = 0;  // shared-memory form: DAG list words
 };
 cudaError_t launch_sweep(const BatchArgs& a, const SweepPlan& p, int grid, cudaStream_t st);
 cudaError_t sweep_occupancy(const SweepPlan& p, int* blocks_per_sm);
-uint32_t sweep_smem(int mem, int dist_bits, uint32_t n, uint32_t cap);  // dynamic shared memory of a team
 // One instantiation set each (a == nullptr: occupancy into *occ).
 cudaError_t sweep32_prune_global(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
 cudaError_t sweep32_prune_bits(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);

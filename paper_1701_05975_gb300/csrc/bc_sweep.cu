@@ -28,12 +28,4 @@ cudaError_t launch_sweep(const BatchArgs& a, const SweepPlan& p, int grid, cudaS
 
 cudaError_t sweep_occupancy(const SweepPlan& p, int* blocks_per_sm) { return dispatch(p, nullptr, 0, nullptr, blocks_per_sm); }
 
-uint32_t sweep_smem(int mem, int dist_bits, uint32_t n, uint32_t cap) {
-  const uint32_t bits = ((n + 31) / 32) * 8;
-  if (mem == 0) return 0;
-  if (mem == 1) return bits;
-  const uint32_t n8 = (n + 9) & ~7u;
-  return n8 * (16 + (uint32_t)dist_bits / 8 + 4 + 5 * 2) + cap * 4 + bits + bits / 2;
-}
-
 }  // namespace bcgpu

@@ -47,10 +47,12 @@ namespace {
 
 constexpr int SW_UNR = 4;              // entries in flight per thread
 constexpr int SW_STEPS = 4;            // eight threads per row: SW_UNR * SW_STEPS * 8 entries, then whole warps
-constexpr uint32_t SW_FIRST = 4;       // one thread per row: its own entries, then eight threads take SW_SECOND more,
-constexpr uint32_t SW_SECOND = 16;     // ... then whole warps
+constexpr uint32_t SW_SECOND = 16;     // one thread per row: FIRST entries, eight threads SW_SECOND more, then whole warps
 constexpr int32_t SW_NO_BOUND = 0x7fffffff;  // no entry's test word exceeds it
-constexpr uint32_t SW_LIST = 8;        // DAG lists up to this length are one thread's work
+constexpr uint32_t SW_LIST = 4;        // DAG lists: one thread's work up to this length,
+constexpr uint32_t SW_LIST8 = 64;      // ... eight threads' up to this many more, then a warp's
+constexpr uint32_t SW_SCAN = 8;        // the pass over the lists before sigma: one thread up to this length
+constexpr int SW_FOLDS = 3;            // ... and its repetitions
 constexpr uint32_t SW_WARP_MAX = 2048; // longer rows and lists are the whole team's work
 constexpr uint32_t SW_TEAM_CAP = 64;   // rows handed to the whole team per pass (the rest stay with a warp)
 constexpr uint32_t SW_HEAD = 2;        // words before a DAG list: successors listed, successors counted
@@ -79,7 +81,7 @@ struct SweepShared {
   uint32_t nwide[3];  // rows left to whole warps
   uint32_t nteam[3];  // rows left to the whole team
   uint32_t tpos;
-  uint32_t S_len, def_len, ndef, dag_len, dag_over;
+  uint32_t S_len, def_len, ndef, dag_len, dag_over, nkeep, nfold;
   unsigned long long cyc[4];
   long long tmark;
   uint32_t team_v[SW_TEAM_CAP], team_e[SW_TEAM_CAP];
@@ -95,6 +97,9 @@ struct SweepTeam {
   static constexpr bool SM = MEM == MEM_ALL;
   using Idx = typename std::conditional<SM, uint16_t, uint32_t>::type;
   static constexpr int NW = TEAM / 32;
+  // entries that one thread walks before its warp helps: small graphs run at
+  // latency, so more of them at once
+  static constexpr uint32_t FIRST = SM ? 8 : 4;
 
   const BatchArgs& a;
   Sh& sh;
@@ -139,7 +144,6 @@ struct SweepTeam {
     if constexpr (MEM == MEM_GLOBAL) return ldcg(p);
     else return *reinterpret_cast<const volatile uint32_t*>(p);
   }
-  static __device__ __forceinline__ uint32_t ld_slab_bits(const uint32_t* p) { return ld(p); }
   static __device__ __forceinline__ bool test_bit(const uint32_t* b, uint32_t v) {
     return (ld_bits(&b[v >> 5]) >> (v & 31)) & 1u;
   }
@@ -320,6 +324,9 @@ struct SweepTeam {
     if constexpr (sizeof(D) == 8) return (D)__shfl_sync(FULL, (unsigned long long)x, src);
     else return __shfl_sync(FULL, x, src);
   }
+  // Rows that one warp takes at a time: all 32 lanes' worth, or an even share
+  // of a short list, so that no warp idles while another walks long rows.
+  static __device__ __forceinline__ uint32_t rows_per_warp(uint32_t len) { return min(32u, (len + NW - 1) / NW); }
   // Lane of the (lane / 8)-th row in m, or -1.
   static __device__ __forceinline__ int tier_row(uint32_t m) {
     for (uint32_t k = (threadIdx.x & 31) >> 3; k > 0; --k) m &= m - 1;
@@ -327,30 +334,31 @@ struct SweepTeam {
   }
 
   // Visit every walkable entry of the rows get(0) .. get(len - 1): G = 1: one
-  // thread per row for SW_FIRST entries, then eight lanes of its warp for
+  // thread per row for FIRST entries, then eight lanes of its warp for
   // SW_SECOND more; G = 8: eight threads per row.  The rest of longer rows goes
   // to whole warps, and to the whole team above SW_WARP_MAX.  Ends with the
   // team synchronised.
   template <typename Get, typename Visit>
   __device__ __forceinline__ void walk(uint32_t len, Get&& get, Visit&& visit) {
-    constexpr uint32_t P0 = G == 1 ? SW_FIRST + SW_SECOND : SW_UNR * SW_STEPS * G;
+    constexpr uint32_t P0 = G == 1 ? FIRST + SW_SECOND : SW_UNR * SW_STEPS * G;
     const uint32_t lane = threadIdx.x & 31;
     if constexpr (G == 1) {
-      for (uint32_t base = (uint32_t)t - lane; base < len; base += TEAM) {
-        const uint32_t v = base + lane < len ? get(base + lane) : NONE;
+      const uint32_t rpw = rows_per_warp(len);
+      for (uint32_t base = ((uint32_t)t >> 5) * rpw; base < len; base += NW * rpw) {
+        const uint32_t v = lane < rpw && base + lane < len ? get(base + lane) : NONE;
         Row r{};
         if (v != NONE) r = row_of(v);
         bool more;
         {
-          uint2 x[SW_FIRST];
-          bool ok[SW_FIRST];
+          uint2 x[FIRST];
+          bool ok[FIRST];
 #pragma unroll
-          for (uint32_t q = 0; q < SW_FIRST; ++q) ok[q] = entry(r, q, r.deg, x[q]);
-          D du[SW_FIRST];
+          for (uint32_t q = 0; q < FIRST; ++q) ok[q] = entry(r, q, r.deg, x[q]);
+          D du[FIRST];
 #pragma unroll
-          for (uint32_t q = 0; q < SW_FIRST; ++q) du[q] = ok[q] ? ld(&d[x[q].x]) : 0;
+          for (uint32_t q = 0; q < FIRST; ++q) du[q] = ok[q] ? ld(&d[x[q].x]) : 0;
           visit(v, r, ok, x, du, 0u, 1u);
-          more = r.deg > SW_FIRST && (!PRUNE || ok[SW_FIRST - 1]);
+          more = r.deg > FIRST && (!PRUNE || ok[FIRST - 1]);
         }
         uint32_t m = __ballot_sync(FULL, more);
         while (m) {
@@ -361,7 +369,7 @@ struct SweepTeam {
           m &= m - 1;
           m &= m - 1;
           m &= m - 1;
-          const uint32_t e = SW_FIRST + (lane & 7);
+          const uint32_t e = FIRST + (lane & 7);
           uint2 x[2];
           bool ok[2];
 #pragma unroll
@@ -645,20 +653,20 @@ struct SweepTeam {
       uint32_t mask = 0;
       bool more;
       if constexpr (G == 1) {
-        uint2 x[SW_FIRST];
-        bool ok[SW_FIRST];
+        uint2 x[FIRST];
+        bool ok[FIRST];
 #pragma unroll
-        for (uint32_t q = 0; q < SW_FIRST; ++q) ok[q] = entry(r, q, r.deg, x[q]);
-        D du[SW_FIRST];
+        for (uint32_t q = 0; q < FIRST; ++q) ok[q] = entry(r, q, r.deg, x[q]);
+        D du[FIRST];
 #pragma unroll
-        for (uint32_t q = 0; q < SW_FIRST; ++q) du[q] = ok[q] ? ld(&d[x[q].x]) : INF;
+        for (uint32_t q = 0; q < FIRST; ++q) du[q] = ok[q] ? ld(&d[x[q].x]) : INF;
 #pragma unroll
-        for (uint32_t q = 0; q < SW_FIRST; ++q)
+        for (uint32_t q = 0; q < FIRST; ++q)
           if (ok[q]) {
             ++nscan;
             if (du[q] == r.dv + (D)x[q].y) mask |= 1u << q;
           }
-        more = r.deg > SW_FIRST && (!PRUNE || ok[SW_FIRST - 1]);
+        more = r.deg > FIRST && (!PRUNE || ok[FIRST - 1]);
         uint32_t m = __ballot_sync(FULL, more);
         while (m) {
           const int src = tier_row(m);
@@ -666,16 +674,16 @@ struct SweepTeam {
           uint2 z[2];
           bool in[2], fit[2];
 #pragma unroll
-          for (int k = 0; k < 2; ++k) in[k] = entry(y, SW_FIRST + (lane & 7) + 8 * k, src < 0 ? 0u : y.deg, z[k]);
+          for (int k = 0; k < 2; ++k) in[k] = entry(y, FIRST + (lane & 7) + 8 * k, src < 0 ? 0u : y.deg, z[k]);
 #pragma unroll
           for (int k = 0; k < 2; ++k) fit[k] = in[k] && ld(&d[z[k].x]) == y.dv + (D)z[k].y;
           nscan += in[0] + in[1];
           const uint32_t f0 = __ballot_sync(FULL, fit[0]), f1 = __ballot_sync(FULL, fit[1]);
-          const uint32_t on = __ballot_sync(FULL, (lane & 7) == 7 && in[1] && y.deg > SW_FIRST + SW_SECOND);
+          const uint32_t on = __ballot_sync(FULL, (lane & 7) == 7 && in[1] && y.deg > FIRST + SW_SECOND);
           // the rows' own lanes collect their bits
           const uint32_t k = __popc(m & ((1u << lane) - 1u));
           if (((m >> lane) & 1u) && k < 4) {
-            mask |= (((f0 >> (8 * k)) & 0xffu) << SW_FIRST) | (((f1 >> (8 * k)) & 0xffu) << (SW_FIRST + 8));
+            mask |= (((f0 >> (8 * k)) & 0xffu) << FIRST) | (((f1 >> (8 * k)) & 0xffu) << (FIRST + 8));
             more = (on >> (8 * k + 7)) & 1u;
           }
           m &= m - 1;
@@ -730,11 +738,11 @@ struct SweepTeam {
         succ[pos] = total;
         succ[pos + 1] = 0;
       }
-      pos += head;
       if (G == 1 && stream) {
         const uint32_t has = __ballot_sync(FULL, head != 0);
         if (lane == 0 && i < len) bits2[i >> 5] = has;
       }
+      pos += head;
       while (__any_sync(FULL, mask != 0)) {
         uint32_t e[SW_UNR], u[SW_UNR];
 #pragma unroll
@@ -850,96 +858,155 @@ struct SweepTeam {
   }
 
   // Replace the listed successors that have no successor themselves and one
-  // predecessor by a count.  bits0 becomes "has successors" on the way and is
-  // zero at the end.
-  __device__ __forceinline__ void drop_leaves() {
-    const uint32_t lane = threadIdx.x & 31;
-    uint32_t len = reached_count();
-    const uint32_t all = len;
-    // the vertices with successors, as bits and as a list
-    const Idx* list = S;
+  // predecessor by a count; then fold, a few times over: a vertex with one
+  // predecessor whose successors are all counted has its dependency (the
+  // count), so it goes into BC and its predecessor counts it too.  bits0
+  // becomes "has successors and is not folded" on the way and is zero at the
+  // end.
+  __device__ __forceinline__ void drop_leaves(int folds) {
+    const uint32_t lane = threadIdx.x & 31, all = reached_count();
+    // the vertices with successors: as bits, and as a list in vertex order
+    uint32_t len = all;
     if (stream) {
       if (G == 1) {
-        for (uint32_t w = t; w < (len + 31) / 32; w += TEAM) bits0[w] = ld_slab_bits(&bits2[w]);
+        for (uint32_t w = t; w < (all + 31) / 32; w += TEAM) bits0[w] = ld(&bits2[w]);
       } else {
-        for (uint32_t base = (uint32_t)t & ~31u; base < len; base += TEAM) {
+        for (uint32_t base = (uint32_t)t & ~31u; base < all; base += TEAM) {
           const uint32_t v = base + lane;
-          const bool has = v < len && (test_bit(bits0, v) || v == s) && ld(&off[v]) != 0;
+          const bool has = v < all && (test_bit(bits0, v) || v == s) && ld(&off[v]) != 0;
           const uint32_t m = __ballot_sync(FULL, has);
           if (lane == 0) bits0[base >> 5] = m;
         }
       }
       team_sync<TEAM>();
-      if constexpr (TEAM > 32) {
-        len = ordered<false>(bits0, S);
-      } else {
-        list = nullptr;
-      }
+      len = ordered<false>(bits0, S);
     } else {
-      for (uint32_t i = t; i < len; i += TEAM) {
+      for (uint32_t i = t; i < all; i += TEAM) {
         const uint32_t v = ld(&S[i]);
         if (ld(&off[v]) == 0) clear_bit(bits0, v);
       }
       team_sync<TEAM>();
     }
-    for (uint32_t i = t; i < len; i += TEAM) {
-      const uint32_t v = list ? (uint32_t)ld(&list[i]) : i;
-      if (!test_bit(bits0, v) && v != s) continue;
-      const uint32_t o = ld(&off[v]);
-      if (o == 0) continue;
-      const uint32_t n = ld(&succ[o]);
-      if (n > SW_LIST) {
-        wide[push_pos(&sh.nwide[sel])] = (Idx)v;
-        continue;
-      }
-      uint32_t kept = 0;
-      for (uint32_t j0 = 0; j0 < n; j0 += SW_UNR) {
-        uint32_t u[SW_UNR];
+    const Idx* list = S;
+    Idx *keep = qa, *spare = qb;
+    for (int pass = 0;; ++pass) {
+      if (t == 0) sh.nkeep = sh.nfold = 0;
+      team_sync<TEAM>();
+      const bool last = pass >= folds;
+      for (uint32_t base = (uint32_t)t - lane; base < len; base += TEAM) {
+        const uint32_t i = base + lane;
+        uint32_t v = 0, o = 0, n = 0;
+        if (i < len) {
+          v = ld(&list[i]);
+          o = ld(&off[v]);
+          if (o) n = ld(&succ[o]);
+        }
+        if (n > SW_SCAN) {
+          wide[push_pos(&sh.nwide[sel])] = (Idx)v;
+          n = 0;
+        }
+        uint32_t kept = 0, gone = 0;
+        for (uint32_t j0 = 0; j0 < n; j0 += SW_UNR) {
+          uint32_t x[SW_UNR];
 #pragma unroll
-        for (int q = 0; q < SW_UNR; ++q) u[q] = j0 + q < n ? ld(&succ[o + SW_HEAD + j0 + q]) : NONE;
+          for (int q = 0; q < SW_UNR; ++q) x[q] = j0 + q < n ? ld(&succ[o + SW_HEAD + j0 + q]) : NONE;
 #pragma unroll
-        for (int q = 0; q < SW_UNR; ++q)
-          if (u[q] != NONE && (test_bit(bits1, u[q]) || test_bit(bits0, u[q]))) {
-            if (kept != j0 + q) succ[o + SW_HEAD + kept] = u[q];
-            ++kept;
-          }
-      }
-      if (kept != n) {
-        succ[o] = kept;
-        succ[o + 1] = n - kept;
-      }
-    }
-    team_sync<TEAM>();
-    const uint32_t nw = sh.nwide[sel];
-    for (uint32_t i = (uint32_t)t >> 5; i < nw; i += NW) {
-      const uint32_t o = ld(&off[ld(&wide[i])]);
-      const uint32_t n = ld(&succ[o]);
-      uint32_t kept = 0;
-      for (uint32_t j0 = 0; j0 < n; j0 += 128) {
-        uint32_t u[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) u[q] = j0 + q * 32 + lane < n ? ld(&succ[o + SW_HEAD + j0 + q * 32 + lane]) : NONE;
-        __syncwarp();
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const bool keep = u[q] != NONE && (test_bit(bits1, u[q]) || test_bit(bits0, u[q]));
-          const uint32_t m = __ballot_sync(FULL, keep);
-          if (keep) succ[o + SW_HEAD + kept + __popc(m & ((1u << lane) - 1u))] = u[q];
-          kept += __popc(m);
+          for (int q = 0; q < SW_UNR; ++q)
+            if (x[q] != NONE) {
+              if (listed(x[q])) {
+                if (kept != j0 + q) succ[o + SW_HEAD + kept] = x[q];
+                ++kept;
+              } else {
+                gone += counted(x[q], pass);
+              }
+            }
+        }
+        if (kept != n) {
+          succ[o] = kept;
+          succ[o + 1] = pass == 0 ? gone : gone + ld(&succ[o + 1]);
         }
         __syncwarp();
+        if (!last) {
+          const bool fold[1] = {n > 0 && kept == 0 && v != s && !test_bit(bits1, v)};
+          const bool stay[1] = {kept > 0};
+          const uint32_t val[1] = {v};
+          push_many(&sh.nfold, def, fold, val);
+          push_many(&sh.nkeep, keep, stay, val);
+        }
       }
-      if (lane == 0) {
-        succ[o] = kept;
-        succ[o + 1] = n - kept;
+      team_sync<TEAM>();
+      const uint32_t nw = sh.nwide[sel];
+      for (uint32_t i = (uint32_t)t >> 5; i < nw; i += NW) {
+        const uint32_t v = ld(&wide[i]);
+        const uint32_t o = ld(&off[v]);
+        const uint32_t n = ld(&succ[o]);
+        uint32_t kept = 0, gone = 0;
+        for (uint32_t j0 = 0; j0 < n; j0 += 128) {
+          uint32_t x[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) x[q] = j0 + q * 32 + lane < n ? ld(&succ[o + SW_HEAD + j0 + q * 32 + lane]) : NONE;
+          __syncwarp();
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const bool stays = x[q] != NONE && listed(x[q]);
+            if (x[q] != NONE && !stays) gone += counted(x[q], pass);
+            const uint32_t m = __ballot_sync(FULL, stays);
+            if (stays) succ[o + SW_HEAD + kept + __popc(m & ((1u << lane) - 1u))] = x[q];
+            kept += __popc(m);
+          }
+          __syncwarp();
+        }
+#pragma unroll
+        for (int k = 16; k > 0; k >>= 1) gone += __shfl_xor_sync(FULL, gone, k);
+        if (lane == 0) {
+          succ[o] = kept;
+          succ[o + 1] += gone;
+          if (!last) {
+            if (kept) keep[atomicAdd(&sh.nkeep, 1u)] = (Idx)v;
+            else if (v != s && !test_bit(bits1, v)) def[atomicAdd(&sh.nfold, 1u)] = (Idx)v;
+          }
+        }
       }
+      if (nw) team_sync<TEAM>();
+      rotate();
+      const uint32_t nf = sh.nfold;
+      // one more pass only where it removes a fair share of what is left
+      if (last || nf < len / 12) break;
+      for (uint32_t i = t; i < nf; i += TEAM) {
+        const uint32_t v = ld(&def[i]);
+        clear_bit(bits0, v);
+        add_bc(v, (double)ld(&succ[ld(&off[v]) + 1]));
+      }
+      len = sh.nkeep;
+      list = keep;
+      Idx* tmp = keep;
+      keep = spare;
+      spare = tmp;
+      team_sync<TEAM>();
     }
-    if (nw) team_sync<TEAM>();
-    clear_bits0(all);
-    rotate();
+    team_sync<TEAM>();
+    clear_bits0();
+  }
+  __device__ __forceinline__ uint32_t succ_vertex(uint32_t x) const { return a.ebc ? entry_col(x) : x; }
+  __device__ __forceinline__ void add_bc(uint32_t v, double delta) {
+    atomicAdd(&a.bc[a.g.n2o ? __ldg(&a.g.n2o[v]) : v], delta);
+  }
+  // Whether list word x stays listed: its vertex has several predecessors, or
+  // successors of its own that are not folded.
+  __device__ __forceinline__ bool listed(uint32_t x) const {
+    const uint32_t u = succ_vertex(x);
+    return test_bit(bits1, u) || test_bit(bits0, u);
+  }
+  // What a word leaving its list adds to the dependency: its vertex, and on
+  // later passes (where it is a folded one) what was counted below it.
+  __device__ __forceinline__ uint32_t counted(uint32_t x, int pass) {
+    const uint32_t c = pass == 0 ? 1u : 1u + ld(&succ[ld(&off[succ_vertex(x)]) + 1]);
+    if (a.ebc) atomicAdd(&a.ebc[entry_out(x)], (double)c);
+    return c;
   }
   // bits0 back to zero (it holds reached vertices only).  Ends synchronised.
-  __device__ __forceinline__ void clear_bits0(uint32_t len) {
+  __device__ __forceinline__ void clear_bits0() {
+    const uint32_t len = reached_count();
     if (stream) {
       for (uint32_t w = t; w < (len + 31) / 32; w += TEAM) bits0[w] = 0;
     } else {
@@ -962,7 +1029,6 @@ struct SweepTeam {
     node[u].aux = 0ull;
     return true;
   }
-  __device__ __forceinline__ uint32_t succ_vertex(uint32_t x) const { return a.ebc ? entry_col(x) : x; }
 
   // Levels of the DAG from the source; order holds them back to back, lvl
   // their bounds.  A vertex without successors needs no level of its own
@@ -1015,31 +1081,52 @@ struct SweepTeam {
                push(on, u, any ? ld(&node[v].sig) : 0.0);
              });
       } else {
-        for (uint32_t b = l0 + ((uint32_t)t & ~31u); b < l1; b += TEAM) {
-          const uint32_t i = b + ((uint32_t)t & 31u);
-          uint32_t o = 0, len = 0;
+        const uint32_t lane = threadIdx.x & 31, rpw = rows_per_warp(l1 - l0);
+        for (uint32_t b = l0 + ((uint32_t)t >> 5) * rpw; b < l1; b += NW * rpw) {
+          uint32_t v = 0, o = 0, len = 0;
           double sv = 0.0;
-          uint32_t v = 0;
-          if (i < l1) {
-            v = ld(&order[i]);
+          if (lane < rpw && b + lane < l1) {
+            v = ld(&order[b + lane]);
             o = ld(&off[v]);
             sv = ld(&node[v].sig);
             if (o) len = ld(&succ[o]);
           }
-          if (len > SW_LIST) {
+          if (len > SW_LIST + SW_LIST8) {
             wide[push_pos(&sh.nwide[sel])] = (Idx)v;
             len = 0;
           }
           __syncwarp();
-          for (uint32_t j = 0; __any_sync(FULL, j < len); j += SW_UNR) {
-            bool on[SW_UNR];
-            uint32_t u[SW_UNR];
+          if (__any_sync(FULL, len > 0)) {
+            bool on[SW_LIST];
+            uint32_t u[SW_LIST];
 #pragma unroll
-            for (int q = 0; q < SW_UNR; ++q) {
-              on[q] = j + q < len;
-              u[q] = on[q] ? succ_vertex(ld(&succ[o + SW_HEAD + j + q])) : 0u;
+            for (uint32_t q = 0; q < SW_LIST; ++q) {
+              on[q] = q < len;
+              u[q] = on[q] ? succ_vertex(ld(&succ[o + SW_HEAD + q])) : 0u;
             }
             push(on, u, sv);
+          }
+          uint32_t m = __ballot_sync(FULL, len > SW_LIST);
+          while (m) {
+            const int src = tier_row(m);
+            const uint32_t qo = __shfl_sync(FULL, o, src < 0 ? 0 : src);
+            uint32_t ql = __shfl_sync(FULL, len, src < 0 ? 0 : src);
+            const double qs = __shfl_sync(FULL, sv, src < 0 ? 0 : src);
+            if (src < 0) ql = 0;
+            for (uint32_t k = SW_LIST + (lane & 7); __any_sync(FULL, k < ql); k += 16) {
+              bool on[2];
+              uint32_t u[2];
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                on[q] = k + 8 * q < ql;
+                u[q] = on[q] ? succ_vertex(ld(&succ[qo + SW_HEAD + k + 8 * q])) : 0u;
+              }
+              push(on, u, qs);
+            }
+            m &= m - 1;
+            m &= m - 1;
+            m &= m - 1;
+            m &= m - 1;
           }
         }
         team_sync<TEAM>();
@@ -1120,7 +1207,7 @@ struct SweepTeam {
   }
   __device__ __forceinline__ void finish(uint32_t v, double delta) {
     node[v].aux = (unsigned long long)__double_as_longlong(delta);
-    if (v != s) atomicAdd(&a.bc[a.g.n2o ? __ldg(&a.g.n2o[v]) : v], delta);
+    if (v != s) add_bc(v, delta);
   }
   __device__ __forceinline__ double pull(uint32_t x, const SweepNode& u, double sig) {
     const double c = coeff(u);
@@ -1153,26 +1240,62 @@ struct SweepTeam {
         }
         team_sync<TEAM>();
       } else {
-        for (uint32_t i = b0 + t; i < b1; i += TEAM) {
-          const uint32_t v = ld(&order[i]);
-          const uint32_t o = ld(&off[v]);
-          const double sig = ld(&node[v].sig);
-          if (o == 0) continue;
-          const uint32_t len = ld(&succ[o]);
-          const uint32_t leaves = ld(&succ[o + 1]);
-          if (len > SW_LIST) {
+        const uint32_t lane = threadIdx.x & 31, rpw = rows_per_warp(b1 - b0);
+        for (uint32_t b = b0 + ((uint32_t)t >> 5) * rpw; b < b1; b += NW * rpw) {
+          uint32_t v = 0, o = 0, len = 0, below = 0;
+          double sig = 0.0, acc = 0.0;
+          if (lane < rpw && b + lane < b1) {
+            v = ld(&order[b + lane]);
+            o = ld(&off[v]);
+            sig = ld(&node[v].sig);
+            if (o) {
+              len = ld(&succ[o]);
+              below = ld(&succ[o + 1]);
+            }
+          }
+          if (len > SW_LIST + SW_LIST8) {
             wide[push_pos(&sh.nwide[sel])] = (Idx)v;
-            continue;
+            len = o = 0;
           }
-          double acc = 0.0;
-          for (uint32_t j = 0; j < len; j += 2) {
-            const uint32_t x0 = ld(&succ[o + SW_HEAD + j]), x1 = j + 1 < len ? ld(&succ[o + SW_HEAD + j + 1]) : NONE;
-            SweepNode n0 = ld_node(&node[succ_vertex(x0)]), n1{1.0, 0ull};
-            if (x1 != NONE) n1 = ld_node(&node[succ_vertex(x1)]);
-            acc += pull(x0, n0, sig);
-            if (x1 != NONE) acc += pull(x1, n1, sig);
+          __syncwarp();
+          {
+            uint32_t x[SW_LIST];
+#pragma unroll
+            for (uint32_t q = 0; q < SW_LIST; ++q) x[q] = q < len ? ld(&succ[o + SW_HEAD + q]) : NONE;
+#pragma unroll
+            for (uint32_t h = 0; h < SW_LIST; h += 2) {
+              SweepNode u0{1.0, 0ull}, u1{1.0, 0ull};
+              if (h < len) u0 = ld_node(&node[succ_vertex(x[h])]);
+              if (h + 1 < len) u1 = ld_node(&node[succ_vertex(x[h + 1])]);
+              if (h < len) acc += pull(x[h], u0, sig);
+              if (h + 1 < len) acc += pull(x[h + 1], u1, sig);
+            }
           }
-          finish(v, sig * acc + (double)leaves);
+          uint32_t m = __ballot_sync(FULL, len > SW_LIST);
+          while (m) {
+            const int src = tier_row(m);
+            const uint32_t qo = __shfl_sync(FULL, o, src < 0 ? 0 : src);
+            uint32_t ql = __shfl_sync(FULL, len, src < 0 ? 0 : src);
+            const double qs = __shfl_sync(FULL, sig, src < 0 ? 0 : src);
+            if (src < 0) ql = 0;
+            double part = 0.0;
+            for (uint32_t k = SW_LIST + (lane & 7); k < ql; k += 8) {
+              const uint32_t x = ld(&succ[qo + SW_HEAD + k]);
+              part += pull(x, ld_node(&node[succ_vertex(x)]), qs);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int k = 4; k > 0; k >>= 1) part += __shfl_xor_sync(FULL, part, k);
+            // the lists' own lanes collect their sums
+            const uint32_t k = __popc(m & ((1u << lane) - 1u));
+            part = __shfl_sync(FULL, part, (k & 3) * 8);
+            if (((m >> lane) & 1u) && k < 4) acc += part;
+            m &= m - 1;
+            m &= m - 1;
+            m &= m - 1;
+            m &= m - 1;
+          }
+          if (o) finish(v, sig * acc + (double)below);
         }
         team_sync<TEAM>();
         wide_lists([&](uint32_t v, uint32_t o, uint32_t len, uint32_t l, uint32_t lanes) {
@@ -1327,12 +1450,12 @@ struct SweepTeam {
       team_sync<TEAM>();
       over = sh.dag_over != 0;
       const bool all = over || (a.flags & RUN_FORWARD_ONLY);
-      const bool drop = !all && !a.ebc;
-      every = !drop;
+      const bool drop = !all;
+      every = all;
       if (drop) {
-        drop_leaves();
+        drop_leaves(rounds < SW_DEEP ? SW_FOLDS : 0);
       } else {
-        clear_bits0(reached_count());
+        clear_bits0();
       }
       lap(0);
       nlev = sigma_levels(qa, qb, over, all, drop, rounds < SW_DEEP);
@@ -1428,51 +1551,24 @@ __global__ void __launch_bounds__(BLOCK, (sweep_min_blocks<D, TEAM, BLOCK>())) b
   if (t < 3) sh.qlen[t] = sh.nwide[t] = sh.nteam[t] = 0;
   bool dirty = false;
   const uint32_t words = (a.g.act_n + 31) / 32;
+  char* base = SM ? reinterpret_cast<char*>(sweep_arrays) : a.slabs + (uint64_t)slot * a.lay.stride;
+  w.d = reinterpret_cast<D*>(base + a.lay.off_d);
+  w.node = reinterpret_cast<SweepNode*>(base + a.lay.off_sig);
+  w.qa = reinterpret_cast<Idx*>(base + a.lay.off_near);
+  w.qb = reinterpret_cast<Idx*>(base + a.lay.off_far);
+  w.def = reinterpret_cast<Idx*>(base + a.lay.off_far2);
+  w.wide = reinterpret_cast<Idx*>(base + a.lay.off_ends);
+  w.S = reinterpret_cast<Idx*>(base + a.lay.off_S);
+  w.off = reinterpret_cast<uint32_t*>(base + a.lay.off_acc);
+  w.succ = reinterpret_cast<uint32_t*>(base + a.lay.off_pairs);
+  w.succ_cap = a.lay.pair_cap;
+  w.bits0 = reinterpret_cast<uint32_t*>(MEM == MEM_BITS ? reinterpret_cast<char*>(sweep_arrays) : base + a.lay.off_pend);
+  w.bits1 = w.bits0 + words;
+  w.bits2 = reinterpret_cast<uint32_t*>(base + a.lay.off_pend) + 2 * words;
   if constexpr (SM) {
-    const uint32_t n8 = (a.g.n + 9) & ~7u;
-    unsigned char* p = sweep_arrays;
-    w.node = reinterpret_cast<SweepNode*>(p);
-    p += n8 * 16;
-    w.d = reinterpret_cast<D*>(p);
-    p += n8 * sizeof(D);
-    w.off = reinterpret_cast<uint32_t*>(p);
-    p += n8 * 4;
-    w.succ = reinterpret_cast<uint32_t*>(p);
-    p += a.sm_succ_cap * 4;
-    w.bits0 = reinterpret_cast<uint32_t*>(p);
-    w.bits1 = w.bits0 + words;
-    w.bits2 = w.bits1 + words;
-    p += words * 12;
-    Idx* q = reinterpret_cast<Idx*>(p);
-    w.qa = q;
-    w.qb = q + n8;
-    w.S = q + 2 * n8;
-    w.def = q + 3 * n8;
-    w.wide = q + 4 * n8;
-    w.succ_cap = a.sm_succ_cap;
     const SweepNode zero{0.0, 0ull};
     for (uint32_t v = t; v < a.g.n; v += TEAM) w.node[v] = zero;
     w.fill_distances();
-  } else {
-    char* base = a.slabs + (uint64_t)slot * a.lay.stride;
-    w.d = reinterpret_cast<D*>(base + a.lay.off_d);
-    w.node = reinterpret_cast<SweepNode*>(base + a.lay.off_sig);
-    w.qa = reinterpret_cast<Idx*>(base + a.lay.off_near);
-    w.qb = reinterpret_cast<Idx*>(base + a.lay.off_far);
-    w.def = reinterpret_cast<Idx*>(base + a.lay.off_far2);
-    w.wide = reinterpret_cast<Idx*>(base + a.lay.off_ends);
-    w.S = reinterpret_cast<Idx*>(base + a.lay.off_S);
-    w.off = reinterpret_cast<uint32_t*>(base + a.lay.off_acc);
-    w.succ = reinterpret_cast<uint32_t*>(base + a.lay.off_pairs);
-    w.succ_cap = a.lay.pair_cap;
-    w.bits2 = reinterpret_cast<uint32_t*>(base + a.lay.off_pend) + 2 * words;
-    if constexpr (MEM == MEM_BITS) {
-      w.bits0 = reinterpret_cast<uint32_t*>(sweep_arrays);
-      w.bits1 = w.bits0 + words;
-    } else {
-      w.bits0 = reinterpret_cast<uint32_t*>(base + a.lay.off_pend);
-      w.bits1 = w.bits0 + words;
-    }
   }
   if constexpr (MEM != MEM_GLOBAL)
     for (uint32_t i = t; i < 2 * words; i += TEAM) w.bits0[i] = 0;

@@ -53,11 +53,10 @@ __device__ __forceinline__ D dmax(D a, D b) {
 
 template <int TEAM>
 __device__ __forceinline__ void team_sync() {
-  if constexpr (TEAM == 32) {
-    __syncwarp();
-  } else {
-    __syncthreads();
-  }
+  // __syncthreads alone does not bring the lanes of a diverged warp back
+  // together; left apart they issue every later instruction twice over
+  __syncwarp();
+  if constexpr (TEAM > 32) __syncthreads();
 }
 
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x) {
