@@ -107,7 +107,8 @@ typedef struct bc_config {
   uint64_t bucket_width;  /* near/far split width, in distance units (>= 1); 0 = tuned value, else the
                              mean over non-empty rows of the row's smallest weight (Delta_node).  With
                              BC_ALGO_DELTA the width of a distance bucket; 0 = tuned value, else one bucket
-                             under landmark bounds and 4 max_weight / (average degree) without */
+                             under landmark bounds, and 4 (average degree below 6: 8) max_weight / (average
+                             degree) without */
   uint64_t phase_cap;     /* device cap on phases + queue refills per source; hitting it returns BC_ERR_TIMEOUT.
                              0 = automatic: 4n + 64, above what any valid input needs (phases <= n,
                              refills <= 3n + 2) */
@@ -384,12 +385,13 @@ int bc_step_destroy(bc_step_t step);
  * before any stream capture.  Calls share the array and each re-initialises
  * it; calls whose work overlaps on the GPU (other streams or threads without
  * ordering) race on it.  On BC_ERR_INVALID no source runs and d_out_bc is all
- * zeros.  The bc_config fields that apply: bucket_width (0 = a fixed 64: the
- * call never reads the weights on the host, so it cannot derive the mean
- * Delta_node that bc_compute uses; pass the graph's own width for high-weight
- * graphs), settle_in, phase_cap, warp_degree and team_degree.  The team size
- * follows the average degree (>= 20: 512, >= 12: 256, else 128 threads); the
- * other fields are ignored.
+ * zeros.  The sweep schedule runs unless one of the bc_config fields of the
+ * strict schedule is set (bucket_width, settle_in, warp_degree, team_degree), algorithm
+ * is BC_ALGO_STRICT or only a strict slab fits; phase_cap applies to both, the other fields are
+ * ignored.  The strict schedule's bucket_width 0 means a fixed 64 (the call
+ * never reads the weights on the host; the sweep schedule's width comes from the
+ * largest weight, found on the device), and its team size follows the average
+ * degree (>= 20: 512, >= 12: 256, else 128 threads).
  */
 #define BC_NOALLOC_SCRATCH_BYTES (64ull << 20)
 int bc_compute_noalloc(const uint64_t *d_row_ptr, const uint32_t *d_col_idx, const uint32_t *d_w, uint32_t n,

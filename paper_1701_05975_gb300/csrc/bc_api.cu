@@ -22,19 +22,11 @@
 
 #include "../../include/bcgpu.h"
 #include "bc_common.h"
+#include "bc_slab.h"
 
 using namespace bcgpu;
 
 namespace {
-
-// Graphs of up to this many vertices run the sweep schedule from shared memory.
-#ifndef BCGPU_SWEEP_SMEM_N
-#define BCGPU_SWEEP_SMEM_N 2048u
-#endif
-constexpr uint32_t SWEEP_SMEM_N = BCGPU_SWEEP_SMEM_N;
-// The vertex bits are in shared memory while 1024 threads' worth of teams
-// keep theirs within this many bytes of an SM's 227 KB.
-constexpr uint32_t SWEEP_BITS_MAX = 212u << 10;
 
 thread_local std::string g_last_error;
 
@@ -68,88 +60,6 @@ bc_config g_cfg = {BC_MODE_BATCHED, 0, 0, 0, 0, 0, 0.0, 0, 0};
 bc_config config_snapshot() {
   std::lock_guard<std::mutex> lk(g_cfg_mu);
   return g_cfg;
-}
-
-uint64_t align256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
-
-// What a workspace's slabs hold: the layouts and the values their arrays keep
-// between sources differ by schedule.
-enum SlabKind : int { SLAB_STRICT = 0, SLAB_SWEEP = 1, SLAB_NONE = 2 };
-
-SlabLayout make_layout(uint32_t n, int dist_bits, SlabKind kind) {
-  SlabLayout L{};
-  uint64_t off = 0;
-  const uint64_t grain = kind == SLAB_NONE ? 16 : 256;
-  auto take = [&](uint64_t bytes) {
-    const uint64_t at = off;
-    off += (bytes + grain - 1) & ~(grain - 1);
-    return at;
-  };
-  if (kind == SLAB_NONE) {
-    // every per-source array in a CTA's shared memory, queue entries in 16 bits
-    L.off_sig = take((uint64_t)n * 16);
-    L.off_d = take((uint64_t)n * (dist_bits / 8));
-    L.off_acc = take((uint64_t)n * 4);
-    L.pair_cap = 3 * n + 64;
-    L.off_pairs = take(((uint64_t)L.pair_cap + 8) * 4);
-    L.off_pend = take((((uint64_t)n + 31) / 32) * 12);
-    for (uint64_t* q : {&L.off_near, &L.off_far, &L.off_far2, &L.off_ends, &L.off_S}) *q = take(((uint64_t)n + 2) * 2);
-    L.smem = (uint32_t)off;
-    L.stride = 256;  // nothing of it is in the slab
-    return L;
-  }
-  const uint64_t w = (uint64_t)n * 4, w2 = ((uint64_t)n + 2) * 4;
-  L.off_d = take((uint64_t)n * (dist_bits / 8));
-  if (kind == SLAB_SWEEP) {
-    L.off_sig = take((uint64_t)n * 16);
-    L.off_near = take(w2);
-    L.off_far = take(w2);
-    L.off_far2 = take(w);
-    L.off_ends = take(w);
-    L.off_S = take(w);
-    L.off_acc = take(w);
-    L.off_pend = take((((uint64_t)n + 31) / 32) * 12);
-    // DAG lists (two words per vertex with successors, then the successors):
-    // 8 n words cover six DAG edges per vertex; a source beyond that walks
-    // the rows again instead
-    L.pair_cap = (uint32_t)std::min<uint64_t>(8ull * n + 64, 0xffffffffull);
-    L.off_pairs = take(((uint64_t)L.pair_cap + 8) * 4);
-    L.stride = off;
-    return L;
-  }
-  L.off_sig = take((uint64_t)n * 8);
-  L.off_S = take(w);
-  L.off_ends = take(w2);
-  L.off_near = take(w);
-  L.off_far = take(w);
-  L.off_far2 = take(w);
-  L.off_acc = take((uint64_t)n * 8);
-  L.off_pend = take(w2);
-  // DAG edge list: 2 n pairs covers every graph whose shortest-path DAG has at
-  // most two in-edges per vertex on average (sources beyond it fall back to
-  // the per-entry backward scan)
-  L.pair_cap = (uint32_t)std::min<uint64_t>(2ull * n + 64, 0xffffffffull);
-  L.off_pairs = take((uint64_t)L.pair_cap * 8);
-  L.off_pair_e = take((uint64_t)L.pair_cap * 4);
-  L.stride = off;
-  return L;
-}
-
-// The values every slab holds between sources: distances INF, backward
-// accumulators (strict) or vertex records and bits (sweep) zero; other arrays are
-// written before they are read.
-cudaError_t init_slabs(char* slabs, const SlabLayout& lay, SlabKind kind, uint32_t slots, uint32_t n, int dist_bits,
-                       cudaStream_t st) {
-  if (kind == SLAB_NONE) return cudaSuccess;
-  cudaError_t e = launch_fill_slabs(slabs, lay.stride, slots, lay.off_d, align256((uint64_t)n * (dist_bits / 8)),
-                                    0xffffffffu, st);
-  if (e != cudaSuccess) return e;
-  if (kind == SLAB_SWEEP) {
-    e = launch_fill_slabs(slabs, lay.stride, slots, lay.off_sig, align256((uint64_t)n * 16), 0u, st);
-    if (e != cudaSuccess) return e;
-    return launch_fill_slabs(slabs, lay.stride, slots, lay.off_pend, align256((((uint64_t)n + 31) / 32) * 8), 0u, st);
-  }
-  return launch_fill_slabs(slabs, lay.stride, slots, lay.off_acc, align256((uint64_t)n * 8), 0u, st);
 }
 
 // Control block of one launch: source counter, status word, counters, debug.
@@ -328,19 +238,7 @@ void plan_sweep(const bc_graph* g, RunCfg& r, bool allow_smem) {
   p.prune = g->kadj != nullptr;
   const double avg_deg = g->n ? (double)g->nnz / g->n : 0.0;
   p.group = (!p.prune && avg_deg >= 12.0) ? 8 : 1;
-  if (r.team >= 128) {
-    if (allow_smem && g->n <= SWEEP_SMEM_N) {
-      p.mem = 2;
-      p.group = 1;
-      p.smem_bytes = make_layout(g->n, g->dist_bits, SLAB_NONE).smem;
-    } else {
-      const uint32_t bits = ((g->act_n + 31) / 32) * 8;
-      if (bits <= SWEEP_BITS_MAX * r.team / 1024) {
-        p.mem = 1;
-        p.smem_bytes = bits;
-      }
-    }
-  }
+  sweep_place(p, g->n, g->act_n, allow_smem);
   r.sweep = p;
 }
 
@@ -352,11 +250,9 @@ uint32_t sweep_team_default(const bc_graph* g) {
 }
 
 // Bucket width of the sweep schedule: one bucket where the landmark bounds
-// leave few vertices to relax; else 4 max_w / (average degree).
+// leave few vertices to relax.
 uint64_t sweep_width_default(const bc_graph* g) {
-  if (g->kadj) return ~0ull;
-  const double avg_deg = g->n ? (double)g->nnz / g->n : 0.0;
-  return (uint64_t)std::max(1.0, 4.0 * g->max_w / std::max(avg_deg, 1.0));
+  return g->kadj ? ~0ull : sweep_bucket_width(g->max_w, g->n, g->nnz);
 }
 
 RunCfg resolve(const bc_graph* g, uint32_t force_algo = BC_ALGO_AUTO) {
@@ -876,10 +772,15 @@ void free_landmarks(bc_graph* g) {
 constexpr double LAND_KEEP_MAX = 0.5;
 constexpr uint32_t LAND_PROBES = 4;
 constexpr uint32_t LAND_MIN_N = 256;
+constexpr uint32_t LAND_MAX_N_FLAT = 32768;
 
 cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<uint64_t>& tdeg) {
   const uint32_t n = g->n;
   if (g->dist_bits != 32 || n < LAND_MIN_N || g->nnz == 0) return cudaSuccess;
+  // without hubs the bounds only help small graphs (the prefix test keeps 28% of
+  // the entries of a degree-16 random graph at n = 1024, 62% at 262144, all of a
+  // grid's): do not pay for 68 searches to find that out
+  if (!g->relabeled && (n > LAND_MAX_N_FLAT || g->nnz < 6ull * n)) return cudaSuccess;
   const uint32_t L = std::min<uint32_t>(SWEEP_MAX_LAND, n / 16);
   std::vector<uint32_t> ids(n);
   for (uint32_t v = 0; v < n; ++v) ids[v] = v;

@@ -141,6 +141,7 @@ struct BatchArgs {
   uint32_t flags;      // RUN_*
   uint32_t* debug_out; // RUN_FORWARD_ONLY: [0] = levels, [1] = reached
   uint32_t* dist_out;  // RUN_DIST_ONLY: [k][n] distances
+  const unsigned long long* width_dev;  // sweep schedule: bucket width in device memory (nullptr: width)
 };
 
 // Strict schedule (bc_batched.cu).  team: 32, 128, 256, 512 or (32-bit
@@ -148,6 +149,18 @@ struct BatchArgs {
 cudaError_t launch_batched(const BatchArgs& a, int dist_bits, int team, int grid, cudaStream_t st);
 int batched_block_threads(int team);
 cudaError_t batched_occupancy(int dist_bits, int team, int* blocks_per_sm);
+
+// Bucket width of the sweep schedule without landmark bounds: 4 max_w /
+// (average degree), twice that below an average degree of 6.  Rounds against
+// entries walked again: Erdos-Renyi 262k (degree 16) 39.5 / 40.6 / 45.8 ms at
+// 1/8, 1/4 (this) and 1/2 max_w; 200 x 200 and 512 x 512 grids 6.2 and 32.9 ms at
+// 1 max_w, 5.8 and 32.5 at 2 (this), 5.6 and 33.4 at 4.
+__host__ __device__ inline unsigned long long sweep_bucket_width(uint32_t max_w, uint32_t n, uint64_t nnz) {
+  if (nnz == 0) return 1;
+  const double deg = (double)nnz / n;
+  const double w = (deg < 6.0 ? 8.0 : 4.0) * max_w / (deg < 1.0 ? 1.0 : deg);
+  return w < 1.0 ? 1ull : (unsigned long long)w;
+}
 
 // Sweep schedule (bc_sweep*.cu): the kernel variant and its dynamic shared memory.
 struct SweepPlan {

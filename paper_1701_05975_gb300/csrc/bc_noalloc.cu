@@ -32,6 +32,7 @@
 
 #include "../../include/bcgpu.h"
 #include "bc_common.h"
+#include "bc_slab.h"
 
 namespace bcgpu {
 namespace {
@@ -89,6 +90,8 @@ struct NaCtl {
   // sums over all entries (v -> u, w) of hash(v, u, w) and of hash(u, v, w):
   // equal for a symmetric CSR (the two multisets are the same)
   unsigned long long sym[2];
+  unsigned long long width;  // sweep schedule: bucket width, from the largest weight
+  uint32_t max_w;
 };
 
 // The device status word carries DEV_* codes; the caller reads them as BC_* codes.
@@ -97,38 +100,6 @@ static_assert(DEV_OK == BC_OK && DEV_ERR_INVALID == BC_ERR_INVALID && DEV_ERR_TI
 
 constexpr uint64_t kCtlBytes = 256;
 static_assert(sizeof(NaCtl) <= kCtlBytes, "control block must fit its reserved bytes");
-
-uint64_t al256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
-
-// Per-source slab with 64-bit distances (weights are not inspected on the
-// host, so the wide distance type is always safe).
-SlabLayout na_layout(uint32_t n) {
-  SlabLayout L{};
-  uint64_t off = 0;
-  L.off_d = off;
-  off += al256((uint64_t)n * 8);
-  L.off_sig = off;
-  off += al256((uint64_t)n * 8);
-  L.off_S = off;
-  off += al256((uint64_t)n * 4);
-  L.off_ends = off;
-  off += al256(((uint64_t)n + 2) * 4);
-  L.off_near = off;
-  off += al256((uint64_t)n * 4);
-  L.off_far = off;
-  off += al256((uint64_t)n * 4);
-  L.off_far2 = off;
-  off += al256((uint64_t)n * 4);
-  L.off_acc = off;
-  off += al256((uint64_t)n * 8);
-  L.off_pend = off;
-  off += al256(((uint64_t)n + 2) * 4);
-  L.pair_cap = (uint32_t)std::min<uint64_t>(2ull * n + 64, 0xffffffffull);
-  L.off_pairs = off;
-  off += al256((uint64_t)L.pair_cap * 8);
-  L.stride = off;
-  return L;
-}
 
 // 64-bit finaliser of SplitMix64 (Steele, Lea and Flood, "Fast splittable
 // pseudorandom number generators", OOPSLA 2014).
@@ -156,6 +127,7 @@ __global__ void na_validate_prep(uint32_t n, uint64_t nnz, const uint64_t* __res
   const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t nth = (uint64_t)gridDim.x * blockDim.x;
   bool bad = false;
+  uint32_t heaviest = 0;
   unsigned long long fwd = 0, rev = 0;
   if (tid == 0 && (row_ptr[0] != 0 || row_ptr[n] != nnz)) bad = true;
   for (uint64_t v = tid; v < n; v += nth) {
@@ -169,6 +141,7 @@ __global__ void na_validate_prep(uint32_t n, uint64_t nnz, const uint64_t* __res
         if (c >= n || ww == 0) bad = true;
         adj[e] = make_uint2(c < n ? c : 0u, ww);
         m = min(m, ww);
+        heaviest = max(heaviest, ww);
         fwd += entry_hash((uint32_t)v, c, ww);
         rev += entry_hash(c, (uint32_t)v, ww);
       }
@@ -180,8 +153,10 @@ __global__ void na_validate_prep(uint32_t n, uint64_t nnz, const uint64_t* __res
   for (int o = 16; o > 0; o >>= 1) {
     fwd += __shfl_xor_sync(0xffffffffu, fwd, o);
     rev += __shfl_xor_sync(0xffffffffu, rev, o);
+    heaviest = max(heaviest, __shfl_xor_sync(0xffffffffu, heaviest, o));
   }
   if ((threadIdx.x & 31) == 0) {
+    atomicMax(&ctl->max_w, heaviest);
     atomicAdd(&ctl->sym[0], fwd);
     atomicAdd(&ctl->sym[1], rev);
   }
@@ -193,8 +168,11 @@ __global__ void na_validate_prep(uint32_t n, uint64_t nnz, const uint64_t* __res
 
 // An asymmetric CSR (some entry without its reverse entry of the same
 // weight) makes the two hash sums differ; it is then rejected like any other
-// invalid input.  Single thread.
-__global__ void na_check_symmetry(NaCtl* ctl) {
+// invalid input.  Also the sweep schedule's bucket width, by the same rule as
+// for a prepared graph (the weights are only known on the device).  Single
+// thread.
+__global__ void na_check_symmetry(NaCtl* ctl, uint32_t n, uint64_t nnz, unsigned long long width) {
+  ctl->width = width ? width : sweep_bucket_width(ctl->max_w, n, nnz);
   if (ctl->sym[0] != ctl->sym[1]) {
     atomicCAS(&ctl->err, DEV_OK, DEV_ERR_INVALID);
     atomicExch(&ctl->counter, 0x80000000u);
@@ -217,16 +195,18 @@ extern "C" int bc_compute_noalloc(const uint64_t* d_row_ptr, const uint32_t* d_c
   if (k > 0 && !d_sources) return na_fail(BC_ERR_INVALID, "bc_compute_noalloc: null sources");
   if (nnz >= (1ull << 32)) return na_fail(BC_ERR_INVALID, "bc_compute_noalloc: nnz must be below 2^32");
   if (k >= 0x80000000u) return na_fail(BC_ERR_INVALID, "bc_compute_noalloc: k must be below 2^31");
-  const SlabLayout lay = na_layout(n);
+  SlabLayout strict_lay = make_layout(n, 64, SLAB_STRICT);
+  strict_lay.stride = strict_lay.off_pair_e;  // its last array is for edge output, which this call has not
+  strict_lay.off_pair_e = 0;
   const uint64_t off_adj = kCtlBytes;
-  const uint64_t off_dnode = off_adj + al256(std::max<uint64_t>(nnz, 1) * 8);
-  const uint64_t off_slabs = off_dnode + al256((uint64_t)n * 4);
-  if (off_slabs + lay.stride > BC_NOALLOC_SCRATCH_BYTES) {
+  const uint64_t off_dnode = off_adj + align256(std::max<uint64_t>(nnz, 1) * 8);
+  const uint64_t off_slabs = off_dnode + align256((uint64_t)n * 4);
+  if (off_slabs + strict_lay.stride > BC_NOALLOC_SCRATCH_BYTES) {
     char msg[256];
     snprintf(msg, sizeof msg,
              "bc_compute_noalloc: graph needs %llu scratch bytes for one source, above the fixed maximum of %llu "
              "(BC_NOALLOC_SCRATCH_BYTES); use bc_graph_create + bc_compute_async",
-             (unsigned long long)(off_slabs + lay.stride), (unsigned long long)BC_NOALLOC_SCRATCH_BYTES);
+             (unsigned long long)(off_slabs + strict_lay.stride), (unsigned long long)BC_NOALLOC_SCRATCH_BYTES);
     return na_fail(BC_ERR_NOMEM, msg);
   }
   int dev = 0;
@@ -251,10 +231,31 @@ extern "C" int bc_compute_noalloc(const uint64_t* d_row_ptr, const uint32_t* d_c
   int sms = 0;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return na_fail(BC_ERR_CUDA, cudaGetErrorString(e));
+  bc_config cfg;
+  bc_get_config(&cfg);
   const double avg_deg = (double)nnz / n;
-  const int team = avg_deg >= 20.0 ? 512 : (avg_deg >= 12.0 ? 256 : 128);
+  int team = avg_deg >= 20.0 ? 512 : (avg_deg >= 12.0 ? 256 : 128);
+  SlabKind kind = SLAB_STRICT;
+  SlabLayout lay = strict_lay;
+  SweepPlan plan;
+  // the sweep schedule unless a knob of the strict one is set; its slab is a
+  // little larger, so a graph of which just one strict slab fits stays strict
+  if (cfg.algorithm != BC_ALGO_STRICT && !cfg.bucket_width && !cfg.settle_in && !cfg.warp_degree &&
+      !cfg.team_degree) {
+    plan.dist_bits = 64;
+    plan.team = 256;
+    plan.group = avg_deg >= 12.0 ? 8 : 1;
+    sweep_place(plan, n, n, true);
+    const SlabKind sk = plan.mem == 2 ? SLAB_NONE : SLAB_SWEEP;
+    const SlabLayout sl = make_layout(n, 64, sk);
+    if (off_slabs + sl.stride <= BC_NOALLOC_SCRATCH_BYTES) {
+      kind = sk;
+      lay = sl;
+      team = plan.team;
+    }
+  }
   int bps = 0;
-  e = batched_occupancy(64, team, &bps);
+  e = kind == SLAB_STRICT ? batched_occupancy(64, team, &bps) : sweep_occupancy(plan, &bps);
   if (e != cudaSuccess) return na_fail(BC_ERR_CUDA, cudaGetErrorString(e));
   const uint32_t per_block = (uint32_t)(batched_block_threads(team) / team);
   uint64_t slots = (uint64_t)std::max(bps, 1) * sms * per_block;
@@ -265,8 +266,6 @@ extern "C" int bc_compute_noalloc(const uint64_t* d_row_ptr, const uint32_t* d_c
   uint2* adj = reinterpret_cast<uint2*>(base + off_adj);
   uint32_t* dnode = reinterpret_cast<uint32_t*>(base + off_dnode);
   char* slabs = base + off_slabs;
-  bc_config cfg;
-  bc_get_config(&cfg);
 
   e = cudaMemsetAsync(ctl, 0, sizeof(NaCtl), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(d_out_bc, 0, (size_t)n * 8, st);
@@ -278,13 +277,10 @@ extern "C" int bc_compute_noalloc(const uint64_t* d_row_ptr, const uint32_t* d_c
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
-    na_check_symmetry<<<1, 1, 0, st>>>(ctl);
+    na_check_symmetry<<<1, 1, 0, st>>>(ctl, n, nnz, cfg.bucket_width);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = launch_fill_slabs(slabs, lay.stride, (uint32_t)slots, lay.off_d, al256((uint64_t)n * 8),
-                                              0xffffffffu, st);
-  if (e == cudaSuccess)
-    e = launch_fill_slabs(slabs, lay.stride, (uint32_t)slots, lay.off_acc, al256((uint64_t)n * 8), 0u, st);
+  if (e == cudaSuccess) e = init_slabs(slabs, lay, kind, (uint32_t)slots, n, 64, st);
   if (e == cudaSuccess) {
     BatchArgs a{};
     a.g.n = n;
@@ -293,6 +289,7 @@ extern "C" int bc_compute_noalloc(const uint64_t* d_row_ptr, const uint32_t* d_c
     a.g.adj = adj;
     a.g.adjp = nullptr;
     a.g.dnode = dnode;
+    a.g.act_n = n;
     a.sources = d_sources;
     a.k = k;
     a.counter = &ctl->counter;
@@ -302,6 +299,7 @@ extern "C" int bc_compute_noalloc(const uint64_t* d_row_ptr, const uint32_t* d_c
     a.lay = lay;
     a.nslots = (uint32_t)slots;
     a.width = cfg.bucket_width ? cfg.bucket_width : 64;
+    a.width_dev = kind == SLAB_STRICT ? nullptr : &ctl->width;
     a.settle_in = cfg.settle_in == 2 ? 0u : 1u;
     a.phase_cap = cfg.phase_cap ? cfg.phase_cap : 4ull * n + 64;  // phases + refills <= 4n + 2
     a.err = &ctl->err;
@@ -311,7 +309,7 @@ extern "C" int bc_compute_noalloc(const uint64_t* d_row_ptr, const uint32_t* d_c
     a.warp_deg = cfg.warp_degree ? cfg.warp_degree : 32u;
     a.team_deg = std::max<uint32_t>(cfg.team_degree ? cfg.team_degree : 8u * team, a.warp_deg);
     const int grid = (int)((slots + per_block - 1) / per_block);
-    e = launch_batched(a, 64, team, grid, st);
+    e = kind == SLAB_STRICT ? launch_batched(a, 64, team, grid, st) : launch_sweep(a, plan, grid, st);
   }
   if (e == cudaSuccess && scale != 1.0) e = launch_scale(d_out_bc, n, scale, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_status, &ctl->err, sizeof(int), cudaMemcpyDeviceToDevice, st);

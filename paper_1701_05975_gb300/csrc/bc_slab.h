@@ -1,0 +1,120 @@
+// Per-source slabs: what they hold for each schedule, and where the sweep
+// schedule keeps its arrays.
+#pragma once
+
+#include <algorithm>
+#include <cstdint>
+
+#include "bc_common.h"
+
+namespace bcgpu {
+
+// Graphs of up to this many vertices run the sweep schedule from shared memory.
+#ifndef BCGPU_SWEEP_SMEM_N
+#define BCGPU_SWEEP_SMEM_N 2048u
+#endif
+constexpr uint32_t SWEEP_SMEM_N = BCGPU_SWEEP_SMEM_N;
+// The vertex bits are in shared memory while 1024 threads' worth of teams
+// keep theirs within this many bytes of an SM's 227 KB.
+constexpr uint32_t SWEEP_BITS_MAX = 212u << 10;
+
+inline uint64_t align256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
+
+// What a workspace's slabs hold: the layouts and the values their arrays keep
+// between sources differ by schedule.
+enum SlabKind : int { SLAB_STRICT = 0, SLAB_SWEEP = 1, SLAB_NONE = 2 };
+
+inline SlabLayout make_layout(uint32_t n, int dist_bits, SlabKind kind) {
+  SlabLayout L{};
+  uint64_t off = 0;
+  const uint64_t grain = kind == SLAB_NONE ? 16 : 256;
+  auto take = [&](uint64_t bytes) {
+    const uint64_t at = off;
+    off += (bytes + grain - 1) & ~(grain - 1);
+    return at;
+  };
+  if (kind == SLAB_NONE) {
+    // every per-source array in a CTA's shared memory, queue entries in 16 bits
+    L.off_sig = take((uint64_t)n * 16);
+    L.off_d = take((uint64_t)n * (dist_bits / 8));
+    L.off_acc = take((uint64_t)n * 4);
+    L.pair_cap = 3 * n + 64;
+    L.off_pairs = take(((uint64_t)L.pair_cap + 8) * 4);
+    L.off_pend = take((((uint64_t)n + 31) / 32) * 12);
+    for (uint64_t* q : {&L.off_near, &L.off_far, &L.off_far2, &L.off_ends, &L.off_S}) *q = take(((uint64_t)n + 2) * 2);
+    L.smem = (uint32_t)off;
+    L.stride = 256;  // nothing of it is in the slab
+    return L;
+  }
+  const uint64_t w = (uint64_t)n * 4, w2 = ((uint64_t)n + 2) * 4;
+  L.off_d = take((uint64_t)n * (dist_bits / 8));
+  if (kind == SLAB_SWEEP) {
+    L.off_sig = take((uint64_t)n * 16);
+    L.off_near = take(w2);
+    L.off_far = take(w2);
+    L.off_far2 = take(w);
+    L.off_ends = take(w);
+    L.off_S = take(w);
+    L.off_acc = take(w);
+    L.off_pend = take((((uint64_t)n + 31) / 32) * 12);
+    // DAG lists (two words per vertex with successors, then the successors):
+    // 8 n words cover six DAG edges per vertex; a source beyond that walks
+    // the rows again instead
+    L.pair_cap = (uint32_t)std::min<uint64_t>(8ull * n + 64, 0xffffffffull);
+    L.off_pairs = take(((uint64_t)L.pair_cap + 8) * 4);
+    L.stride = off;
+    return L;
+  }
+  L.off_sig = take((uint64_t)n * 8);
+  L.off_S = take(w);
+  L.off_ends = take(w2);
+  L.off_near = take(w);
+  L.off_far = take(w);
+  L.off_far2 = take(w);
+  L.off_acc = take((uint64_t)n * 8);
+  L.off_pend = take(w2);
+  // DAG edge list: 2 n pairs covers every graph whose shortest-path DAG has at
+  // most two in-edges per vertex on average (sources beyond it fall back to
+  // the per-entry backward scan)
+  L.pair_cap = (uint32_t)std::min<uint64_t>(2ull * n + 64, 0xffffffffull);
+  L.off_pairs = take((uint64_t)L.pair_cap * 8);
+  L.off_pair_e = take((uint64_t)L.pair_cap * 4);
+  L.stride = off;
+  return L;
+}
+
+// The values every slab holds between sources: distances INF, backward
+// accumulators (strict) or vertex records and bits (sweep) zero; other arrays are
+// written before they are read.
+inline cudaError_t init_slabs(char* slabs, const SlabLayout& lay, SlabKind kind, uint32_t slots, uint32_t n, int dist_bits,
+                       cudaStream_t st) {
+  if (kind == SLAB_NONE) return cudaSuccess;
+  cudaError_t e = launch_fill_slabs(slabs, lay.stride, slots, lay.off_d, align256((uint64_t)n * (dist_bits / 8)),
+                                    0xffffffffu, st);
+  if (e != cudaSuccess) return e;
+  if (kind == SLAB_SWEEP) {
+    e = launch_fill_slabs(slabs, lay.stride, slots, lay.off_sig, align256((uint64_t)n * 16), 0u, st);
+    if (e != cudaSuccess) return e;
+    return launch_fill_slabs(slabs, lay.stride, slots, lay.off_pend, align256((((uint64_t)n + 31) / 32) * 8), 0u, st);
+  }
+  return launch_fill_slabs(slabs, lay.stride, slots, lay.off_acc, align256((uint64_t)n * 8), 0u, st);
+}
+
+// Memory form of a sweep plan whose distance width and team are set: n
+// vertices, the ones from act_n on without entries.
+inline void sweep_place(SweepPlan& p, uint32_t n, uint32_t act_n, bool allow_smem) {
+  p.mem = 0;
+  p.smem_bytes = 0;
+  if (p.team < 128) return;
+  const uint64_t bits = ((uint64_t)act_n + 31) / 32 * 8;
+  if (allow_smem && n <= SWEEP_SMEM_N) {
+    p.mem = 2;
+    p.group = 1;
+    p.smem_bytes = make_layout(n, p.dist_bits, SLAB_NONE).smem;
+  } else if (bits <= (uint64_t)SWEEP_BITS_MAX * p.team / 1024) {
+    p.mem = 1;
+    p.smem_bytes = (uint32_t)bits;
+  }
+}
+
+}  // namespace bcgpu

@@ -97,9 +97,7 @@ struct SweepTeam {
   static constexpr bool SM = MEM == MEM_ALL;
   using Idx = typename std::conditional<SM, uint16_t, uint32_t>::type;
   static constexpr int NW = TEAM / 32;
-  // entries that one thread walks before its warp helps: small graphs run at
-  // latency, so more of them at once
-  static constexpr uint32_t FIRST = SM ? 8 : 4;
+  static constexpr uint32_t FIRST = 4;  // entries that one thread walks before its warp helps
 
   const BatchArgs& a;
   Sh& sh;
@@ -118,6 +116,7 @@ struct SweepTeam {
   uint32_t nrelax, nscan, nreach;
   uint32_t sel;   // rotates over qlen / nwide / nteam
   bool seeded, stream;
+  uint64_t width;  // bucket width, all ones = one bucket
 
   __device__ SweepTeam(const BatchArgs& args, Sh& shared, int thread) : a(args), sh(shared), t(thread) {}
 
@@ -507,7 +506,7 @@ struct SweepTeam {
 
   __device__ __forceinline__ int distances(uint32_t& rounds, uint32_t& advances) {
     const D INF = dinf<D>();
-    D bound = (seeded || a.width == ~0ull) ? INF : sat_add<D>((D)0, a.width);
+    D bound = (seeded || width == ~0ull) ? INF : sat_add<D>((D)0, width);
     const uint32_t order_min = TEAM > 32 ? a.g.n / SW_ORDER + TEAM : ~0u;
     uint32_t len = 1;
     Idx *cur = qa, *nxt = qb;
@@ -575,7 +574,7 @@ struct SweepTeam {
           if (du >= bound) lo = dmin(lo, du);
         }
         team_min2<D, TEAM>(lo, dummy, sh.red);
-        const D nb = lo == INF ? bound : sat_add<D>(lo, a.width);
+        const D nb = lo == INF ? bound : sat_add<D>(lo, width);
         if (t == 0) sh.ndef = 0;
         team_sync<TEAM>();
         for (uint32_t j = t; j < dl; j += TEAM) {
@@ -1415,7 +1414,7 @@ struct SweepTeam {
       }
       if (in_land) C = (int32_t)c;  // a source that does not reach the landmark walks whole rows
     }
-    seeded = PRUNE && in_land && a.width == ~0ull;
+    seeded = PRUNE && in_land && width == ~0ull;
     if (dirty && !seeded) {
       fill_distances();
       dirty = false;
@@ -1548,6 +1547,7 @@ __global__ void __launch_bounds__(BLOCK, (sweep_min_blocks<D, TEAM, BLOCK>())) b
   SweepShared<D, TEAM>& sh = shared_teams[team];
   T w(a, sh, t);
   w.sel = 0;
+  w.width = a.width_dev ? (uint64_t)__ldg(a.width_dev) : a.width;
   if (t < 3) sh.qlen[t] = sh.nwide[t] = sh.nteam[t] = 0;
   bool dirty = false;
   const uint32_t words = (a.g.act_n + 31) / 32;

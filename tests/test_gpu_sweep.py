@@ -132,3 +132,24 @@ def test_directed_landmarks_and_unreached_parts(isolated):
             assert_bc_close(G.compute(src, 1.0), oracle.bc_directed(g, src, 1.0))
             ebc, _ = G.edge_compute(src, 1.0)
             assert_bc_close(ebc, oracle.edge_bc(g, src, 1.0))
+
+
+@pytest.mark.parametrize("n,per,wmax", [(2048, 4, 300), (2049, 12, 300), (6000, 2, 1), (3000, 8, 1 << 30)])
+def test_noalloc_runs_the_sweep_schedule_with_64bit_words(n, per, wmax):
+    """bc_compute_noalloc: arrays in shared memory up to 2048 vertices, slabs
+    above, the bucket width from the largest weight on the device."""
+    torch = pytest.importorskip("torch")
+    g = gen.er_graph(n, per * n, 1, wmax, seed=n)
+    src = np.arange(0, n, max(1, n // 61), dtype=np.uint32)
+    dev = lambda x, t: torch.from_numpy(np.ascontiguousarray(x).view(t)).cuda()  # noqa: E731
+    rp, col, w = dev(g.row_ptr, np.int64), dev(g.col, np.int32), dev(g.w, np.int32)
+    d_src, out = dev(src, np.int32), torch.empty(n, dtype=torch.float64, device="cuda")
+    status = torch.full((1,), 9, dtype=torch.int32, device="cuda")
+    st = torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())  # the inputs are written on the current stream
+    for _ in range(2):
+        bc.bc_compute_noalloc(rp.data_ptr(), col.data_ptr(), w.data_ptr(), n, g.nnz, d_src.data_ptr(), len(src), 0.5,
+                              out.data_ptr(), status.data_ptr(), st.cuda_stream)
+        st.synchronize()
+        assert int(status.item()) == bc.BC_OK
+        assert_bc_close(out.cpu().numpy(), oracle.bc(g, src, 0.5))
