@@ -222,6 +222,7 @@ struct RunCfg {
   uint32_t warp_deg;
   uint32_t team_deg;
   uint32_t algo;  // ALGO_STRICT or ALGO_DELTA
+  bool algo_auto; // not asked for by the configuration or the caller
   uint32_t hot_n;
   SweepPlan sweep;  // ALGO_DELTA
 };
@@ -242,11 +243,30 @@ void plan_sweep(const bc_graph* g, RunCfg& r, bool allow_smem) {
   r.sweep = p;
 }
 
-// Threads per source of the sweep schedule.
-uint32_t sweep_team_default(const bc_graph* g) {
+// Threads per source of the sweep schedule for a run of k sources (0: many).
+// Teams of T threads run 1024 / T to an SM.  Sparse graphs without landmarks
+// have small frontiers in many rounds, so latency counts: the widest team that
+// still has every source in flight at once, 128 where none has (1024 sources of
+// a 256 x 256 grid: 12.4 ms at 128 threads, 17.1 at 256; 512 sources of a 512 x
+// 512 one: 44.0 and 32.6).  The others by size, the frontiers growing with it
+// (BA 4096 2.06 / 2.40 / 3.39 ms at 128 / 256 / 512, BA 16k 15.4 / 14.8 / 15.6,
+// BA 65k 17.0 / 16.3 / 14.9, Erdos-Renyi 65k 47.5 / 36.2 / 28.9 and 25.3 at 1024,
+// R-MAT scale 20 359 / 305 / 270 / 222 at 128 / 256 / 512 / 1024), doubled while
+// that leaves no source waiting.
+uint32_t sweep_team_default(const bc_graph* g, uint32_t k) {
   const double avg_deg = g->n ? (double)g->nnz / g->n : 0.0;
-  if (avg_deg < 6.0 || g->n < 32768) return 256u;
-  return g->n < 131072 ? 512u : 1024u;
+  const uint32_t wide = g->dist_bits == 32 ? 1024u : 512u;
+  auto in_flight = [&](uint32_t team) { return (uint64_t)g->sm_count * (1024 / team); };
+  if (!g->kadj && avg_deg < 6.0) {
+    // 64-bit words spill at 512 threads (200 x 200 grid, 304 sources: 5.6 ms at 256, 5.9 at 512)
+    if (k && g->dist_bits == 32 && in_flight(512) >= k) return 512u;
+    return k && in_flight(256) >= k ? 256u : 128u;
+  }
+  if (g->n <= SWEEP_SMEM_N) return 256u;
+  uint32_t team = g->n < 4096 || (g->n < 8192 && avg_deg < 12.0) ? 128u
+                  : g->n < 32768 ? 256u : (g->n < 131072 && g->kadj ? 512u : wide);
+  while (k && team < wide && in_flight(2 * team) >= k) team *= 2;
+  return team;
 }
 
 // Bucket width of the sweep schedule: one bucket where the landmark bounds
@@ -255,7 +275,8 @@ uint64_t sweep_width_default(const bc_graph* g) {
   return g->kadj ? ~0ull : sweep_bucket_width(g->max_w, g->n, g->nnz);
 }
 
-RunCfg resolve(const bc_graph* g, uint32_t force_algo = BC_ALGO_AUTO) {
+// k: sources of the run (0: not known, many).
+RunCfg resolve(const bc_graph* g, uint32_t k, uint32_t force_algo = BC_ALGO_AUTO) {
   bc_config c = config_snapshot();
   if (force_algo) c.algorithm = force_algo;
   RunCfg r;
@@ -276,10 +297,11 @@ RunCfg resolve(const bc_graph* g, uint32_t force_algo = BC_ALGO_AUTO) {
                                      ? (uint32_t)BC_ALGO_STRICT
                                      : (g->tuned.algo ? g->tuned.algo : (uint32_t)BC_ALGO_DELTA));
   r.algo = (al == BC_ALGO_DELTA) ? ALGO_DELTA : ALGO_STRICT;
+  r.algo_auto = c.algorithm == BC_ALGO_AUTO;
   const bool sweep = r.algo == ALGO_DELTA;
   const uint32_t tuned_team = sweep ? g->tuned.sweep_team : g->tuned.team;
   r.team = c.team_threads ? c.team_threads
-                          : (tuned_team ? tuned_team : (sweep ? sweep_team_default(g) : team_default));
+                          : (tuned_team ? tuned_team : (sweep ? sweep_team_default(g, k) : team_default));
   if (r.team == 1024 && g->dist_bits != 32) r.team = 512;  // 1024-thread teams hold 32-bit distances only
   const uint64_t tuned_width = sweep ? g->tuned.sweep_width : g->tuned.width;
   r.width = c.bucket_width ? c.bucket_width
@@ -315,18 +337,24 @@ cudaError_t launch_run(const BatchArgs& a, const bc_graph* g, const RunCfg& r, i
                               : launch_batched(a, g->dist_bits, (int)r.team, grid, st);
 }
 
-// Number of sources in flight for a run of k sources.
-int plan_slots(const bc_graph* g, const RunCfg& r, uint32_t k, uint32_t* slots_out) {
+// Number of sources in flight for a run of k sources.  A sweep slab is a
+// quarter larger than a strict one: where the memory fraction holds none and
+// the schedule was not asked for, the run (r) becomes a strict one.
+int plan_slots(const bc_graph* g, RunCfg& r, uint32_t k, uint32_t* slots_out) {
+  size_t free_b = 0, total_b = 0;
+  CK(cudaMemGetInfo(&free_b, &total_b));
+  const uint64_t budget = (uint64_t)((double)free_b * r.mem_fraction);
+  uint64_t stride = make_layout(g->n, g->dist_bits, slab_kind(r)).stride;
+  if (stride > budget && r.algo == ALGO_DELTA && r.algo_auto) {
+    r = resolve(g, k, BC_ALGO_STRICT);
+    stride = make_layout(g->n, g->dist_bits, SLAB_STRICT).stride;
+  }
   int bps = 0;
   cudaError_t e = run_occupancy(g, r, &bps);
   if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
   const uint32_t per_block = (uint32_t)(batched_block_threads((int)r.team) / (int)r.team);
   uint64_t slots = (uint64_t)std::max(bps, 1) * g->sm_count * per_block;
-  size_t free_b = 0, total_b = 0;
-  CK(cudaMemGetInfo(&free_b, &total_b));
-  const uint64_t stride = make_layout(g->n, g->dist_bits, slab_kind(r)).stride;
-  const uint64_t by_mem = (uint64_t)((double)free_b * r.mem_fraction) / std::max<uint64_t>(stride, 1);
-  slots = std::min<uint64_t>(slots, by_mem);
+  slots = std::min<uint64_t>(slots, budget / std::max<uint64_t>(stride, 1));
   if (r.max_slots) slots = std::min<uint64_t>(slots, r.max_slots);
   slots = std::min<uint64_t>(slots, std::max<uint32_t>(k, 1));
   if (slots == 0) return fail(BC_ERR_NOMEM, "device memory too small for one per-source slab (%llu bytes)",
@@ -589,15 +617,15 @@ int check_graph(bc_graph_t g) {
 
 // Synchronous batched run with host sources and host outputs.
 int compute_sync(bc_graph* g, const uint32_t* sources, uint32_t k, double scale, double* out_bc, double* out_ebc,
-                 const RunCfg& r) {
+                 RunCfg r) {
   for (uint32_t i = 0; i < k; ++i)
     if (sources[i] >= g->n) return fail(BC_ERR_INVALID, "source %u out of range (n = %u)", sources[i], g->n);
-  if (out_ebc && r.algo == ALGO_STRICT)
-    if (int rc = ensure_edge_map(g)) return rc;
   cudaStream_t st = g->stream;
   uint32_t slots = 0;
   int rc = plan_slots(g, r, k, &slots);
   if (rc) return rc;
+  if (out_ebc && r.algo == ALGO_STRICT)
+    if ((rc = ensure_edge_map(g))) return rc;
   Workspace* w = nullptr;
   if ((rc = ws_acquire(g, slab_kind(r), slots, k, st, &w))) return rc;
   if (k) {
@@ -811,7 +839,7 @@ cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<u
     return p;
   };
   cudaStream_t st = g->stream;
-  RunCfg r = resolve(g, BC_ALGO_DELTA);
+  RunCfg r = resolve(g, 0, BC_ALGO_DELTA);
   r.team = n >= 16384 ? 1024u : 256u;
   r.width = sweep_width_default(g);
   r.phase_cap = 4ull * n + 64;
@@ -927,8 +955,13 @@ uint32_t bcgpu::graph_n(const bc_graph* g) { return g->n; }
 uint64_t bcgpu::graph_nnz(const bc_graph* g) { return g->nnz; }
 void bcgpu::graph_serving_ref(bc_graph* g, int delta) { g->serving_refs += delta; }
 
-int bcgpu::serve_plan(bc_graph* g, ServePlan* out) {
-  RunCfg r = resolve(g);
+int bcgpu::serve_plan(bc_graph* g, uint32_t k, uint64_t budget, ServePlan* out) {
+  RunCfg r = resolve(g, k);
+  out->fixed_bytes = (uint64_t)g->n * 16 + 4096;
+  if (r.algo == ALGO_DELTA && r.algo_auto &&
+      make_layout(g->n, g->dist_bits, slab_kind(r)).stride + out->fixed_bytes > budget)
+    r = resolve(g, k, BC_ALGO_STRICT);
+  out->algorithm = r.algo == ALGO_DELTA ? BC_ALGO_DELTA : BC_ALGO_STRICT;
   int bps = 0;
   cudaError_t e = run_occupancy(g, r, &bps);
   if (e != cudaSuccess) return cuda_fail(e, "occupancy");
@@ -936,15 +969,14 @@ int bcgpu::serve_plan(bc_graph* g, ServePlan* out) {
   out->team = r.team;
   out->max_slots = (uint32_t)std::max(bps, 1) * (uint32_t)g->sm_count * per_block;
   out->slot_bytes = make_layout(g->n, g->dist_bits, slab_kind(r)).stride;
-  out->fixed_bytes = (uint64_t)g->n * 16 + 4096;
   return BC_OK;
 }
 
-int bcgpu::serve_open(bc_graph* g, const uint32_t* sources, uint32_t k, uint32_t slot_cap, cudaStream_t st,
-                      ServeLease** out) {
+int bcgpu::serve_open(bc_graph* g, const ServePlan& plan, const uint32_t* sources, uint32_t k, uint32_t slot_cap,
+                      cudaStream_t st, ServeLease** out) {
   Workspace* w = nullptr;
   const uint32_t cap = std::max<uint32_t>(slot_cap, 1);
-  RunCfg r = resolve(g);
+  RunCfg r = resolve(g, k, plan.algorithm);
   r.mode = BC_MODE_BATCHED;
   int rc = ws_acquire(g, slab_kind(r), cap, k, st, &w);
   if (rc) return rc;
@@ -1322,7 +1354,7 @@ int bc_graph_get_info(bc_graph_t g, bc_graph_info* out) {
   out->max_weight = g->max_w;
   out->dist_bits = (uint32_t)g->dist_bits;
   out->device_bytes = g->device_bytes;
-  out->slab_bytes = make_layout(g->n, g->dist_bits, slab_kind(resolve(g))).stride;
+  out->slab_bytes = make_layout(g->n, g->dist_bits, slab_kind(resolve(g, 0))).stride;
   out->relabeled = g->relabeled ? 1u : 0u;
   out->directed = g->directed ? 1u : 0u;
   return BC_OK;
@@ -1333,7 +1365,7 @@ int bc_compute(bc_graph_t g, const uint32_t* sources, uint32_t k, double scale, 
   if (!out_bc) return fail(BC_ERR_INVALID, "null out_bc");
   if (k && !sources) return fail(BC_ERR_INVALID, "null sources");
   CK(cudaSetDevice(g->device));
-  RunCfg r = resolve(g);
+  RunCfg r = resolve(g, k);
   if (r.mode == BC_MODE_PLAIN) return compute_plain(g, sources, k, scale, out_bc, r);
   return compute_sync(g, sources, k, scale, out_bc, nullptr, r);
 }
@@ -1349,10 +1381,8 @@ int compute_async(bc_graph* g, const uint32_t* d_sources, uint32_t k, double sca
   if (!d_out_bc) return fail(BC_ERR_INVALID, "null d_out_bc");
   if (k && !d_sources) return fail(BC_ERR_INVALID, "null d_sources");
   CK(cudaSetDevice(g->device));
-  RunCfg r = resolve(g);
+  RunCfg r = resolve(g, k);
   if (r.mode != BC_MODE_BATCHED) return fail(BC_ERR_INVALID, "the async entry points run the batched mode only");
-  if (d_out_ebc && r.algo == ALGO_STRICT)
-    if (int rc = ensure_edge_map(g)) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the workspace this stream kept from its previous async call: that run
   // and its status copy are ordered before this one on the stream
@@ -1369,6 +1399,8 @@ int compute_async(bc_graph* g, const uint32_t* d_sources, uint32_t k, double sca
   uint32_t slots = 0;
   int rc = plan_slots(g, r, k, &slots);
   if (rc) return rc;
+  if (d_out_ebc && r.algo == ALGO_STRICT)
+    if ((rc = ensure_edge_map(g))) return rc;
   Workspace* w = nullptr;
   if ((rc = ws_acquire(g, slab_kind(r), slots, 0, st, &w))) return rc;
   rc = enqueue_batched(g, w, r, d_sources, k, scale, d_out_bc, d_out_ebc, slots, 0, st, true);
@@ -1458,7 +1490,7 @@ int bc_edge_compute(bc_graph_t g, const uint32_t* sources, uint32_t k, double sc
   if (!out_ebc) return fail(BC_ERR_INVALID, "null out_ebc");
   if (k && !sources) return fail(BC_ERR_INVALID, "null sources");
   CK(cudaSetDevice(g->device));
-  RunCfg r = resolve(g);
+  RunCfg r = resolve(g, k);
   std::vector<double> tmp;
   if (!out_bc) {
     tmp.resize(g->n);
@@ -1473,7 +1505,7 @@ int bc_sssp_debug(bc_graph_t g, uint32_t s, uint64_t* out_dist, double* out_sigm
   CK(cudaSetDevice(g->device));
   // the strict schedule's levels unless the sweep schedule is asked for by name
   const bool sweep = config_snapshot().algorithm == BC_ALGO_DELTA;
-  RunCfg r = resolve(g, sweep ? BC_ALGO_DELTA : BC_ALGO_STRICT);
+  RunCfg r = resolve(g, 1, sweep ? BC_ALGO_DELTA : BC_ALGO_STRICT);
   plan_sweep(g, r, false);  // the arrays are read back from a slab
   cudaStream_t st = g->stream;
   Workspace* w = nullptr;
@@ -1541,7 +1573,7 @@ int bc_compute_paper_variant(bc_graph_t g, const uint32_t* sources, uint32_t k, 
   for (uint32_t i = 0; i < k; ++i)
     if (sources[i] >= g->n) return fail(BC_ERR_INVALID, "source %u out of range (n = %u)", sources[i], g->n);
   CK(cudaSetDevice(g->device));
-  RunCfg r = resolve(g);
+  RunCfg r = resolve(g, k);
   cudaStream_t st = g->stream;
   if (!g->paper) {
     cudaError_t e;
@@ -1606,16 +1638,19 @@ int bc_autotune(bc_graph_t g, const uint32_t* sources, uint32_t k_probe) {
   // bounds), then sources in flight
   double sweep_ms = 1e300;
   if (try_sweep) {
-    RunCfg base = resolve(g, BC_ALGO_DELTA);
+    RunCfg base = resolve(g, k_probe, BC_ALGO_DELTA);
     base.mode = BC_MODE_BATCHED;
     base.max_slots = user.max_slots;
-    if (int rc = timed(base, &ms)) return rc;  // warm-up: workspace allocation
+    const int first = timed(base, &ms);  // warm-up: workspace allocation
+    // a memory fraction that only holds strict slabs leaves the strict schedule
+    const bool fits = !(first == BC_ERR_NOMEM && try_strict);
+    if (first && fits) return first;
     const uint64_t w0 = sweep_width_default(g);
     std::vector<uint64_t> sw = {w0};
     if (!g->kadj) sw = {std::max<uint64_t>(1, w0 / 2), w0, 2 * w0, 4 * w0};
     if (user.bucket_width) sw = {user.bucket_width};
     for (uint32_t team : teams) {
-      if (user.team_threads && user.team_threads != team) continue;
+      if (!fits || (user.team_threads && user.team_threads != team)) continue;
       for (uint64_t width : sw) {
         RunCfg r = base;
         r.team = team;
@@ -1645,10 +1680,10 @@ int bc_autotune(bc_graph_t g, const uint32_t* sources, uint32_t k_probe) {
         best.sweep_slots = r.max_slots;
       }
     }
-    best.algo = BC_ALGO_DELTA;
+    if (fits) best.algo = BC_ALGO_DELTA;
   }
   if (try_strict) {
-    RunCfg base = resolve(g, BC_ALGO_STRICT);
+    RunCfg base = resolve(g, k_probe, BC_ALGO_STRICT);
     base.mode = BC_MODE_BATCHED;
     base.settle_in = 1;
     base.refine = (g->dnode2 && user.settle_in == 1) ? 1u : 0u;
@@ -1777,12 +1812,12 @@ int bc_step_create(bc_graph_t g, const uint32_t* d_sources, uint32_t k, double s
   if (!d_out_bc) return fail(BC_ERR_INVALID, "null d_out_bc");
   if (k && !d_sources) return fail(BC_ERR_INVALID, "null d_sources");
   CK(cudaSetDevice(g->device));
-  RunCfg r = resolve(g);
+  RunCfg r = resolve(g, k);
   if (r.mode != BC_MODE_BATCHED) return fail(BC_ERR_INVALID, "step graphs capture the batched mode only");
   auto s = std::make_unique<bc_step>();
   s->g = g;
-  s->r = r;
   if (int rc = plan_slots(g, r, k, &s->slots)) return rc;
+  s->r = r;
   Workspace& w = s->ws;
   w.slots = s->slots;
   w.kind = slab_kind(r);

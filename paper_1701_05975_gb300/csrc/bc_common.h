@@ -250,14 +250,16 @@ namespace bcgpu {
 // workspace.
 struct ServeLease;
 struct ServePlan {
+  uint32_t algorithm;   // BC_ALGO_STRICT or BC_ALGO_DELTA: the lease's slabs belong to it
   uint32_t team;        // threads per source
   uint32_t max_slots;   // sources the GPU holds at once for this team size
   uint64_t slot_bytes;  // device bytes per source in flight
   uint64_t fixed_bytes; // per-request device bytes besides the slabs
 };
-int serve_plan(bc_graph* g, ServePlan* out);
+// budget: device bytes a request may take (a strict slab is smaller than a sweep one).
+int serve_plan(bc_graph* g, uint32_t k, uint64_t budget, ServePlan* out);
 // Reserve a workspace of up to slot_cap slabs and stage the sources (on st).
-int serve_open(bc_graph* g, const uint32_t* sources, uint32_t k, uint32_t slot_cap, cudaStream_t st,
+int serve_open(bc_graph* g, const ServePlan& plan, const uint32_t* sources, uint32_t k, uint32_t slot_cap, cudaStream_t st,
                ServeLease** out);
 uint32_t serve_slot_cap(const ServeLease* l);  // slabs actually held
 // Enqueue sources [first, first + count) with `slots` of them in flight; the

@@ -183,7 +183,7 @@ struct Server {
   // Admission of the head of the queue: its workspace within the memory budget.
   // Returns false when it has to wait for memory.
   bool try_open(std::shared_ptr<Request>& r) {
-    if (serve_plan(r->g, &r->plan) != BC_OK) {
+    if (serve_plan(r->g, (uint32_t)r->sources.size(), mem_budget(), &r->plan) != BC_OK) {
       retire(r, BC_REQ_FAILED, BC_ERR_CUDA);
       return true;
     }
@@ -194,7 +194,7 @@ struct Server {
     if (free_mem < p.fixed_bytes + p.slot_bytes) return false;
     cap = std::min<uint64_t>(cap, (free_mem - p.fixed_bytes) / p.slot_bytes);
     ServeLease* lease = nullptr;
-    const int rc = serve_open(r->g, r->sources.data(), (uint32_t)r->sources.size(), (uint32_t)cap, open_stream,
+    const int rc = serve_open(r->g, p, r->sources.data(), (uint32_t)r->sources.size(), (uint32_t)cap, open_stream,
                               &lease);
     if (rc != BC_OK) {
       retire(r, BC_REQ_FAILED, rc);
@@ -383,7 +383,7 @@ int bc_request_submit(bc_graph_t g, const uint32_t* sources, uint32_t k, double 
   std::lock_guard<std::mutex> lk(s.mu);
   if (int rc = s.ensure_started(graph_device(g))) return rc;
   ServePlan p;
-  if (int rc = serve_plan(g, &p)) return rc;
+  if (int rc = serve_plan(g, k, s.mem_budget(), &p)) return rc;
   if (p.fixed_bytes + p.slot_bytes > s.mem_budget())
     return set_error(BC_ERR_NOMEM, "bc_request_submit: one source of this graph needs more device memory than the "
                                    "serving budget");

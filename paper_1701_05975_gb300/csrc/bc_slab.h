@@ -9,11 +9,12 @@
 
 namespace bcgpu {
 
-// Graphs of up to this many vertices run the sweep schedule from shared memory.
-#ifndef BCGPU_SWEEP_SMEM_N
-#define BCGPU_SWEEP_SMEM_N 2048u
-#endif
-constexpr uint32_t SWEEP_SMEM_N = BCGPU_SWEEP_SMEM_N;
+// Graphs of up to this many vertices run the sweep schedule from shared memory:
+// three 256-thread teams to an SM at 1536 (46 bytes per vertex).  Against slabs,
+// all sources, best team of each: Erdos-Renyi 600 184 / 257 us, 1024 386 / 451,
+// 1500 818 / 929, 2048 1356 / 1461; BA 1500 501 / 549, 2048 843 / 676; 45 x 45 grid
+// 2673 / 1737 (two teams to an SM there).
+constexpr uint32_t SWEEP_SMEM_N = 1536;
 // The vertex bits are in shared memory while 1024 threads' worth of teams
 // keep theirs within this many bytes of an SM's 227 KB.
 constexpr uint32_t SWEEP_BITS_MAX = 212u << 10;

@@ -82,8 +82,8 @@ def two_parts(seed):
 CASES = {
     "landmark-min-n": lambda: hubs(256, 1500, 60, 1),
     "below-landmark-n": lambda: hubs(255, 1500, 60, 2),
-    "shared-memory-last": lambda: hubs(2048, 9000, 200, 3),
-    "shared-memory-past": lambda: hubs(2049, 9000, 200, 4),
+    "shared-memory-last": lambda: hubs(1536, 9000, 200, 3),
+    "shared-memory-past": lambda: hubs(1537, 9000, 200, 4),
     "bits-word-edge": lambda: hubs(2080, 9000, 200, 5, isolated=0),
     "bits-isolated-tail": lambda: hubs(4000, 9000, 200, 6, isolated=1441),
     "row-of-4-5-20-21": lambda: build(2200, np.repeat([0, 1, 2, 3], [4, 5, 20, 21]), np.arange(10, 60),
@@ -134,9 +134,9 @@ def test_directed_landmarks_and_unreached_parts(isolated):
             assert_bc_close(ebc, oracle.edge_bc(g, src, 1.0))
 
 
-@pytest.mark.parametrize("n,per,wmax", [(2048, 4, 300), (2049, 12, 300), (6000, 2, 1), (3000, 8, 1 << 30)])
+@pytest.mark.parametrize("n,per,wmax", [(1536, 4, 300), (1537, 12, 300), (6000, 2, 1), (3000, 8, 1 << 30)])
 def test_noalloc_runs_the_sweep_schedule_with_64bit_words(n, per, wmax):
-    """bc_compute_noalloc: arrays in shared memory up to 2048 vertices, slabs
+    """bc_compute_noalloc: arrays in shared memory up to 1536 vertices, slabs
     above, the bucket width from the largest weight on the device."""
     torch = pytest.importorskip("torch")
     g = gen.er_graph(n, per * n, 1, wmax, seed=n)
@@ -153,3 +153,29 @@ def test_noalloc_runs_the_sweep_schedule_with_64bit_words(n, per, wmax):
         st.synchronize()
         assert int(status.item()) == bc.BC_OK
         assert_bc_close(out.cpu().numpy(), oracle.bc(g, src, 0.5))
+
+
+def test_memory_fraction_that_only_holds_strict_slabs():
+    """A sweep slab is a quarter larger than a strict one: a budget between the
+    two runs the strict schedule on every entry point, as it did before."""
+    torch = pytest.importorskip("torch")
+    g = gen.ba_graph(3000, 4, 1, 100, seed=31)
+    src = np.arange(0, g.n, 97, dtype=np.uint32)
+    want = oracle.bc(g, src, 0.5)
+    with bc.Graph(g) as G:
+        sweep = G.info().slab_bytes
+        bc.bc_set_config(algorithm=bc.BC_ALGO_STRICT)
+        strict = G.info().slab_bytes
+        assert strict < sweep
+        free_b = torch.cuda.mem_get_info()[0]
+        bc.bc_set_config(algorithm=bc.BC_ALGO_AUTO, mem_fraction=(strict + sweep) / 2 / free_b)
+        assert_bc_close(G.compute(src, 0.5), want)
+        assert G.stats().algorithm == bc.BC_ALGO_STRICT and G.stats().slots == 1
+        ebc, _ = G.edge_compute(src, 0.5)
+        assert_bc_close(ebc, oracle.edge_bc(g, src, 0.5))
+        G.autotune(src)
+        assert_bc_close(G.compute(src, 0.5), want)
+        bc.bc_set_config(algorithm=bc.BC_ALGO_DELTA)
+        with pytest.raises(bc.BCError) as ei:
+            G.compute(src, 0.5)
+        assert ei.value.code == bc.BC_ERR_NOMEM
