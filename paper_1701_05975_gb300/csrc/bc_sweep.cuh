@@ -33,6 +33,26 @@
 // shortest path never fails the test (d(v) + w = d(s, u) <= D(s, h) + D(h, u)),
 // so distances, sigma and the DAG are exact.  Same idea as the landmark bounds
 // of A* search (Goldberg and Harrelson, SODA 2005), here as a row order.
+//
+// What bounds it (GB300, per pass; the strict schedule on the same graphs in
+// brackets): R-MAT scale 20, 4096 sources: 220 ms (855), 1.0 TB of DRAM traffic
+// (3.9) at 0.63-0.67 of the measured bandwidth: random distance gathers of the
+// DAG build (35% of the cycles) and of the rounds (22%), 2.2 gathers per DAG edge.
+// Barabasi-Albert 65k, 2048 sources: 15 ms (72), 31% DAG build, 40% the passes
+// over the lists, latency of their dependent loads.  Erdos-Renyi 262k, 256 sources:
+// 39 ms (83): no landmarks, every entry walked 2.2 times; 152 teams hold 256
+// sources in two unequal waves.  512 x 512 grid, 512 sources: 32 ms (110): 1530 rounds
+// and 2 x 805 levels of ~300 vertices each, ~7 us a round (six dependent L2 round
+// trips and a barrier).  1024 vertices in shared memory, 1024 sources: 0.39-0.42 ms
+// (0.94): 608 teams for 1024 sources, ~35 steps of ~9 k cycles.
+//
+// Why these forms (BA 65k / R-MAT scale 20, ms, each against the one before):
+// predecessor counts and round stamps by atomics on the records 30.9 / 441; two bits
+// per vertex in shared memory instead, frontiers in vertex order, leaves as counts
+// 21.1 / 252; rows in tiers of one thread (4 entries), eight lanes (16) and whole
+// warps, atomics of one kind issued together 17.1 / 225; folding and lists in the
+// same tiers 14.9 / 222 (0 / 1 / 2 / 3 passes: 18.9 / 16.6 / 15.5 / 14.9 and
+// 232 / 221 / 222 / 225).  64 landmarks against 8 / 16 / 32: R-MAT 288 / 273 / 260 / 252.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -57,7 +77,9 @@ constexpr uint32_t SW_WARP_MAX = 2048; // longer rows and lists are the whole te
 constexpr uint32_t SW_TEAM_CAP = 64;   // rows handed to the whole team per pass (the rest stay with a warp)
 constexpr uint32_t SW_HEAD = 2;        // words before a DAG list: successors listed, successors counted
 constexpr uint32_t SW_ORDER = 64;      // frontiers above n / SW_ORDER are put into vertex order
-constexpr uint32_t SW_DEEP = 256;      // ... and levels, where the distances took fewer rounds than this
+constexpr uint32_t SW_DEEP = 256;      // ... and levels, and vertices folded, where the distances took fewer rounds
+                                       // than this (random and scale-free graphs take 8-62, grids from 32 x 32 on 65;
+                                       // folding costs the 512 x 512 grid 10%)
 
 // Where a team's arrays are.
 enum : int {
