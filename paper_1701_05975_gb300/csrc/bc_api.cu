@@ -140,7 +140,7 @@ struct bc_graph {
   void* land_in = nullptr;      // undirected graphs: land_out
   uint64_t land_stride = 0;
   uint32_t land_bits = 0, nland = 0, land_n = 0;
-  uint32_t act_n = 0;           // vertices from this id on have no entries
+  uint32_t act_n = 0;           // vertices from this id on have no entries (active_vertices)
   uint32_t* esm = nullptr;  // edge output: walked entry -> caller's output entry (built on first use)
   int esm_state = 0;        // 0 not built, 1 ready, 2 unavailable (an entry without a twin)
   std::vector<uint32_t> h_o2n;  // host copy of old -> new
@@ -1206,10 +1206,7 @@ int bc_graph_create(const uint64_t* row_ptr, const uint32_t* col_idx, const uint
     }
     g->width_default = rows ? std::max<uint64_t>(1, (uint64_t)(sum / (double)rows + 0.5)) : 1;
   }
-  for (g->act_n = n; g->act_n > 0; --g->act_n) {
-    const uint32_t v = g->act_n - 1;
-    if (row_ptr[v + 1] > row_ptr[v] || (directed && irp[v + 1] > irp[v])) break;
-  }
+  g->act_n = active_vertices(n, row_ptr, col_idx);
   g->dist_bits = distance_bits(n, row_ptr, col_idx, w, max_w, directed);
   g->fingerprint = fingerprint(n, nnz, row_ptr, col_idx, w);
   {

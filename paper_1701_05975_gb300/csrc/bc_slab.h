@@ -21,6 +21,18 @@ constexpr uint32_t SWEEP_BITS_MAX = 212u << 10;
 
 inline uint64_t align256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
 
+// Vertices from this id on are neither a row's owner nor any entry's neighbour:
+// the sweep schedule's vertex bits cover the ids below it.  A row's neighbours
+// count as much as the row: a CSR that stores an edge in one direction only is
+// accepted, and its targets need not have rows.
+inline uint32_t active_vertices(uint32_t n, const uint64_t* row_ptr, const uint32_t* col) {
+  uint32_t last = n;
+  while (last > 0 && row_ptr[last] == row_ptr[last - 1]) --last;
+  if (last < n)
+    for (uint64_t e = 0; e < row_ptr[n]; ++e) last = std::max(last, col[e] + 1);
+  return last;
+}
+
 // What a workspace's slabs hold: the layouts and the values their arrays keep
 // between sources differ by schedule.
 enum SlabKind : int { SLAB_STRICT = 0, SLAB_SWEEP = 1, SLAB_NONE = 2 };
