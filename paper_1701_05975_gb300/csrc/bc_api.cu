@@ -1504,6 +1504,9 @@ int bc_sssp_debug(bc_graph_t g, uint32_t s, uint64_t* out_dist, double* out_sigm
   const bool sweep = config_snapshot().algorithm == BC_ALGO_DELTA;
   RunCfg r = resolve(g, 1, sweep ? BC_ALGO_DELTA : BC_ALGO_STRICT);
   plan_sweep(g, r, false);  // the arrays are read back from a slab
+  // no plan_slots here, so the kernel's shared memory limit is raised by this query alone
+  int bps = 0;
+  CK(run_occupancy(g, r, &bps));
   cudaStream_t st = g->stream;
   Workspace* w = nullptr;
   int rc = ws_acquire(g, slab_kind(r), 1, 1, st, &w);
