@@ -203,29 +203,10 @@ void ws_free(Workspace* w) {
   if (w->done) cudaEventDestroy(w->done);
 }
 
-// Settings for a run: explicit config fields win, then the graph's tuned
-// values, then heuristics.
 // Default L2 evict-last prefix (vertex ids after degree relabeling).
 #ifndef BCGPU_HOT_VERTICES
 #define BCGPU_HOT_VERTICES 32768u
 #endif
-
-struct RunCfg {
-  uint32_t team;
-  uint64_t width;
-  uint32_t settle_in;
-  uint32_t refine;  // settled-neighbour refinement of Delta_node (undirected graphs)
-  uint64_t phase_cap;
-  uint32_t max_slots;
-  double mem_fraction;
-  uint32_t mode;
-  uint32_t warp_deg;
-  uint32_t team_deg;
-  uint32_t algo;  // ALGO_STRICT or ALGO_DELTA
-  bool algo_auto; // not asked for by the configuration or the caller
-  uint32_t hot_n;
-  SweepPlan sweep;  // ALGO_DELTA
-};
 
 SlabKind slab_kind(const RunCfg& r) {
   return r.algo != ALGO_DELTA ? SLAB_STRICT : (r.sweep.mem == 2 ? SLAB_NONE : SLAB_SWEEP);
@@ -275,7 +256,8 @@ uint64_t sweep_width_default(const bc_graph* g) {
   return g->kadj ? ~0ull : sweep_bucket_width(g->max_w, g->n, g->nnz);
 }
 
-// k: sources of the run (0: not known, many).
+// Settings for a run: explicit config fields win, then the graph's tuned
+// values, then heuristics.  k: sources of the run (0: not known, many).
 RunCfg resolve(const bc_graph* g, uint32_t k, uint32_t force_algo = BC_ALGO_AUTO) {
   bc_config c = config_snapshot();
   if (force_algo) c.algorithm = force_algo;
@@ -961,12 +943,12 @@ int bcgpu::serve_plan(bc_graph* g, uint32_t k, uint64_t budget, ServePlan* out) 
   if (r.algo == ALGO_DELTA && r.algo_auto &&
       make_layout(g->n, g->dist_bits, slab_kind(r)).stride + out->fixed_bytes > budget)
     r = resolve(g, k, BC_ALGO_STRICT);
-  out->algorithm = r.algo == ALGO_DELTA ? BC_ALGO_DELTA : BC_ALGO_STRICT;
+  r.mode = BC_MODE_BATCHED;
+  out->run = r;
   int bps = 0;
   cudaError_t e = run_occupancy(g, r, &bps);
   if (e != cudaSuccess) return cuda_fail(e, "occupancy");
   const uint32_t per_block = (uint32_t)(batched_block_threads((int)r.team) / (int)r.team);
-  out->team = r.team;
   out->max_slots = (uint32_t)std::max(bps, 1) * (uint32_t)g->sm_count * per_block;
   out->slot_bytes = make_layout(g->n, g->dist_bits, slab_kind(r)).stride;
   return BC_OK;
@@ -976,8 +958,8 @@ int bcgpu::serve_open(bc_graph* g, const ServePlan& plan, const uint32_t* source
                       cudaStream_t st, ServeLease** out) {
   Workspace* w = nullptr;
   const uint32_t cap = std::max<uint32_t>(slot_cap, 1);
-  RunCfg r = resolve(g, k, plan.algorithm);
-  r.mode = BC_MODE_BATCHED;
+  // the settings that were planned (and whose kernel was prepared), whatever the configuration says by now
+  const RunCfg& r = plan.run;
   int rc = ws_acquire(g, slab_kind(r), cap, k, st, &w);
   if (rc) return rc;
   cudaError_t e = cudaSuccess;

@@ -188,6 +188,24 @@ cudaError_t sweep64_full1_bits(const SweepPlan& p, const BatchArgs* a, int grid,
 cudaError_t sweep64_full8_bits(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
 cudaError_t sweep64_full1_all(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
 
+// Settings of one batched run.
+struct RunCfg {
+  uint32_t team;
+  uint64_t width;
+  uint32_t settle_in;
+  uint32_t refine;  // settled-neighbour refinement of Delta_node (undirected graphs)
+  uint64_t phase_cap;
+  uint32_t max_slots;
+  double mem_fraction;
+  uint32_t mode;
+  uint32_t warp_deg;
+  uint32_t team_deg;
+  uint32_t algo;  // ALGO_STRICT or ALGO_DELTA
+  bool algo_auto; // not asked for by the configuration or the caller
+  uint32_t hot_n;
+  SweepPlan sweep;  // ALGO_DELTA
+};
+
 // Landmark preparation (bc_land.cu); g.adj holds the rows walked.
 cudaError_t land_symmetry(const GraphDev& g, unsigned long long* out, cudaStream_t st);
 cudaError_t land_judge(const GraphDev& g, const uint32_t* from_h, const uint32_t* probe, uint32_t h,
@@ -250,8 +268,7 @@ namespace bcgpu {
 // workspace.
 struct ServeLease;
 struct ServePlan {
-  uint32_t algorithm;   // BC_ALGO_STRICT or BC_ALGO_DELTA: the lease's slabs belong to it
-  uint32_t team;        // threads per source
+  RunCfg run;           // settings at admission: the lease's slabs and kernel belong to them
   uint32_t max_slots;   // sources the GPU holds at once for this team size
   uint64_t slot_bytes;  // device bytes per source in flight
   uint64_t fixed_bytes; // per-request device bytes besides the slabs

@@ -256,11 +256,11 @@ struct Server {
       }
     if (si < 0) return false;
     const ServePlan& p = r->plan;
-    const uint64_t share = std::max<uint64_t>(thread_cap / std::max<uint64_t>(1, sharers), p.team);
+    const uint64_t share = std::max<uint64_t>(thread_cap / std::max<uint64_t>(1, sharers), p.run.team);
     const uint64_t free_threads = thread_cap > threads_used ? thread_cap - threads_used : 0;
     const uint32_t left = (uint32_t)(r->sources.size() - r->next);
     const uint64_t slots = std::min<uint64_t>({(uint64_t)serve_slot_cap(r->lease), (uint64_t)std::max(left, 1u),
-                                               std::min(share, free_threads) / p.team});
+                                               std::min(share, free_threads) / p.run.team});
     if (slots == 0) return false;
     const uint32_t count = (uint32_t)std::min<uint64_t>(left, slots * BCGPU_SERVE_WAVES);
     const bool last = r->next + count >= r->sources.size();
@@ -272,7 +272,7 @@ struct Server {
     r->next += count;
     r->batch_entries = (uint64_t)count * std::max<uint64_t>(graph_nnz(r->g), 1);
     r->in_batch = true;
-    r->threads = slots * p.team;
+    r->threads = slots * p.run.team;
     threads_used += r->threads;
     r->stream_idx = si;
     stream_busy[si] = true;

@@ -45,3 +45,36 @@ with bc.Graph(g) as G:
 want = oracle.sssp(g, 77)
 assert np.array_equal(d, want[0]) and np.array_equal(sig, want[1])
 """)
+
+
+def test_settings_may_change_while_requests_are_admitted():
+    """The configuration flips between teams and schedules while the server admits
+    requests: each runs with the settings it was planned with, none is refused."""
+    fresh_process("""
+import threading
+graphs = [gen.ba_graph(1500, 5, 1, 100, seed=1), gen.grid_graph(470, 470, wmin=1, wmax=9, seed=2)]
+src = [np.arange(0, g.n, g.n // 40, dtype=np.uint32) for g in graphs]
+want = [oracle.bc(g, s, 0.5, nthreads=8) for g, s in zip(graphs, src)]
+stop = threading.Event()
+def flip():
+    while not stop.is_set():
+        for team in (32, 128, 256, 512, 1024):
+            for algo in (bc.BC_ALGO_DELTA, bc.BC_ALGO_STRICT):
+                bc.bc_set_config(team_threads=team, algorithm=algo)
+t = threading.Thread(target=flip)
+handles = [bc.Graph(g) for g in graphs]
+t.start()
+try:
+    for _ in range(30):
+        reqs = [(i, handles[i].submit(src[i], 0.5)) for i in (0, 1, 0, 0, 1, 0)]
+        for i, r in reqs:
+            got = r.result(60000)
+            assert np.array_equal(got == 0, want[i] == 0)
+            nz = want[i] != 0
+            assert np.all(np.abs(got[nz] - want[i][nz]) <= 1e-9 * want[i][nz])
+finally:
+    stop.set()
+    t.join()
+for h in handles:
+    h.close()
+""")
