@@ -417,6 +417,26 @@ void ws_release(bc_graph* g, Workspace* w, cudaStream_t st) {
   w->busy = false;
 }
 
+// Free the pool's idle workspaces but the smallest one with at least `slots` slabs of `kind`.
+void ws_trim(bc_graph* g, SlabKind kind, uint32_t slots) {
+  std::vector<std::unique_ptr<Workspace>> drop;
+  {
+    std::lock_guard<std::mutex> lk(g->mu);
+    const Workspace* keep = nullptr;
+    for (auto& p : g->pool)
+      if (!p->busy && p->kind == kind && p->slots >= slots && (!keep || p->slots < keep->slots)) keep = p.get();
+    for (size_t i = g->pool.size(); i-- > 0;)
+      if (!g->pool[i]->busy && g->pool[i].get() != keep) {
+        drop.push_back(std::move(g->pool[i]));
+        g->pool.erase(g->pool.begin() + i);
+      }
+  }
+  for (auto& w : drop) {
+    cudaEventSynchronize(w->done);  // its last run may still be in flight on a caller's stream
+    ws_free(w.get());
+  }
+}
+
 // Edge output over the DAG edge list needs, for every entry the forward pass
 // walks (out-entries of an undirected graph, in-entries of a directed one),
 // the caller's index of the entry that carries its share: the twin u -> v of
@@ -1589,10 +1609,12 @@ int bc_last_run_stats(bc_graph_t g, bc_run_stats* out) {
   return BC_OK;
 }
 
-int bc_autotune(bc_graph_t g, const uint32_t* sources, uint32_t k_probe) {
-  if (int rc = check_graph(g)) return rc;
-  if (!sources || k_probe == 0) return fail(BC_ERR_INVALID, "autotune needs probe sources");
-  CK(cudaSetDevice(g->device));
+}  // extern "C"
+
+namespace {
+
+// Times the candidates and stores the fastest as the graph's tuned settings.
+int autotune(bc_graph* g, const uint32_t* sources, uint32_t k_probe) {
   bc_config user = config_snapshot();
   // candidates: team size x near/far split width, then sources in flight
   std::vector<uint32_t> teams = {128, 256, 512};
@@ -1759,6 +1781,24 @@ int bc_autotune(bc_graph_t g, const uint32_t* sources, uint32_t k_probe) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   g_tune_cache[g->fingerprint] = best;
   return BC_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int bc_autotune(bc_graph_t g, const uint32_t* sources, uint32_t k_probe) {
+  if (int rc = check_graph(g)) return rc;
+  if (!sources || k_probe == 0) return fail(BC_ERR_INVALID, "autotune needs probe sources");
+  CK(cudaSetDevice(g->device));
+  const int rc = autotune(g, sources, k_probe);
+  // the candidates' workspaces (teams of 128 threads have eight times the slabs of 1024; strict and
+  // sweep slabs do not serve each other) go, but one that the next run takes
+  RunCfg r = resolve(g, k_probe);
+  uint32_t slots = 0;
+  if (rc || plan_slots(g, r, k_probe, &slots)) slots = 0xffffffffu;
+  ws_trim(g, slab_kind(r), slots);
+  return rc;
 }
 
 // ---- step graphs --------------------------------------------------------

@@ -78,3 +78,27 @@ finally:
 for h in handles:
     h.close()
 """)
+
+
+def test_autotune_gives_the_other_candidates_workspaces_back():
+    """Both schedules are timed at up to 1216 slabs; afterwards one workspace is left, not one per candidate."""
+    torch = pytest.importorskip("torch")
+    g = gen.ba_graph(30000, 4, 1, 1000, seed=41)
+    src = np.arange(0, g.n, 12, dtype=np.uint32)
+    with bc.Graph(g) as G:
+        slab = G.info().slab_bytes
+        most = 1216 * slab + (64 << 20)  # the largest workspace of one candidate
+        free0 = torch.cuda.mem_get_info()[0]
+        assert free0 > 4 * most  # no candidate is short of memory
+        G.autotune(src)
+        assert free0 - torch.cuda.mem_get_info()[0] <= most
+        assert_bc_close(G.compute(src, 0.5), oracle.bc(g, src, 0.5, nthreads=8))
+        assert free0 - torch.cuda.mem_get_info()[0] <= most
+        # a workspace whose run has not been read yet is nobody's to free
+        s = torch.cuda.Stream()
+        d_src, out = torch.from_numpy(src.astype(np.int32)).cuda(), torch.empty(g.n, dtype=torch.float64, device="cuda")
+        s.wait_stream(torch.cuda.current_stream())
+        G.compute_async(d_src, out, 0.5, stream=s)
+        G.autotune(src[:64])
+        G.sync(s)
+        assert_bc_close(out.cpu().numpy(), oracle.bc(g, src, 0.5, nthreads=8))
