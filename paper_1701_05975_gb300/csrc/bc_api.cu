@@ -1210,12 +1210,6 @@ int bc_graph_create(const uint64_t* row_ptr, const uint32_t* col_idx, const uint
   }
   g->act_n = active_vertices(n, row_ptr, col_idx);
   g->dist_bits = distance_bits(n, row_ptr, col_idx, w, max_w, directed);
-  g->fingerprint = fingerprint(n, nnz, row_ptr, col_idx, w);
-  {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tune_cache.find(g->fingerprint);
-    if (it != g_tune_cache.end()) g->tuned = it->second;
-  }
   uint32_t* d_col = nullptr;
   uint32_t* d_w = nullptr;
   cudaError_t e = cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking);
@@ -1307,6 +1301,14 @@ int bc_graph_create(const uint64_t* row_ptr, const uint32_t* col_idx, const uint
                     (packed && g->adj ? 8ull * nnz : 0) +
                     (g->kadj ? (g->kw ? 16ull : 12ull) * nnz +
                                    g->land_stride * g->nland * (g->land_bits / 8) * (directed ? 2 : 1) : 0);
+  // tuned settings mean something for the same direction and row order only
+  g->fingerprint = fingerprint(n, nnz, row_ptr, col_idx, w) + (directed ? "-directed" : "") +
+                   (g->kadj ? "-landmarks" : "");
+  {
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    auto it = g_tune_cache.find(g->fingerprint);
+    if (it != g_tune_cache.end()) g->tuned = it->second;
+  }
   *out = g.release();
   return BC_OK;
 }

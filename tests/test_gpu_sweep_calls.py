@@ -102,3 +102,28 @@ def test_autotune_gives_the_other_candidates_workspaces_back():
         G.autotune(src[:64])
         G.sync(s)
         assert_bc_close(out.cpu().numpy(), oracle.bc(g, src, 0.5, nthreads=8))
+
+
+def test_tuned_settings_stay_with_the_row_order_they_were_timed_on():
+    """The same CSR with and without landmarks (in its own order, past 32,768 vertices, it gets none):
+    one unlimited bucket, right under landmark bounds, is not inherited by the other."""
+    g0 = gen.ba_graph(33000, 4, 1, 1000, seed=43)
+    u, v, w = (np.asarray(x) for x in g0.edges())
+    deg = np.bincount(u, minlength=g0.n) + np.bincount(v, minlength=g0.n)
+    new = np.empty(g0.n, np.int64)
+    new[np.argsort(-deg, kind="stable")] = np.arange(g0.n)
+    once = u < v
+    g = gen.csr_from_undirected(g0.n, new[u[once]], new[v[once]], w[once])  # numbered by decreasing degree already
+    src = np.arange(0, g.n, 330, dtype=np.uint32)
+    unlimited = (1 << 64) - 1
+    with bc.Graph(g) as A, bc.Graph(g, flags=bc.BC_KEEP_ORDER) as B:
+        for G in (A, B):
+            G.compute(src, 0.5)
+        assert A.stats().bucket_width == unlimited and B.stats().bucket_width < unlimited
+        A.autotune(src)
+        A.compute(src, 0.5)
+        with bc.Graph(g) as C, bc.Graph(g, flags=bc.BC_KEEP_ORDER) as D:
+            for G in (C, D):
+                G.compute(src, 0.5)
+            assert C.stats().bucket_width == A.stats().bucket_width  # the same graph again: tuned
+            assert D.stats().bucket_width == B.stats().bucket_width
