@@ -155,7 +155,8 @@ typedef struct bc_graph_info {
   uint32_t max_weight;
   uint32_t dist_bits;     /* 32 or 64: device distance width chosen for this graph */
   uint64_t device_bytes;  /* resident CSR + per-vertex graph data */
-  uint64_t slab_bytes;    /* device bytes one in-flight source needs */
+  uint64_t slab_bytes;    /* bytes one in-flight source needs: device memory, or shared memory where the
+                             sweep schedule keeps a whole source there (up to 1536 vertices) */
   uint32_t relabeled;     /* 1 when vertices are stored internally in decreasing-degree order */
   uint32_t directed;      /* 1 for a BC_DIRECTED graph */
 } bc_graph_info;

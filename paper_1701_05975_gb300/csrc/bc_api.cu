@@ -1355,7 +1355,8 @@ int bc_graph_get_info(bc_graph_t g, bc_graph_info* out) {
   out->max_weight = g->max_w;
   out->dist_bits = (uint32_t)g->dist_bits;
   out->device_bytes = g->device_bytes;
-  out->slab_bytes = make_layout(g->n, g->dist_bits, slab_kind(resolve(g, 0))).stride;
+  const SlabLayout lay = make_layout(g->n, g->dist_bits, slab_kind(resolve(g, 0)));
+  out->slab_bytes = lay.smem ? lay.smem : lay.stride;
   out->relabeled = g->relabeled ? 1u : 0u;
   out->directed = g->directed ? 1u : 0u;
   return BC_OK;

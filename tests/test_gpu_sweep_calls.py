@@ -127,3 +127,11 @@ def test_tuned_settings_stay_with_the_row_order_they_were_timed_on():
                 G.compute(src, 0.5)
             assert C.stats().bucket_width == A.stats().bucket_width  # the same graph again: tuned
             assert D.stats().bucket_width == B.stats().bucket_width
+
+
+@pytest.mark.parametrize("n", [1, 300, 1536, 1537, 5000])
+def test_slab_bytes_hold_a_source(n):
+    """Distances (4), records (16), list offsets (4) and queues of every vertex, in either kind of memory."""
+    g = gen.er_graph(n, 4 * n, 1, 50, seed=n) if n > 1 else gen.csr_from_undirected(1, [], [], [])
+    with bc.Graph(g) as G:
+        assert 24 * n <= G.info().slab_bytes <= 120 * n + 16384
