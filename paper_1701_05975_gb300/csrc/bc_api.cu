@@ -900,24 +900,24 @@ cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<u
   }
   if (e == cudaSuccess && !g->directed) e = land_symmetry(fwd, sums, st);
   if (e == cudaSuccess) e = land_judge(fwd, tab, tab + (uint64_t)L * n, h, probes, sums + 2, st);
-  if (e == cudaSuccess) e = land_max((uint64_t)L * n, tab, reinterpret_cast<uint32_t*>(sums + 6), st);
+  if (e == cudaSuccess) e = land_max((uint64_t)L * n, tab, reinterpret_cast<uint32_t*>(sums + 5), st);
   if (e == cudaSuccess && g->directed)
-    e = land_max((uint64_t)L * n, tab_in, reinterpret_cast<uint32_t*>(sums + 6), st);
+    e = land_max((uint64_t)L * n, tab_in, reinterpret_cast<uint32_t*>(sums + 5), st);
   std::vector<unsigned char> host(2 * sizeof(Ctl) + 8 * 8);
   if (e == cudaSuccess) e = cudaMemcpyAsync(host.data(), ctl, host.size(), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return done(e);
-  unsigned long long hs[7];
+  unsigned long long hs[6];
   memcpy(hs, host.data() + 2 * sizeof(Ctl), sizeof hs);
   const Ctl* hc = reinterpret_cast<const Ctl*>(host.data());
-  const uint32_t max_d = (uint32_t)hs[6];
+  const uint32_t max_d = (uint32_t)hs[5];
   if (hc[0].err != DEV_OK || hc[1].err != DEV_OK || hs[0] != hs[1]) return done(cudaSuccess);
   if (hs[2] == 0 || (double)hs[3] > LAND_KEEP_MAX * (double)hs[2]) return done(cudaSuccess);
 
   g->land_bits = max_d < 0x3fffu ? 16 : 32;  // every sum of two distances below 0x7fff
   g->land_stride = ((uint64_t)n + 7) & ~7ull;
   g->nland = L;
-  g->land_n = g->directed ? g->act_n : (uint32_t)hs[5];
+  g->land_n = g->directed ? g->act_n : (uint32_t)hs[4];
   const uint64_t tab_bytes = g->land_stride * L * (g->land_bits / 8);
   unsigned long long* key = static_cast<unsigned long long*>(alloc(g->nnz * 8));
   if (!key) return done(cudaErrorMemoryAllocation);
@@ -931,7 +931,7 @@ cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<u
   if (e == cudaSuccess && g->directed)
     e = land_pack(n, g->land_stride, L, tab_in, (int)g->land_bits, g->land_in, st);
   if (e == cudaSuccess)
-    e = land_rows(fwd, tab, key, g->adjp ? g->col_bits : 0u, g->kadj, g->kw, g->k2o, st);
+    e = land_rows(fwd, rp, tab, key, g->adjp ? g->col_bits : 0u, g->kadj, g->kw, g->k2o, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   return done(e);
 }

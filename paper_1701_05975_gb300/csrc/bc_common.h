@@ -213,8 +213,8 @@ cudaError_t land_judge(const GraphDev& g, const uint32_t* from_h, const uint32_t
 cudaError_t land_max(uint64_t count, const uint32_t* tab, uint32_t* out, cudaStream_t st);
 cudaError_t land_pack(uint32_t n, uint64_t stride, uint32_t rows, const uint32_t* tab, int bits, void* out,
                       cudaStream_t st);
-cudaError_t land_rows(const GraphDev& g, const uint32_t* from_h, unsigned long long* key, uint32_t col_bits,
-                      uint2* kadj, uint32_t* kw, uint32_t* k2o, cudaStream_t st);
+cudaError_t land_rows(const GraphDev& g, const uint64_t* host_row_ptr, const uint32_t* from_h, unsigned long long* key,
+                      uint32_t col_bits, uint2* kadj, uint32_t* kw, uint32_t* k2o, cudaStream_t st);
 
 // Graph preparation and small helpers (bc_prep.cu).
 // dnode2 / dnode_arg may be nullptr (not computed).

@@ -135,3 +135,21 @@ def test_slab_bytes_hold_a_source(n):
     g = gen.er_graph(n, 4 * n, 1, 50, seed=n) if n > 1 else gen.csr_from_undirected(1, [], [], [])
     with bc.Graph(g) as G:
         assert 24 * n <= G.info().slab_bytes <= 120 * n + 16384
+
+
+@pytest.mark.parametrize("spokes", [32768, 32769, 65537, 100001])
+def test_hub_rows_are_in_landmark_order(spokes):
+    """A hub's row at and past the length that is sorted by the whole GPU: spokes closer
+    to the hub by another way than by their own edge give the row many different keys."""
+    rng = np.random.default_rng(spokes)
+    u = np.concatenate([np.zeros(spokes, np.int64), rng.integers(1, spokes + 1, 2 * spokes)])
+    v = np.concatenate([np.arange(1, spokes + 1), rng.integers(1, spokes + 1, 2 * spokes)])
+    w = np.concatenate([rng.integers(1, 4001, spokes), rng.integers(1, 401, 2 * spokes)])
+    key = np.unique(np.minimum(u, v) * (spokes + 1) + np.maximum(u, v), return_index=True)[1]
+    key = key[u[key] != v[key]]
+    g = gen.csr_from_undirected(spokes + 1, u[key], v[key], w[key])
+    src = np.concatenate([[0], rng.integers(1, spokes + 1, 11)]).astype(np.uint32)
+    with bc.Graph(g) as G:
+        assert_bc_close(G.compute(src, 0.5), oracle.bc(g, src, 0.5, nthreads=8))
+        assert G.stats().bucket_width == (1 << 64) - 1  # landmarks are in use
+        assert G.stats().entries_scanned < 1.5 * g.nnz * len(src)
