@@ -212,24 +212,41 @@ SlabKind slab_kind(const RunCfg& r) {
   return r.algo != ALGO_DELTA ? SLAB_STRICT : (r.sweep.mem == 2 ? SLAB_NONE : SLAB_SWEEP);
 }
 
+// Sparse graphs without landmarks: small frontiers in many rounds.
+bool sweep_sparse(const bc_graph* g) { return !g->kadj && (double)g->nnz < 6.0 * g->n; }
+
+// Whether a run of k sources (0: many) keeps its sources in shared memory.  Sparse
+// graphs want many teams in flight: where fewer than four of 256 threads fit an SM
+// (above 1150 vertices) and the sources are more than four an SM, slabs hold more
+// (us in shared memory and slabs: 38 x 38 grid 769 / 766 at 608 sources, 821 / 781 at
+// 900, 1080 / 833 at 1216; Barabasi-Albert 1500 with 2 edges a vertex 667 / 471 at
+// 1216; 30 x 30 grid 650 / 690 at 900).
+bool sweep_in_smem(const bc_graph* g, uint32_t k) {
+  if (g->n > SWEEP_SMEM_N) return false;
+  if (!sweep_sparse(g) || g->dist_bits != 32) return true;
+  if (k && k <= 4ull * g->sm_count) return true;
+  return sweep_teams_per_sm(32, 256, make_layout(g->n, 32, SLAB_NONE).smem) >= 4;
+}
+
 // Kernel variant of the sweep schedule for `team` threads per source.
-void plan_sweep(const bc_graph* g, RunCfg& r, bool allow_smem) {
+void plan_sweep(const bc_graph* g, RunCfg& r, uint32_t k, bool allow_smem) {
   SweepPlan p;
   p.dist_bits = g->dist_bits;
   p.team = (int)r.team;
   p.prune = g->kadj != nullptr;
   const double avg_deg = g->n ? (double)g->nnz / g->n : 0.0;
   p.group = (!p.prune && avg_deg >= 12.0) ? 8 : 1;
-  sweep_place(p, g->n, g->act_n, allow_smem);
+  sweep_place(p, g->n, g->act_n, allow_smem && sweep_in_smem(g, k));
   r.sweep = p;
 }
 
 // Threads per source of the sweep schedule for a run of k sources (0: many).
-// Teams of T threads run 1024 / T to an SM.  Sparse graphs without landmarks
-// have small frontiers in many rounds, so latency counts: the widest team that
-// still has every source in flight at once, 128 where none has (1024 sources of
+// Sparse graphs without landmarks: latency counts, so the widest team that still
+// has every source in flight at once, 128 where none has (1024 sources of
 // a 256 x 256 grid: 12.4 ms at 128 threads, 17.1 at 256; 512 sources of a 512 x
-// 512 one: 44.0 and 32.6).  The others by size, the frontiers growing with it
+// 512 one: 44.0 and 32.6; 64-bit words hold three teams of 256 to an SM, not four: 500
+// sources of a 200 x 200 grid 6.8 ms at 128, 9.4 at 256).  The others by size, the
+// frontiers growing with it
 // (BA 4096 2.06 / 2.40 / 3.39 ms at 128 / 256 / 512, BA 16k 15.4 / 14.8 / 15.6,
 // BA 65k 17.0 / 16.3 / 14.9, Erdos-Renyi 65k 47.5 / 36.2 / 28.9 and 25.3 at 1024,
 // R-MAT scale 20 359 / 305 / 270 / 222 at 128 / 256 / 512 / 1024), doubled while
@@ -237,8 +254,11 @@ void plan_sweep(const bc_graph* g, RunCfg& r, bool allow_smem) {
 uint32_t sweep_team_default(const bc_graph* g, uint32_t k) {
   const double avg_deg = g->n ? (double)g->nnz / g->n : 0.0;
   const uint32_t wide = g->dist_bits == 32 ? 1024u : 512u;
-  auto in_flight = [&](uint32_t team) { return (uint64_t)g->sm_count * (1024 / team); };
-  if (!g->kadj && avg_deg < 6.0) {
+  // in shared memory a second wave costs less than a narrower team (38 x 38 grid with 64-bit
+  // words, 500 sources: 708 us at 256 threads, 740 at 128), so what fits there is not counted
+  const int bits = sweep_in_smem(g, k) ? 32 : g->dist_bits;
+  auto in_flight = [&](uint32_t team) { return (uint64_t)g->sm_count * sweep_teams_per_sm(bits, team, 0); };
+  if (sweep_sparse(g)) {
     // 64-bit words spill at 512 threads (200 x 200 grid, 304 sources: 5.6 ms at 256, 5.9 at 512)
     if (k && g->dist_bits == 32 && in_flight(512) >= k) return 512u;
     return k && in_flight(256) >= k ? 256u : 128u;
@@ -305,7 +325,7 @@ RunCfg resolve(const bc_graph* g, uint32_t k, uint32_t force_algo = BC_ALGO_AUTO
   r.team_deg = std::max(r.team_deg, r.warp_deg);
   const uint32_t hot = c.hot_vertices ? c.hot_vertices : BCGPU_HOT_VERTICES;
   r.hot_n = g->relabeled ? std::min<uint32_t>(g->n, hot) : 0u;
-  plan_sweep(g, r, true);
+  plan_sweep(g, r, k, true);
   return r;
 }
 
@@ -845,8 +865,8 @@ cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<u
   r.team = n >= 16384 ? 1024u : 256u;
   r.width = sweep_width_default(g);
   r.phase_cap = 4ull * n + 64;
-  plan_sweep(g, r, true);
   const uint32_t k = (uint32_t)ids.size();
+  plan_sweep(g, r, k, true);
   int bps = 0;
   cudaError_t e = run_occupancy(g, r, &bps);
   if (e != cudaSuccess) return e;
@@ -1508,7 +1528,7 @@ int bc_sssp_debug(bc_graph_t g, uint32_t s, uint64_t* out_dist, double* out_sigm
   // the strict schedule's levels unless the sweep schedule is asked for by name
   const bool sweep = config_snapshot().algorithm == BC_ALGO_DELTA;
   RunCfg r = resolve(g, 1, sweep ? BC_ALGO_DELTA : BC_ALGO_STRICT);
-  plan_sweep(g, r, false);  // the arrays are read back from a slab
+  plan_sweep(g, r, 1, false);  // the arrays are read back from a slab
   // no plan_slots here, so the kernel's shared memory limit is raised by this query alone
   int bps = 0;
   CK(run_occupancy(g, r, &bps));
@@ -1662,7 +1682,7 @@ int autotune(bc_graph* g, const uint32_t* sources, uint32_t k_probe) {
         RunCfg r = base;
         r.team = team;
         r.width = width;
-        plan_sweep(g, r, true);
+        plan_sweep(g, r, k_probe, true);
         if (int rc = timed(r, &ms)) return rc;
         if (ms < sweep_ms) {
           sweep_ms = ms;
@@ -1677,7 +1697,7 @@ int autotune(bc_graph* g, const uint32_t* sources, uint32_t k_probe) {
       RunCfg r = base;
       r.team = best.sweep_team;
       r.width = best.sweep_width;
-      plan_sweep(g, r, true);
+      plan_sweep(g, r, k_probe, true);
       uint32_t full = 0;
       if (int rc = plan_slots(g, r, k_probe, &full)) return rc;
       r.max_slots = std::max<uint32_t>(1, full / 2);

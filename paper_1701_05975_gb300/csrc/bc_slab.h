@@ -113,6 +113,15 @@ inline cudaError_t init_slabs(char* slabs, const SlabLayout& lay, SlabKind kind,
   return launch_fill_slabs(slabs, lay.stride, slots, lay.off_acc, align256((uint64_t)n * 8), 0u, st);
 }
 
+// Teams of `team` threads that an SM holds: by the registers the kernels are
+// compiled for (64 a thread; 64-bit distance words leave room for 7/8 of them up
+// to 256 threads), and by the bytes of shared memory a team keeps its source in
+// (0: in a slab), 3 KB more for its own state and the system's share.
+inline uint32_t sweep_teams_per_sm(int dist_bits, uint32_t team, uint32_t smem) {
+  const uint32_t by_regs = (dist_bits == 64 && team <= 256 ? 896u : 1024u) / team;
+  return smem ? std::min<uint32_t>(by_regs, (228u << 10) / (smem + 3072u)) : by_regs;
+}
+
 // Memory form of a sweep plan whose distance width and team are set: n
 // vertices, the ones from act_n on without entries.
 inline void sweep_place(SweepPlan& p, uint32_t n, uint32_t act_n, bool allow_smem) {

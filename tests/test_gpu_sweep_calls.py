@@ -153,3 +153,14 @@ def test_hub_rows_are_in_landmark_order(spokes):
         assert_bc_close(G.compute(src, 0.5), oracle.bc(g, src, 0.5, nthreads=8))
         assert G.stats().bucket_width == (1 << 64) - 1  # landmarks are in use
         assert G.stats().entries_scanned < 1.5 * g.nnz * len(src)
+
+
+@pytest.mark.parametrize("side,wmax,k", [(200, 1 << 24, 456), (200, 1 << 24, 457), (38, 50, 609), (38, 50, 1216)])
+def test_sparse_graphs_have_their_sources_in_flight(side, wmax, k):
+    """The team rule counts the teams an SM really holds: seven eighths with 64-bit words, few in shared memory."""
+    g = gen.grid_graph(side, side, wmin=1, wmax=wmax, seed=3)
+    src = np.arange(k, dtype=np.uint32)
+    with bc.Graph(g) as G:
+        assert_bc_close(G.compute(src, 0.5), oracle.bc(g, src, 0.5, nthreads=8))
+        assert G.stats().algorithm == bc.BC_ALGO_DELTA
+        assert G.stats().slots == k

@@ -63,3 +63,14 @@ def test_vertex_bits_cover_every_neighbour(tmp_path):
     std::cout << active_vertices(n, rp.data(), col.data()) << "\\n";
   }""", "\n".join(text))
     assert [int(x) for x in got] == want
+
+
+def test_teams_per_sm_by_registers_and_shared_memory(tmp_path):
+    """32-bit words: 1024 threads; 64-bit ones 7/8 of that up to 256 a team; and what shared memory holds."""
+    got = run_cpp(tmp_path, """
+  for (uint32_t t : {128u, 256u, 512u, 1024u})
+    std::cout << sweep_teams_per_sm(32, t, 0) << " " << sweep_teams_per_sm(64, t, 0) << " ";
+  for (uint32_t n : {300u, 1024u, 1536u})
+    std::cout << sweep_teams_per_sm(32, 256, make_layout(n, 32, SLAB_NONE).smem) << " "
+              << sweep_teams_per_sm(32, 128, make_layout(n, 32, SLAB_NONE).smem) << " ";""")
+    assert [int(x) for x in got] == [8, 7, 4, 3, 2, 2, 1, 1, 4, 8, 4, 4, 3, 3]
