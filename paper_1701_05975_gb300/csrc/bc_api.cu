@@ -215,16 +215,24 @@ SlabKind slab_kind(const RunCfg& r) {
 // Sparse graphs without landmarks: small frontiers in many rounds.
 bool sweep_sparse(const bc_graph* g) { return !g->kadj && (double)g->nnz < 6.0 * g->n; }
 
-// Whether a run of k sources (0: many) keeps its sources in shared memory.  Sparse
-// graphs want many teams in flight: where fewer than four of 256 threads fit an SM
-// (above 1150 vertices) and the sources are more than four an SM, slabs hold more
-// (us in shared memory and slabs: 38 x 38 grid 769 / 766 at 608 sources, 821 / 781 at
-// 900, 1080 / 833 at 1216; Barabasi-Albert 1500 with 2 edges a vertex 667 / 471 at
-// 1216; 30 x 30 grid 650 / 690 at 900).
+// Whether a run of k sources (0: many) keeps its sources in shared memory.
+// Rows of 24 entries and more without landmark order are walked by eight threads each,
+// which the shared-memory form has not: it gives every row to a warp, the DAG build two
+// times over.  Shared memory and slabs, us: Erdos-Renyi of degree 32 with weights to 4,
+// all sources, n = 1024 1708 and 734, n = 1536 (1216 sources) 3420 and 1055; 40 sources
+// 654 and 321, 943 and 436.  At degree 16, weights to 8, shared memory is level or ahead:
+// n = 1024 534 and 640, n = 1536 896 and 860; 40 sources 226 and 288, 275 and 361.  Below
+// 400 vertices it is ahead on R-MAT (n = 256 201 and 214).
+// Sparse graphs want many teams in flight: where fewer than four of 256 threads fit an
+// SM (above 1150 vertices), slabs hold more for four to eight sources an SM (38 x 38
+// grid 769 and 766 at 608 sources, 821 and 781 at 900, 1080 and 833 at 1216, and 1042 and 1162
+// in a second wave of slabs at 1296; Barabasi-Albert 1500 with 2 edges a vertex 667 and 471
+// at 1216; 30 x 30 grid 650 and 690 at 900).
 bool sweep_in_smem(const bc_graph* g, uint32_t k) {
   if (g->n > SWEEP_SMEM_N) return false;
+  if (!g->kadj && g->n >= 400 && g->nnz >= 24ull * g->n) return false;
   if (!sweep_sparse(g) || g->dist_bits != 32) return true;
-  if (k && k <= 4ull * g->sm_count) return true;
+  if (k <= 4ull * g->sm_count || k > 8ull * g->sm_count) return true;
   return sweep_teams_per_sm(32, 256, make_layout(g->n, 32, SLAB_NONE).smem) >= 4;
 }
 
@@ -819,7 +827,15 @@ void free_landmarks(bc_graph* g) {
 // 3%, Barabasi-Albert 65k 21%).  Undirected graphs must be symmetric for the
 // triangle inequality to hold in both directions.  Running out of device
 // memory here only means no landmarks.
+//
+// Without hubs the bounds are looser (more vertices beat them), and rows of 24 and more
+// entries are walked by eight threads each without landmarks, by one with them: such
+// graphs keep plain rows from 35% on.  Erdos-Renyi of degree 32, 1216 sources, ms
+// with landmarks and without: n = 13,000 weights to 16 (45% kept) 11.1 and 7.6, to 32
+// (42%) 8.9 and 7.6, to 64 (26%) 6.1 and 7.6; n = 4096 to 16 (33%) 2.5 and 2.4,
+// to 64 (28%) 1.9 and 2.5.  Graphs that run in shared memory gain from 50% on.
 constexpr double LAND_KEEP_MAX = 0.5;
+constexpr double LAND_KEEP_MAX_DENSE = 0.35;
 constexpr uint32_t LAND_PROBES = 4;
 constexpr uint32_t LAND_MIN_N = 256;
 constexpr uint32_t LAND_MAX_N_FLAT = 32768;
@@ -932,7 +948,9 @@ cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<u
   const Ctl* hc = reinterpret_cast<const Ctl*>(host.data());
   const uint32_t max_d = (uint32_t)hs[5];
   if (hc[0].err != DEV_OK || hc[1].err != DEV_OK || hs[0] != hs[1]) return done(cudaSuccess);
-  if (hs[2] == 0 || (double)hs[3] > LAND_KEEP_MAX * (double)hs[2]) return done(cudaSuccess);
+  const bool dense = !g->relabeled && n > SWEEP_SMEM_N && g->nnz >= 24ull * n;
+  const double keep_max = dense ? LAND_KEEP_MAX_DENSE : LAND_KEEP_MAX;
+  if (hs[2] == 0 || (double)hs[3] > keep_max * (double)hs[2]) return done(cudaSuccess);
 
   g->land_bits = max_d < 0x3fffu ? 16 : 32;  // every sum of two distances below 0x7fff
   g->land_stride = ((uint64_t)n + 7) & ~7ull;

@@ -164,3 +164,24 @@ def test_sparse_graphs_have_their_sources_in_flight(side, wmax, k):
         assert_bc_close(G.compute(src, 0.5), oracle.bc(g, src, 0.5, nthreads=8))
         assert G.stats().algorithm == bc.BC_ALGO_DELTA
         assert G.stats().slots == k
+
+
+@pytest.mark.parametrize("n,m", [(399, 4800), (400, 4799), (400, 4800), (1024, 16384), (1536, 18432), (1537, 18445),
+                                 (600, 30000)])
+def test_dense_rows_without_landmarks_run_in_slabs(n, m):
+    """24 entries a row and more, weights so small that the prefix test keeps most entries."""
+    g = gen.er_graph(n, m, 1, 2, seed=m)
+    src = np.arange(0, n, 5, dtype=np.uint32)
+    want, wante = oracle.bc(g, src, 0.5, nthreads=8), oracle.edge_bc(g, src, 0.5)
+    bc.bc_set_config(algorithm=bc.BC_ALGO_DELTA)
+    with bc.Graph(g) as G:
+        G.compute(src, 0.5)
+        assert G.stats().bucket_width < (1 << 64) - 1  # no landmarks
+        in_slab = G.info().slab_bytes > 60 * n
+        assert in_slab == (n > 1536 or (n >= 400 and g.nnz >= 24 * n))
+        for team in (0, 32, 128, 512):
+            bc.bc_set_config(team_threads=team)
+            assert_bc_close(G.compute(src, 0.5), want)
+            ebc, vbc = G.edge_compute(src, 0.5)
+            assert_bc_close(ebc, wante)
+            assert_bc_close(vbc, want)
