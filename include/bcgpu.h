@@ -67,9 +67,11 @@ extern "C" {
 #define BC_MODE_PLAIN 1u   /* one source at a time over the whole GPU, host-driven phase loop */
 
 /* ---- per-source schedules of the batched mode --------------------------- */
-#define BC_ALGO_AUTO 0u   /* the graph's tuned schedule, else BC_ALGO_DELTA; BC_ALGO_STRICT while the configuration
-                             sets a knob that only that schedule has (settle_in, bucket_width, warp_degree,
-                             team_degree, hot_vertices) */
+#define BC_ALGO_AUTO 0u   /* the graph's tuned schedule, else BC_ALGO_DELTA, but BC_ALGO_STRICT where its batches are
+                             few (vertex BC of graphs with small weights and many tied paths, by the
+                             shortest-path DAGs of a few probe sources and the number of sources), and while
+                             the configuration sets a knob that only that schedule has (settle_in,
+                             bucket_width, warp_degree, team_degree, hot_vertices) */
 #define BC_ALGO_STRICT 1u /* the paper's phases: settle every vertex that meets the strict OUT (Eq. 2 + Eq. 4) or
                              IN criterion, sigma pulled as each batch settles (Sec. 3.2, Algorithm 2) */
 #define BC_ALGO_DELTA 2u  /* sweep schedule: distances by rounds of frontier relaxation (bucket width =

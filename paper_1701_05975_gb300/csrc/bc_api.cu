@@ -140,6 +140,7 @@ struct bc_graph {
   void* land_in = nullptr;      // undirected graphs: land_out
   uint64_t land_stride = 0;
   uint32_t land_bits = 0, nland = 0, land_n = 0;
+  double ties = -1.0;           // shortest-path DAG edges per vertex and probe source (< 0: not probed)
   uint32_t act_n = 0;           // vertices from this id on have no entries (active_vertices)
   uint32_t* esm = nullptr;  // edge output: walked entry -> caller's output entry (built on first use)
   int esm_state = 0;        // 0 not built, 1 ready, 2 unavailable (an entry without a twin)
@@ -211,6 +212,8 @@ void ws_free(Workspace* w) {
 SlabKind slab_kind(const RunCfg& r) {
   return r.algo != ALGO_DELTA ? SLAB_STRICT : (r.sweep.mem == 2 ? SLAB_NONE : SLAB_SWEEP);
 }
+
+constexpr uint32_t LAND_MIN_N = 256;  // fewer vertices get no landmarks
 
 // Sparse graphs without landmarks: small frontiers in many rounds.
 bool sweep_sparse(const bc_graph* g) { return !g->kadj && (double)g->nnz < 6.0 * g->n; }
@@ -284,34 +287,73 @@ uint64_t sweep_width_default(const bc_graph* g) {
   return g->kadj ? ~0ull : sweep_bucket_width(g->max_w, g->n, g->nnz);
 }
 
+// Threads per source of the strict schedule: the widest CTA teams for dense
+// skewed graphs (large frontiers per batch; half as many sources in flight keeps
+// more of each source's distance array in L2), 128 threads for sparse
+// high-diameter graphs.  By entries walked per vertex: a directed graph's
+// batches walk in- and out-edges.
+uint32_t strict_team_default(const bc_graph* g) {
+  const double walked = g->n ? (double)g->nnz * (g->directed ? 2.0 : 1.0) / g->n : 0.0;
+  return walked >= 20.0 ? (g->dist_bits == 32 ? 1024u : 512u) : (walked >= 6.0 ? 256u : 128u);
+}
+
+// Whether the strict schedule is the faster one for k sources (0: many) of a graph.
+// It wins where its settle batches are few, which is where many paths tie: small
+// weights, seen in the probe sources' shortest-path DAGs (ties: edges per vertex).
+// Then the sweep's rounds, DAG build and two passes over the levels are more dependent
+// steps than the batches, each entry is walked three or four times instead of once
+// or twice, and without landmarks nothing is skipped for it.  Measured over 1035
+// graphs and 5000 runs, strict / sweep time:
+//   Erdos-Renyi of degree 16, all sources, n = 1024: 0.61 at weights to 3 (ties 2.1), 0.93
+//   to 16 (1.22), 1.45 to 64 (1.06); n = 8192, 1216 sources: 0.73 to 6 (1.6), 0.78 to 16
+//   (1.22), 0.92 to 64 (1.06), 1.13 to 128;
+//   a list of DAG edges that outgrows the strict slabs (ties above 2) costs a second scan:
+//   1.0 at weights to 3, and hubs make it worse (R-MAT 2^12 at unit weights 1.34);
+//   its teams are narrow, so few sources favour the sweep's wide ones from 1536 vertices
+//   on (Barabasi-Albert 2500, weights to 2: 0.66 at 1216 sources, 1.05 at 40); 20 and more
+//   entries walked per vertex make the strict teams wide: then only few sources of a
+//   small graph (Erdos-Renyi of degree 32, n = 700, weights to 4: 0.66 at 40, 1.28 at 700);
+//   sparse graphs, not probed: grids 0.71 and 0.96 at weights to 1 and 2 (n = 900), 0.76 / 0.83 / 0.90 / 1.01 at weights to 1 / 2 / 3 / 5
+//   (n = 40,000, 1216 sources), 1.5 and more at 304 sources.
+bool strict_is_faster(const bc_graph* g, uint32_t k) {
+  if (g->kadj) return false;
+  const double walked = (double)g->nnz * (g->directed ? 2.0 : 1.0) / g->n;
+  const bool few = k && k <= (uint32_t)g->sm_count;
+  if (g->ties < 0.0) {
+    if (g->n < LAND_MIN_N) return !g->directed && walked >= 6.0 && walked < 20.0 && g->max_w < 0.5 * walked;
+    if (sweep_sparse(g) && !g->relabeled)
+      return g->n > 700 && g->max_w <= (g->n > 1100 ? 3u : 2u) && (!k || k > 4ull * g->sm_count);
+    return false;
+  }
+  if (walked >= 20.0) return g->n <= SWEEP_SMEM_N && few && g->ties > 1.2;
+  if (g->n <= SWEEP_SMEM_N) return few ? walked >= 6.0 && g->ties > 1.5 : g->ties > 1.25;
+  if (g->n >= 32768 || (k && k < (uint64_t)g->sm_count * (1024 / strict_team_default(g)))) return false;
+  return g->ties > 1.1 && (g->ties < 2.0 || !g->relabeled) && (walked >= 6.0 || g->n < 16000);
+}
+
 // Settings for a run: explicit config fields win, then the graph's tuned
-// values, then heuristics.  k: sources of the run (0: not known, many).
-RunCfg resolve(const bc_graph* g, uint32_t k, uint32_t force_algo = BC_ALGO_AUTO) {
+// values, then heuristics.  k: sources of the run (0: not known, many).  edges:
+// edge output, for which the strict schedule would first have to build its map of
+// twin entries on the host.
+RunCfg resolve(const bc_graph* g, uint32_t k, uint32_t force_algo = BC_ALGO_AUTO, bool edges = false) {
   bc_config c = config_snapshot();
   if (force_algo) c.algorithm = force_algo;
   RunCfg r;
   r.mode = c.mode;
-  // entries walked per vertex: a directed graph's batches walk in- and out-edges
-  const double avg_deg = g->n ? (double)g->nnz * (g->directed ? 2.0 : 1.0) / g->n : 0.0;
-  // measured defaults: the widest CTA teams for dense skewed graphs (large
-  // frontiers per batch; half as many sources in flight keeps more of each
-  // source's distance array in L2), 128-thread teams for sparse high-diameter
-  // graphs
-  const uint32_t wide = g->dist_bits == 32 ? 1024u : 512u;
-  const uint32_t team_default = avg_deg >= 20.0 ? wide : (avg_deg >= 6.0 ? 256u : 128u);
-  // the sweep schedule unless the configuration asks for the strict one or
-  // sets a knob that only the strict one has
+  // the sweep schedule unless the configuration asks for the strict one, sets a
+  // knob that only that one has, or it is the faster one
   const bool strict_knob = c.settle_in || c.bucket_width || c.warp_degree || c.team_degree || c.hot_vertices;
   const uint32_t al = c.algorithm ? c.algorithm
                                   : (strict_knob || g->n >= 0x80000000u || g->nnz + g->n >= (1ull << 32)
                                      ? (uint32_t)BC_ALGO_STRICT
-                                     : (g->tuned.algo ? g->tuned.algo : (uint32_t)BC_ALGO_DELTA));
+                                     : (g->tuned.algo ? g->tuned.algo
+                                                    : (uint32_t)(!edges && strict_is_faster(g, k) ? BC_ALGO_STRICT : BC_ALGO_DELTA)));
   r.algo = (al == BC_ALGO_DELTA) ? ALGO_DELTA : ALGO_STRICT;
   r.algo_auto = c.algorithm == BC_ALGO_AUTO;
   const bool sweep = r.algo == ALGO_DELTA;
   const uint32_t tuned_team = sweep ? g->tuned.sweep_team : g->tuned.team;
   r.team = c.team_threads ? c.team_threads
-                          : (tuned_team ? tuned_team : (sweep ? sweep_team_default(g, k) : team_default));
+                          : (tuned_team ? tuned_team : (sweep ? sweep_team_default(g, k) : strict_team_default(g)));
   if (r.team == 1024 && g->dist_bits != 32) r.team = 512;  // 1024-thread teams hold 32-bit distances only
   const uint64_t tuned_width = sweep ? g->tuned.sweep_width : g->tuned.width;
   r.width = c.bucket_width ? c.bucket_width
@@ -837,7 +879,6 @@ void free_landmarks(bc_graph* g) {
 constexpr double LAND_KEEP_MAX = 0.5;
 constexpr double LAND_KEEP_MAX_DENSE = 0.35;
 constexpr uint32_t LAND_PROBES = 4;
-constexpr uint32_t LAND_MIN_N = 256;
 constexpr uint32_t LAND_MAX_N_FLAT = 32768;
 
 cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<uint64_t>& tdeg) {
@@ -936,18 +977,19 @@ cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<u
   }
   if (e == cudaSuccess && !g->directed) e = land_symmetry(fwd, sums, st);
   if (e == cudaSuccess) e = land_judge(fwd, tab, tab + (uint64_t)L * n, h, probes, sums + 2, st);
-  if (e == cudaSuccess) e = land_max((uint64_t)L * n, tab, reinterpret_cast<uint32_t*>(sums + 5), st);
+  if (e == cudaSuccess) e = land_max((uint64_t)L * n, tab, reinterpret_cast<uint32_t*>(sums + 6), st);
   if (e == cudaSuccess && g->directed)
-    e = land_max((uint64_t)L * n, tab_in, reinterpret_cast<uint32_t*>(sums + 5), st);
+    e = land_max((uint64_t)L * n, tab_in, reinterpret_cast<uint32_t*>(sums + 6), st);
   std::vector<unsigned char> host(2 * sizeof(Ctl) + 8 * 8);
   if (e == cudaSuccess) e = cudaMemcpyAsync(host.data(), ctl, host.size(), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return done(e);
-  unsigned long long hs[6];
+  unsigned long long hs[7];
   memcpy(hs, host.data() + 2 * sizeof(Ctl), sizeof hs);
   const Ctl* hc = reinterpret_cast<const Ctl*>(host.data());
-  const uint32_t max_d = (uint32_t)hs[5];
+  const uint32_t max_d = (uint32_t)hs[6];
   if (hc[0].err != DEV_OK || hc[1].err != DEV_OK || hs[0] != hs[1]) return done(cudaSuccess);
+  g->ties = (double)hs[5] / ((double)probes * n);
   const bool dense = !g->relabeled && n > SWEEP_SMEM_N && g->nnz >= 24ull * n;
   const double keep_max = dense ? LAND_KEEP_MAX_DENSE : LAND_KEEP_MAX;
   if (hs[2] == 0 || (double)hs[3] > keep_max * (double)hs[2]) return done(cudaSuccess);
@@ -1421,7 +1463,7 @@ int compute_async(bc_graph* g, const uint32_t* d_sources, uint32_t k, double sca
   if (!d_out_bc) return fail(BC_ERR_INVALID, "null d_out_bc");
   if (k && !d_sources) return fail(BC_ERR_INVALID, "null d_sources");
   CK(cudaSetDevice(g->device));
-  RunCfg r = resolve(g, k);
+  RunCfg r = resolve(g, k, BC_ALGO_AUTO, d_out_ebc != nullptr);
   if (r.mode != BC_MODE_BATCHED) return fail(BC_ERR_INVALID, "the async entry points run the batched mode only");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // the workspace this stream kept from its previous async call: that run
@@ -1530,7 +1572,7 @@ int bc_edge_compute(bc_graph_t g, const uint32_t* sources, uint32_t k, double sc
   if (!out_ebc) return fail(BC_ERR_INVALID, "null out_ebc");
   if (k && !sources) return fail(BC_ERR_INVALID, "null sources");
   CK(cudaSetDevice(g->device));
-  RunCfg r = resolve(g, k);
+  RunCfg r = resolve(g, k, BC_ALGO_AUTO, true);
   std::vector<double> tmp;
   if (!out_bc) {
     tmp.resize(g->n);

@@ -77,12 +77,12 @@ __global__ void land_symmetry_kernel(uint32_t n, uint64_t nnz, uint32_t chunk, c
 // Judge the main landmark h on probe sources (distances probe[p * n + v],
 // so D(probe p, h) = probe[p * n + h]): out[0] entries of reached rows, out[1] those the
 // prefix test keeps.  out[2]: 1 + the largest vertex with entries that the main
-// landmark reaches.
+// landmark reaches.  out[3]: entries on shortest paths from the probes (tight ones).
 __global__ void land_judge_kernel(uint32_t n, uint64_t nnz, uint32_t chunk, const uint64_t* __restrict__ row_ptr,
                                   const uint2* __restrict__ adj, const uint32_t* __restrict__ from_h,
                                   const uint32_t* __restrict__ probe, uint32_t h, uint32_t nprobe,
                                   unsigned long long* out) {
-  unsigned long long all = 0, kept = 0, last = 0;
+  unsigned long long all = 0, kept = 0, last = 0, tight = 0;
   land_entries(n, nnz, row_ptr, chunk, [&](uint32_t v, uint64_t e) {
     const uint2 x = adj[e];
     const uint32_t hu = from_h[x.x];
@@ -91,6 +91,7 @@ __global__ void land_judge_kernel(uint32_t n, uint64_t nnz, uint32_t chunk, cons
       const uint32_t c = probe[(uint64_t)p * n + h], d = probe[(uint64_t)p * n + v];
       if (c == 0xffffffffu || d == 0xffffffffu) continue;
       ++all;
+      tight += probe[(uint64_t)p * n + x.x] == d + x.y;
       kept += hu == 0xffffffffu || (long long)x.y - (long long)hu <= (long long)c - (long long)d;
     }
   });
@@ -98,12 +99,14 @@ __global__ void land_judge_kernel(uint32_t n, uint64_t nnz, uint32_t chunk, cons
   for (int o = 16; o > 0; o >>= 1) {
     all += __shfl_xor_sync(0xffffffffu, all, o);
     kept += __shfl_xor_sync(0xffffffffu, kept, o);
+    tight += __shfl_xor_sync(0xffffffffu, tight, o);
     last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
   }
   if ((threadIdx.x & 31) == 0) {
     atomicAdd(&out[0], all);
     atomicAdd(&out[1], kept);
     atomicMax(&out[2], last);
+    atomicAdd(&out[3], tight);
   }
 }
 

@@ -185,3 +185,33 @@ def test_dense_rows_without_landmarks_run_in_slabs(n, m):
             ebc, vbc = G.edge_compute(src, 0.5)
             assert_bc_close(ebc, wante)
             assert_bc_close(vbc, want)
+
+
+@pytest.mark.parametrize("graph,k,strict", [
+    (lambda: gen.er_graph(1024, 8192, 1, 3, seed=1), 1024, True),
+    (lambda: gen.er_graph(1024, 8192, 1, 3, seed=1), 100, True),
+    (lambda: gen.er_graph(1024, 8192, 1, 100, seed=1), 1024, False),
+    (lambda: gen.er_graph(9000, 72000, 1, 8, seed=2), 608, True),
+    (lambda: gen.er_graph(9000, 72000, 1, 8, seed=2), 607, False),
+    (lambda: gen.er_graph(2000, 32000, 1, 4, seed=3), 2000, False),
+    (lambda: gen.er_graph(200, 1600, 1, 2, seed=4), 200, True),
+    (lambda: gen.grid_graph(40, 40, wmin=1, wmax=2, seed=5), 1000, True),
+    (lambda: gen.grid_graph(40, 40, wmin=1, wmax=2, seed=5), 100, False),
+    (lambda: gen.ba_graph(3000, 4, 1, 2, seed=6), 3000, True),
+    (lambda: gen.ba_graph(3000, 4, 1, 50, seed=6), 3000, False),
+], ids=str)
+def test_small_weights_take_the_strict_schedule(graph, k, strict):
+    """AUTO's choice by tied paths and sources; edge output and a pinned schedule are not affected."""
+    g = graph()
+    src = np.arange(k, dtype=np.uint32)
+    want = oracle.bc(g, src, 0.5, nthreads=8)
+    with bc.Graph(g) as G:
+        assert_bc_close(G.compute(src, 0.5), want)
+        assert G.stats().algorithm == (bc.BC_ALGO_STRICT if strict else bc.BC_ALGO_DELTA)
+        assert_bc_close(G.submit(src, 0.5).result(60000), want)
+        ebc, vbc = G.edge_compute(src[:40], 0.5)
+        assert G.stats().algorithm == bc.BC_ALGO_DELTA
+        assert_bc_close(ebc, oracle.edge_bc(g, src[:40], 0.5))
+        bc.bc_set_config(algorithm=bc.BC_ALGO_DELTA)
+        assert_bc_close(G.compute(src, 0.5), want)
+        assert G.stats().algorithm == bc.BC_ALGO_DELTA
