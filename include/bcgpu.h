@@ -388,12 +388,14 @@ int bc_step_destroy(bc_step_t step);
  * before any stream capture.  Calls share the array and each re-initialises
  * it; calls whose work overlaps on the GPU (other streams or threads without
  * ordering) race on it.  On BC_ERR_INVALID no source runs and d_out_bc is all
- * zeros.  The sweep schedule runs unless one of the bc_config fields of the
- * strict schedule is set (bucket_width, settle_in, warp_degree, team_degree), algorithm
- * is BC_ALGO_STRICT or only a strict slab fits; phase_cap applies to both, the other fields are
- * ignored.  The strict schedule's bucket_width 0 means a fixed 64 (the call
- * never reads the weights on the host; the sweep schedule's width comes from the
- * largest weight, found on the device), and its team size follows the average
+ * zeros.  The strict schedule runs when one of its bc_config fields is set
+ * (bucket_width, settle_in, warp_degree, team_degree), algorithm is
+ * BC_ALGO_STRICT or only a strict slab fits; else the sweep schedule with
+ * BC_ALGO_DELTA, and by default whichever the largest weight, found on the
+ * device, the degree and the sources make the faster one.  phase_cap applies to
+ * both, the other fields are ignored.  The strict schedule's bucket_width 0 means
+ * a fixed 64 (the call never reads the weights on the host; the sweep schedule's
+ * width comes from the largest weight), and its team size follows the average
  * degree (>= 20: 512, >= 12: 256, else 128 threads).
  */
 #define BC_NOALLOC_SCRATCH_BYTES (64ull << 20)

@@ -310,11 +310,12 @@ uint32_t strict_team_default(const bc_graph* g) {
 //   a list of DAG edges that outgrows the strict slabs (ties above 2) costs a second scan:
 //   1.0 at weights to 3, and hubs make it worse (R-MAT 2^12 at unit weights 1.34);
 //   its teams are narrow, so few sources favour the sweep's wide ones from 1536 vertices
-//   on (Barabasi-Albert 2500, weights to 2: 0.66 at 1216 sources, 1.05 at 40); 20 and more
-//   entries walked per vertex make the strict teams wide: then only few sources of a
-//   small graph (Erdos-Renyi of degree 32, n = 700, weights to 4: 0.66 at 40, 1.28 at 700);
-//   sparse graphs, not probed: grids 0.71 and 0.96 at weights to 1 and 2 (n = 900), 0.76 / 0.83 / 0.90 / 1.01 at weights to 1 / 2 / 3 / 5
-//   (n = 40,000, 1216 sources), 1.5 and more at 304 sources.
+//   on (Erdos-Renyi n = 8192, weights to 4: 1.65 at 40 sources, 1.04 at 304, 0.68 at
+//   608); 20 and more entries walked per vertex make the strict teams wide: then only few
+//   sources of a small graph (Erdos-Renyi of degree 32, n = 700, weights to 4: 0.66 at 40,
+//   1.28 at 700);
+//   sparse graphs, not probed: grids 0.71 and 0.96 at weights to 1 and 2 (n = 900), 0.76 / 0.83
+//   / 0.90 / 1.01 at weights to 1 / 2 / 3 / 5 (n = 40,000, 1216 sources), 1.5 and more at 304.
 bool strict_is_faster(const bc_graph* g, uint32_t k) {
   if (g->kadj) return false;
   const double walked = (double)g->nnz * (g->directed ? 2.0 : 1.0) / g->n;

@@ -226,9 +226,11 @@ cudaError_t launch_pack32(uint64_t nnz, const uint32_t* col, const uint32_t* w, 
 cudaError_t launch_fill_u64(uint64_t* p, uint64_t count, uint64_t value, cudaStream_t st);
 cudaError_t launch_scale(double* p, uint64_t count, double scale, cudaStream_t st);
 cudaError_t launch_check_sources(const uint32_t* src, uint32_t k, uint32_t n, int* err, cudaStream_t st);
-// Fill `bytes` (a multiple of 4) at offset `off` of every slot of a slab array.
+// Fill `bytes` (a multiple of 4) at offset `off` of every slot of a slab array;
+// nothing if *gate, a source counter, is parked (nullptr: always).
+constexpr uint32_t PARKED = 0x80000000u;  // a source counter from here on hands out no source
 cudaError_t launch_fill_slabs(char* base, uint64_t stride, uint32_t nslots, uint64_t off, uint64_t bytes,
-                              uint32_t value, cudaStream_t st);
+                              uint32_t value, cudaStream_t st, const uint32_t* gate = nullptr);
 
 // Record a message for bc_last_error() on the calling thread; returns code.
 int set_error(int code, const char* msg);

@@ -20,7 +20,12 @@
 //
 // All calls share the array, and it keeps whatever the last call left there.
 // Each call therefore re-initialises what must start at a known value: the
-// control block, the distance words (INF) and the backward accumulators (0).
+// control block, and in slabs the distance words (INF) and the vertex records
+// and bits of the sweep schedule or the backward accumulators of the strict one (0).
+//
+// Both schedules are enqueued where either may be the faster one: the largest
+// weight decides, and only the device knows it.  The kernel and the fills of the one
+// not chosen find its source counter parked and leave.
 // Two calls whose work overlaps on the GPU (different streams, or different
 // host threads, without ordering between them) race on the array.
 #include <cuda_runtime.h>
@@ -83,7 +88,7 @@ unsigned long long current_ctx_id() {
 }
 
 struct NaCtl {
-  uint32_t counter;
+  uint32_t counter[2];  // sources handed out by the sweep kernel and by the strict one
   int err;
   uint32_t debug[2];
   unsigned long long stats[STAT_COUNT];
@@ -92,6 +97,7 @@ struct NaCtl {
   unsigned long long sym[2];
   unsigned long long width;  // sweep schedule: bucket width, from the largest weight
   uint32_t max_w;
+  uint32_t blocks_done;      // of the validation kernel
 };
 
 // The device status word carries DEV_* codes; the caller reads them as BC_* codes.
@@ -114,69 +120,117 @@ __device__ __forceinline__ uint64_t entry_hash(uint32_t a, uint32_t b, uint32_t 
   return mix64((((uint64_t)a << 32) | b) ^ mix64((uint64_t)w + 0x9e3779b97f4a7c15ull));
 }
 
+// Strict slabs that the validation kernel initialises on the side (slots 0: none).
+struct NaFill {
+  char* slabs;
+  uint64_t stride, off_acc;  // distances (INF) at 0, accumulators (0) at off_acc
+  uint32_t slots;
+};
+
 // Validates the caller's CSR while packing it (every read stays inside the
 // caller's arrays whatever their contents) and computes Delta_node.  On any
-// violation it records DEV_ERR_INVALID and parks the source counter far above
-// any source index, so the batched kernel that follows does no work.  It also
+// violation it records DEV_ERR_INVALID and parks the source counters far above
+// any source index, so the kernels that follow do no work.  It also
 // sums, mod 2^64, a hash of every entry (v -> u, w) and of its reverse
-// (u -> v, w); na_check_symmetry compares the two sums.
+// (u -> v, w): an asymmetric CSR (some entry without its reverse entry of the same
+// weight) makes the two sums differ; the block that ends last compares them and
+// rejects it like any other invalid input.  That block also derives what follows from
+// the largest weight: the sweep schedule's bucket width, by the same rule as for
+// a prepared graph, and the schedule: the strict one from `strict_from` to `strict_to`.
+// Blocks from `rows` on fill the strict slabs meanwhile: as launches of their own the fills,
+// the check and the strict kernel cost a call 12 us (of 155 at 300 vertices), this way 1.
 __global__ void na_validate_prep(uint32_t n, uint64_t nnz, const uint64_t* __restrict__ row_ptr,
                                  const uint32_t* __restrict__ col, const uint32_t* __restrict__ w,
                                  const uint32_t* __restrict__ src, uint32_t k, uint2* __restrict__ adj,
-                                 uint32_t* __restrict__ dnode, NaCtl* ctl) {
-  const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  const uint64_t nth = (uint64_t)gridDim.x * blockDim.x;
-  bool bad = false;
-  uint32_t heaviest = 0;
-  unsigned long long fwd = 0, rev = 0;
-  if (tid == 0 && (row_ptr[0] != 0 || row_ptr[n] != nnz)) bad = true;
-  for (uint64_t v = tid; v < n; v += nth) {
-    const uint64_t r0 = row_ptr[v], r1 = row_ptr[v + 1];
-    uint32_t m = 0xffffffffu;
-    if (r0 > r1 || r1 > nnz) {
-      bad = true;
-    } else {
-      for (uint64_t e = r0; e < r1; ++e) {
-        const uint32_t c = col[e], ww = w[e];
-        if (c >= n || ww == 0) bad = true;
-        adj[e] = make_uint2(c < n ? c : 0u, ww);
-        m = min(m, ww);
-        heaviest = max(heaviest, ww);
-        fwd += entry_hash((uint32_t)v, c, ww);
-        rev += entry_hash(c, (uint32_t)v, ww);
+                                 uint32_t* __restrict__ dnode, NaCtl* ctl, uint32_t strict_from, uint32_t strict_to,
+                                 uint32_t rows, NaFill fill) {
+  if (blockIdx.x < rows) {
+    const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    const uint64_t nth = (uint64_t)rows * blockDim.x;
+    bool bad = false;
+    uint32_t heaviest = 0;
+    unsigned long long fwd = 0, rev = 0;
+    if (tid == 0 && (row_ptr[0] != 0 || row_ptr[n] != nnz)) bad = true;
+    for (uint64_t v = tid; v < n; v += nth) {
+      const uint64_t r0 = row_ptr[v], r1 = row_ptr[v + 1];
+      uint32_t m = 0xffffffffu;
+      if (r0 > r1 || r1 > nnz) {
+        bad = true;
+      } else {
+        for (uint64_t e = r0; e < r1; ++e) {
+          const uint32_t c = col[e], ww = w[e];
+          if (c >= n || ww == 0) bad = true;
+          adj[e] = make_uint2(c < n ? c : 0u, ww);
+          m = min(m, ww);
+          heaviest = max(heaviest, ww);
+          fwd += entry_hash((uint32_t)v, c, ww);
+          rev += entry_hash(c, (uint32_t)v, ww);
+        }
+      }
+      dnode[v] = m;
+    }
+    for (uint64_t i = tid; i < k; i += nth)
+      if (src[i] >= n) bad = true;
+    for (int o = 16; o > 0; o >>= 1) {
+      fwd += __shfl_xor_sync(0xffffffffu, fwd, o);
+      rev += __shfl_xor_sync(0xffffffffu, rev, o);
+      heaviest = max(heaviest, __shfl_xor_sync(0xffffffffu, heaviest, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+      atomicMax(&ctl->max_w, heaviest);
+      atomicAdd(&ctl->sym[0], fwd);
+      atomicAdd(&ctl->sym[1], rev);
+    }
+    if (bad) {
+      atomicCAS(&ctl->err, DEV_OK, DEV_ERR_INVALID);
+      atomicExch(&ctl->counter[0], PARKED);
+      atomicExch(&ctl->counter[1], PARKED);
+    }
+  } else {
+    for (uint32_t slot = blockIdx.x - rows; slot < fill.slots; slot += gridDim.x - rows) {
+      uint64_t* d = reinterpret_cast<uint64_t*>(fill.slabs + slot * fill.stride);
+      uint64_t* acc = reinterpret_cast<uint64_t*>(fill.slabs + slot * fill.stride + fill.off_acc);
+      for (uint32_t v = threadIdx.x; v < n; v += blockDim.x) {
+        d[v] = ~0ull;
+        acc[v] = 0;
       }
     }
-    dnode[v] = m;
   }
-  for (uint64_t i = tid; i < k; i += nth)
-    if (src[i] >= n) bad = true;
-  for (int o = 16; o > 0; o >>= 1) {
-    fwd += __shfl_xor_sync(0xffffffffu, fwd, o);
-    rev += __shfl_xor_sync(0xffffffffu, rev, o);
-    heaviest = max(heaviest, __shfl_xor_sync(0xffffffffu, heaviest, o));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicMax(&ctl->max_w, heaviest);
-    atomicAdd(&ctl->sym[0], fwd);
-    atomicAdd(&ctl->sym[1], rev);
-  }
-  if (bad) {
-    atomicCAS(&ctl->err, DEV_OK, DEV_ERR_INVALID);
-    atomicExch(&ctl->counter, 0x80000000u);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&ctl->blocks_done, 1u) == gridDim.x - 1) {
+      __threadfence();
+      const uint32_t max_w = atomicMax(&ctl->max_w, 0u);
+      ctl->width = sweep_bucket_width(max_w, n, nnz);
+      atomicExch(&ctl->counter[max_w >= strict_from && max_w <= strict_to ? 0 : 1], PARKED);
+      if (atomicAdd(&ctl->sym[0], 0ull) != atomicAdd(&ctl->sym[1], 0ull)) {
+        atomicCAS(&ctl->err, DEV_OK, DEV_ERR_INVALID);
+        atomicExch(&ctl->counter[0], PARKED);
+        atomicExch(&ctl->counter[1], PARKED);
+      }
+    }
   }
 }
 
-// An asymmetric CSR (some entry without its reverse entry of the same
-// weight) makes the two hash sums differ; it is then rejected like any other
-// invalid input.  Also the sweep schedule's bucket width, by the same rule as
-// for a prepared graph (the weights are only known on the device).  Single
-// thread.
-__global__ void na_check_symmetry(NaCtl* ctl, uint32_t n, uint64_t nnz, unsigned long long width) {
-  ctl->width = width ? width : sweep_bucket_width(ctl->max_w, n, nnz);
-  if (ctl->sym[0] != ctl->sym[1]) {
-    atomicCAS(&ctl->err, DEV_OK, DEV_ERR_INVALID);
-    atomicExch(&ctl->counter, 0x80000000u);
-  }
+// Largest weight at which the strict schedule is the faster one here, where the sweep
+// has neither landmarks nor 32-bit words: one unit of weight per entry of a row up to
+// 500 vertices, two up to 1300, then with the square of the degree (the shared-memory form
+// holds three teams to an SM, and slabs fewer sources than the strict schedule's).
+// Strict / sweep time of this call, all sources: Erdos-Renyi of degree 8 n = 1024
+// 0.85 / 1.02 / 1.34 at weights to 4 / 16 / 32, of degree 16 0.92 / 1.13 / 1.44 at 16 / 32 / 64,
+// of degree 32 0.65 / 0.81 / 1.07 at 32 / 64 / 128; n = 4096, degree 8 1.03 / 1.25 at 16 /
+// 32, degree 16 0.85 / 0.97 at 64 / 128, degree 32 0.63 / 0.82 at 128 / 300; R-MAT 2^12 of
+// degree 27 0.29 at 8.  Few sources leave the narrow strict teams alone on their SMs: half
+// of it.  Sparse rows: grids 0.78 / 0.90 / 1.07 at 3 / 4 / 6.  At unit weights the strict
+// schedule's list of DAG edges outgrows its slab and costs a second scan (1.12 at n = 4096,
+// degree 8; below 1300 vertices the sweep's list in shared memory does, too).
+uint32_t na_strict_to(uint32_t n, uint64_t nnz, uint32_t k) {
+  const double deg = (double)nnz / n;
+  const bool few = k < 608 && k < n;
+  if (deg < 6.0) return n > 500 && !few ? 4u : 0u;
+  const double w = n <= 500 ? deg : (n <= 1300 ? 2.0 * deg : 0.25 * deg * deg);
+  return (uint32_t)std::min(few ? 0.5 * w : w, 4.0e9);
 }
 
 int na_fail(int code, const char* msg) { return set_error(code, msg); }
@@ -234,82 +288,94 @@ extern "C" int bc_compute_noalloc(const uint64_t* d_row_ptr, const uint32_t* d_c
   bc_config cfg;
   bc_get_config(&cfg);
   const double avg_deg = (double)nnz / n;
-  int team = avg_deg >= 20.0 ? 512 : (avg_deg >= 12.0 ? 256 : 128);
-  SlabKind kind = SLAB_STRICT;
-  SlabLayout lay = strict_lay;
-  SweepPlan plan;
   // the sweep schedule unless a knob of the strict one is set; its slab is a
   // little larger, so a graph of which just one strict slab fits stays strict
-  if (cfg.algorithm != BC_ALGO_STRICT && !cfg.bucket_width && !cfg.settle_in && !cfg.warp_degree &&
-      !cfg.team_degree) {
-    plan.dist_bits = 64;
-    plan.team = 256;
-    plan.group = avg_deg >= 12.0 ? 8 : 1;
-    sweep_place(plan, n, n, true);
-    const SlabKind sk = plan.mem == 2 ? SLAB_NONE : SLAB_SWEEP;
-    const SlabLayout sl = make_layout(n, 64, sk);
-    if (off_slabs + sl.stride <= BC_NOALLOC_SCRATCH_BYTES) {
-      kind = sk;
-      lay = sl;
-      team = plan.team;
-    }
+  SweepPlan plan;
+  plan.dist_bits = 64;
+  plan.team = 256;
+  plan.group = avg_deg >= 12.0 ? 8 : 1;
+  sweep_place(plan, n, n, true);
+  const SlabKind kind = plan.mem == 2 ? SLAB_NONE : SLAB_SWEEP;
+  const SlabLayout lay = make_layout(n, 64, kind);
+  const bool sweep = cfg.algorithm != BC_ALGO_STRICT && !cfg.bucket_width && !cfg.settle_in && !cfg.warp_degree &&
+                     !cfg.team_degree && off_slabs + lay.stride <= BC_NOALLOC_SCRATCH_BYTES;
+  const uint32_t strict_to =
+      !sweep ? 0xffffffffu : (cfg.algorithm == BC_ALGO_DELTA ? 0u : na_strict_to(n, nnz, k));
+  const uint32_t strict_from = !sweep ? 0u : (n > 1300 && avg_deg >= 6.0 && avg_deg < 12.0 ? 2u : 1u);
+  const int team = avg_deg >= 20.0 ? 512 : (avg_deg >= 12.0 ? 256 : 128);
+  // sources in flight and CTAs of each schedule
+  auto in_flight = [&](uint64_t stride, uint32_t threads, int bps, uint32_t* slots, int* grid) {
+    const uint32_t per_block = (uint32_t)(batched_block_threads((int)threads) / (int)threads);
+    uint64_t s = (uint64_t)std::max(bps, 1) * sms * per_block;
+    s = std::min<uint64_t>(s, (BC_NOALLOC_SCRATCH_BYTES - off_slabs) / stride);
+    *slots = (uint32_t)std::min<uint64_t>(s, std::max<uint32_t>(k, 1));
+    *grid = (int)((*slots + per_block - 1) / per_block);
+  };
+  uint32_t slots = 0, strict_slots = 0;
+  int grid = 0, strict_grid = 0, bps = 0;
+  if (strict_to) {
+    e = batched_occupancy(64, team, &bps);
+    if (e != cudaSuccess) return na_fail(BC_ERR_CUDA, cudaGetErrorString(e));
+    in_flight(strict_lay.stride, (uint32_t)team, bps, &strict_slots, &strict_grid);
   }
-  int bps = 0;
-  e = kind == SLAB_STRICT ? batched_occupancy(64, team, &bps) : sweep_occupancy(plan, &bps);
-  if (e != cudaSuccess) return na_fail(BC_ERR_CUDA, cudaGetErrorString(e));
-  const uint32_t per_block = (uint32_t)(batched_block_threads(team) / team);
-  uint64_t slots = (uint64_t)std::max(bps, 1) * sms * per_block;
-  slots = std::min<uint64_t>(slots, (BC_NOALLOC_SCRATCH_BYTES - off_slabs) / lay.stride);
-  slots = std::min<uint64_t>(slots, std::max<uint32_t>(k, 1));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   NaCtl* ctl = reinterpret_cast<NaCtl*>(base);
   uint2* adj = reinterpret_cast<uint2*>(base + off_adj);
   uint32_t* dnode = reinterpret_cast<uint32_t*>(base + off_dnode);
   char* slabs = base + off_slabs;
 
+  // strict slabs that share no memory with sweep ones are filled while the input is validated
+  const bool fill_early = strict_to && (!sweep || kind == SLAB_NONE);
   e = cudaMemsetAsync(ctl, 0, sizeof(NaCtl), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(d_out_bc, 0, (size_t)n * 8, st);
   if (e == cudaSuccess) {
     const uint64_t work = std::max<uint64_t>(n, k);
-    const int grid = (int)std::min<uint64_t>((work + 255) / 256, (uint64_t)sms * 8);
-    na_validate_prep<<<std::max(grid, 1), 256, 0, st>>>(n, nnz, d_row_ptr, d_col_idx, d_w, d_sources, k, adj, dnode,
-                                                        ctl);
+    const uint32_t rows = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((work + 255) / 256, (uint64_t)sms * 8));
+    const NaFill fill{slabs, strict_lay.stride, strict_lay.off_acc, fill_early ? strict_slots : 0u};
+    na_validate_prep<<<rows + std::min<uint32_t>(fill.slots, 4u * sms), 256, 0, st>>>(
+        n, nnz, d_row_ptr, d_col_idx, d_w, d_sources, k, adj, dnode, ctl, strict_from, strict_to, rows, fill);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) {
-    na_check_symmetry<<<1, 1, 0, st>>>(ctl, n, nnz, cfg.bucket_width);
-    e = cudaGetLastError();
+  if (e == cudaSuccess && sweep) {  // asked for while the GPU validates
+    e = sweep_occupancy(plan, &bps);
+    in_flight(lay.stride, (uint32_t)plan.team, bps, &slots, &grid);
   }
-  if (e == cudaSuccess) e = init_slabs(slabs, lay, kind, (uint32_t)slots, n, 64, st);
-  if (e == cudaSuccess) {
-    BatchArgs a{};
-    a.g.n = n;
-    a.g.nnz = nnz;
-    a.g.row_ptr = d_row_ptr;
-    a.g.adj = adj;
-    a.g.adjp = nullptr;
-    a.g.dnode = dnode;
-    a.g.act_n = n;
-    a.sources = d_sources;
-    a.k = k;
-    a.counter = &ctl->counter;
-    a.bc = d_out_bc;
-    a.ebc = nullptr;
-    a.slabs = slabs;
-    a.lay = lay;
-    a.nslots = (uint32_t)slots;
+  BatchArgs a{};
+  a.g.n = n;
+  a.g.nnz = nnz;
+  a.g.row_ptr = d_row_ptr;
+  a.g.adj = adj;
+  a.g.adjp = nullptr;
+  a.g.dnode = dnode;
+  a.g.act_n = n;
+  a.sources = d_sources;
+  a.k = k;
+  a.bc = d_out_bc;
+  a.ebc = nullptr;
+  a.slabs = slabs;
+  a.phase_cap = cfg.phase_cap ? cfg.phase_cap : 4ull * n + 64;  // phases + refills <= 4n + 2
+  a.err = &ctl->err;
+  a.stats = ctl->stats;
+  a.flags = 0;
+  a.debug_out = ctl->debug;
+  if (e == cudaSuccess && strict_to) {
+    a.counter = &ctl->counter[1];
+    a.lay = strict_lay;
+    a.nslots = strict_slots;
     a.width = cfg.bucket_width ? cfg.bucket_width : 64;
-    a.width_dev = kind == SLAB_STRICT ? nullptr : &ctl->width;
     a.settle_in = cfg.settle_in == 2 ? 0u : 1u;
-    a.phase_cap = cfg.phase_cap ? cfg.phase_cap : 4ull * n + 64;  // phases + refills <= 4n + 2
-    a.err = &ctl->err;
-    a.stats = ctl->stats;
-    a.flags = 0;
-    a.debug_out = ctl->debug;
     a.warp_deg = cfg.warp_degree ? cfg.warp_degree : 32u;
     a.team_deg = std::max<uint32_t>(cfg.team_degree ? cfg.team_degree : 8u * team, a.warp_deg);
-    const int grid = (int)((slots + per_block - 1) / per_block);
-    e = kind == SLAB_STRICT ? launch_batched(a, 64, team, grid, st) : launch_sweep(a, plan, grid, st);
+    if (!fill_early) e = init_slabs(slabs, strict_lay, SLAB_STRICT, strict_slots, n, 64, st, a.counter);
+    if (e == cudaSuccess) e = launch_batched(a, 64, team, strict_grid, st);
+  }
+  if (e == cudaSuccess && sweep) {
+    a.counter = &ctl->counter[0];
+    a.lay = lay;
+    a.nslots = slots;
+    a.width_dev = &ctl->width;
+    e = init_slabs(slabs, lay, kind, slots, n, 64, st, strict_to ? a.counter : nullptr);
+    if (e == cudaSuccess) e = launch_sweep(a, plan, grid, st);
   }
   if (e == cudaSuccess && scale != 1.0) e = launch_scale(d_out_bc, n, scale, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_status, &ctl->err, sizeof(int), cudaMemcpyDeviceToDevice, st);

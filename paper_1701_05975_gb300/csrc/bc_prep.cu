@@ -85,7 +85,8 @@ __global__ void check_sources_kernel(const uint32_t* src, uint32_t k, uint32_t n
 }
 
 __global__ void fill_slabs_kernel(char* base, uint64_t stride, uint32_t nslots, uint64_t off, uint64_t words,
-                                  uint32_t value) {
+                                  uint32_t value, const uint32_t* gate) {
+  if (gate && *gate >= PARKED) return;
   for (uint32_t slot = blockIdx.y; slot < nslots; slot += gridDim.y) {
     uint32_t* p = reinterpret_cast<uint32_t*>(base + (uint64_t)slot * stride + off);
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < words; i += (uint64_t)gridDim.x * blockDim.x)
@@ -135,11 +136,11 @@ cudaError_t launch_check_sources(const uint32_t* src, uint32_t k, uint32_t n, in
 }
 
 cudaError_t launch_fill_slabs(char* base, uint64_t stride, uint32_t nslots, uint64_t off, uint64_t bytes,
-                              uint32_t value, cudaStream_t st) {
+                              uint32_t value, cudaStream_t st, const uint32_t* gate) {
   if (nslots == 0 || bytes == 0) return cudaSuccess;
   const uint64_t words = bytes / 4;
   dim3 grid((unsigned)std::min<uint64_t>((words + 255) / 256, 64), std::min<uint32_t>(nslots, 65535));
-  fill_slabs_kernel<<<grid, 256, 0, st>>>(base, stride, nslots, off, words, value);
+  fill_slabs_kernel<<<grid, 256, 0, st>>>(base, stride, nslots, off, words, value, gate);
   return cudaGetLastError();
 }
 

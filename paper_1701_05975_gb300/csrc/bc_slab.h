@@ -100,17 +100,18 @@ inline SlabLayout make_layout(uint32_t n, int dist_bits, SlabKind kind) {
 // accumulators (strict) or vertex records and bits (sweep) zero; other arrays are
 // written before they are read.
 inline cudaError_t init_slabs(char* slabs, const SlabLayout& lay, SlabKind kind, uint32_t slots, uint32_t n, int dist_bits,
-                       cudaStream_t st) {
+                       cudaStream_t st, const uint32_t* gate = nullptr) {
   if (kind == SLAB_NONE) return cudaSuccess;
   cudaError_t e = launch_fill_slabs(slabs, lay.stride, slots, lay.off_d, align256((uint64_t)n * (dist_bits / 8)),
-                                    0xffffffffu, st);
+                                    0xffffffffu, st, gate);
   if (e != cudaSuccess) return e;
   if (kind == SLAB_SWEEP) {
-    e = launch_fill_slabs(slabs, lay.stride, slots, lay.off_sig, align256((uint64_t)n * 16), 0u, st);
+    e = launch_fill_slabs(slabs, lay.stride, slots, lay.off_sig, align256((uint64_t)n * 16), 0u, st, gate);
     if (e != cudaSuccess) return e;
-    return launch_fill_slabs(slabs, lay.stride, slots, lay.off_pend, align256((((uint64_t)n + 31) / 32) * 8), 0u, st);
+    return launch_fill_slabs(slabs, lay.stride, slots, lay.off_pend, align256((((uint64_t)n + 31) / 32) * 8), 0u, st,
+                             gate);
   }
-  return launch_fill_slabs(slabs, lay.stride, slots, lay.off_acc, align256((uint64_t)n * 8), 0u, st);
+  return launch_fill_slabs(slabs, lay.stride, slots, lay.off_acc, align256((uint64_t)n * 8), 0u, st, gate);
 }
 
 // Teams of `team` threads that an SM holds: by the registers the kernels are

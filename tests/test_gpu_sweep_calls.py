@@ -215,3 +215,26 @@ def test_small_weights_take_the_strict_schedule(graph, k, strict):
         bc.bc_set_config(algorithm=bc.BC_ALGO_DELTA)
         assert_bc_close(G.compute(src, 0.5), want)
         assert G.stats().algorithm == bc.BC_ALGO_DELTA
+
+
+def test_noalloc_schedule_by_the_largest_weight():
+    """Weights on both sides of the lines where the call changes schedules, over all and over a few sources,
+    one call after the other on the same scratch array."""
+    torch = pytest.importorskip("torch")
+    dev = lambda x, t: torch.from_numpy(np.ascontiguousarray(x).view(t)).cuda()  # noqa: E731
+    calls = [(1024, 8, w, k) for w in (1, 15, 17, 31, 33, 100) for k in (1024, 50)]
+    calls += [(400, 8, w, 400) for w in (16, 17)] + [(1537, 4, w, k) for w in (15, 16, 17) for k in (700, 90)]
+    calls += [(2000, 16, w, 64) for w in (1, 126, 130)] + [(900, 2, w, 900) for w in (4, 5)] + [(5, 1, 1, 5)]
+    for n, per, wmax, k in calls:
+        g = gen.er_graph(n, per * n, 1, wmax, seed=n + wmax)
+        g.w[g.w == g.w.max()] = wmax  # both entries of an edge
+        src = np.arange(k, dtype=np.uint32)
+        rp, col, w, d_src = dev(g.row_ptr, np.int64), dev(g.col, np.int32), dev(g.w, np.int32), dev(src, np.int32)
+        out = torch.empty(n, dtype=torch.float64, device="cuda")
+        status = torch.full((1,), 9, dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        bc.bc_compute_noalloc(rp.data_ptr(), col.data_ptr(), w.data_ptr(), n, g.nnz, d_src.data_ptr(), k, 0.5,
+                              out.data_ptr(), status.data_ptr(), 0)
+        torch.cuda.synchronize()
+        assert int(status.item()) == bc.BC_OK, (n, per, wmax, k)
+        assert_bc_close(out.cpu().numpy(), oracle.bc(g, src, 0.5, nthreads=8))
