@@ -126,6 +126,7 @@ struct bc_graph {
   double* ebc = nullptr;  // lazily allocated [nnz]
   bool relabeled = false;
   bool directed = false;
+  bool symmetric = true;  // directed graphs: nothing is asked of them
   uint64_t* in_row_ptr = nullptr;  // directed graphs: in-edge CSR (same entry form)
   uint2* in_adj = nullptr;
   uint32_t* in_adjp = nullptr;
@@ -232,7 +233,7 @@ bool sweep_sparse(const bc_graph* g) { return !g->kadj && (double)g->nnz < 6.0 *
 // in a second wave of slabs at 1296; Barabasi-Albert 1500 with 2 edges a vertex 667 and 471
 // at 1216; 30 x 30 grid 650 and 690 at 900).
 bool sweep_in_smem(const bc_graph* g, uint32_t k) {
-  if (g->n > SWEEP_SMEM_N) return false;
+  if (g->n > SWEEP_SMEM_N || !g->symmetric) return false;
   if (!g->kadj && g->n >= 400 && g->nnz >= 24ull * g->n) return false;
   if (!sweep_sparse(g) || g->dist_bits != 32) return true;
   if (k <= 4ull * g->sm_count || k > 8ull * g->sm_count) return true;
@@ -248,6 +249,11 @@ void plan_sweep(const bc_graph* g, RunCfg& r, uint32_t k, bool allow_smem) {
   const double avg_deg = g->n ? (double)g->nnz / g->n : 0.0;
   p.group = (!p.prune && avg_deg >= 12.0) ? 8 : 1;
   sweep_place(p, g->n, g->act_n, allow_smem && sweep_in_smem(g, k));
+  if (!g->symmetric) {
+    p.mem = 3;
+    p.group = 1;
+    p.smem_bytes = 0;
+  }
   r.sweep = p;
 }
 
@@ -317,7 +323,7 @@ uint32_t strict_team_default(const bc_graph* g) {
 //   sparse graphs, not probed: grids 0.71 and 0.96 at weights to 1 and 2 (n = 900), 0.76 / 0.83
 //   / 0.90 / 1.01 at weights to 1 / 2 / 3 / 5 (n = 40,000, 1216 sources), 1.5 and more at 304.
 bool strict_is_faster(const bc_graph* g, uint32_t k) {
-  if (g->kadj) return false;
+  if (g->kadj || !g->symmetric) return false;
   const double walked = (double)g->nnz * (g->directed ? 2.0 : 1.0) / g->n;
   const bool few = k && k <= (uint32_t)g->sm_count;
   if (g->ties < 0.0) {
@@ -398,7 +404,7 @@ int plan_slots(const bc_graph* g, RunCfg& r, uint32_t k, uint32_t* slots_out) {
   CK(cudaMemGetInfo(&free_b, &total_b));
   const uint64_t budget = (uint64_t)((double)free_b * r.mem_fraction);
   uint64_t stride = make_layout(g->n, g->dist_bits, slab_kind(r)).stride;
-  if (stride > budget && r.algo == ALGO_DELTA && r.algo_auto) {
+  if (stride > budget && r.algo == ALGO_DELTA && r.algo_auto && g->symmetric) {
     r = resolve(g, k, BC_ALGO_STRICT);
     stride = make_layout(g->n, g->dist_bits, SLAB_STRICT).stride;
   }
@@ -653,7 +659,8 @@ int status_from_dev(int dev) {
   if (dev == DEV_OK) return BC_OK;
   if (dev == DEV_ERR_TIMEOUT) return fail(BC_ERR_TIMEOUT, "device phase cap reached (BC_ERR_TIMEOUT)");
   if (dev == DEV_ERR_INVALID) return fail(BC_ERR_INVALID, "a source is out of range");
-  if (dev == DEV_ERR_INTERNAL) return fail(BC_ERR_CUDA, "device consistency check failed (DAG levels do not cover the reached set)");
+  if (dev == DEV_ERR_INTERNAL)
+    return fail(BC_ERR_CUDA, "device consistency check failed (an undirected graph whose entries lack their reverses)");
   return fail(BC_ERR_CUDA, "unknown device status %d", dev);
 }
 
@@ -884,7 +891,7 @@ constexpr uint32_t LAND_MAX_N_FLAT = 32768;
 
 cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<uint64_t>& tdeg) {
   const uint32_t n = g->n;
-  if (g->dist_bits != 32 || n < LAND_MIN_N || g->nnz == 0) return cudaSuccess;
+  if (g->dist_bits != 32 || n < LAND_MIN_N || g->nnz == 0 || !g->symmetric) return cudaSuccess;
   // without hubs the bounds only help small graphs (the prefix test keeps 28% of
   // the entries of a degree-16 random graph at n = 1024, 62% at 262144, all of a
   // grid's): do not pay for 68 searches to find that out
@@ -939,7 +946,7 @@ cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<u
   uint32_t* d_ids = static_cast<uint32_t*>(alloc(k * 4ull));
   uint32_t* tab = static_cast<uint32_t*>(alloc(dist_bytes));
   uint32_t* tab_in = g->directed ? static_cast<uint32_t*>(alloc((uint64_t)L * n * 4)) : tab;
-  // one control block per launch, then the symmetry sums, the judge's sums and the largest distance
+  // one control block per launch, then the judge's sums and the largest distance
   Ctl* ctl = static_cast<Ctl*>(alloc(2 * sizeof(Ctl) + 8 * 8));
   auto done = [&](cudaError_t err) {
     for (void* p : temp) cudaFree(p);
@@ -976,29 +983,28 @@ cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<u
     rev.adj = g->in_adj;
     e = distances(rev, L, tab_in, ctl + 1);
   }
-  if (e == cudaSuccess && !g->directed) e = land_symmetry(fwd, sums, st);
-  if (e == cudaSuccess) e = land_judge(fwd, tab, tab + (uint64_t)L * n, h, probes, sums + 2, st);
-  if (e == cudaSuccess) e = land_max((uint64_t)L * n, tab, reinterpret_cast<uint32_t*>(sums + 6), st);
+  if (e == cudaSuccess) e = land_judge(fwd, tab, tab + (uint64_t)L * n, h, probes, sums, st);
+  if (e == cudaSuccess) e = land_max((uint64_t)L * n, tab, reinterpret_cast<uint32_t*>(sums + 4), st);
   if (e == cudaSuccess && g->directed)
-    e = land_max((uint64_t)L * n, tab_in, reinterpret_cast<uint32_t*>(sums + 6), st);
+    e = land_max((uint64_t)L * n, tab_in, reinterpret_cast<uint32_t*>(sums + 4), st);
   std::vector<unsigned char> host(2 * sizeof(Ctl) + 8 * 8);
   if (e == cudaSuccess) e = cudaMemcpyAsync(host.data(), ctl, host.size(), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return done(e);
-  unsigned long long hs[7];
+  unsigned long long hs[5];
   memcpy(hs, host.data() + 2 * sizeof(Ctl), sizeof hs);
   const Ctl* hc = reinterpret_cast<const Ctl*>(host.data());
-  const uint32_t max_d = (uint32_t)hs[6];
-  if (hc[0].err != DEV_OK || hc[1].err != DEV_OK || hs[0] != hs[1]) return done(cudaSuccess);
-  g->ties = (double)hs[5] / ((double)probes * n);
+  const uint32_t max_d = (uint32_t)hs[4];
+  if (hc[0].err != DEV_OK || hc[1].err != DEV_OK) return done(cudaSuccess);
+  g->ties = (double)hs[3] / ((double)probes * n);
   const bool dense = !g->relabeled && n > SWEEP_SMEM_N && g->nnz >= 24ull * n;
   const double keep_max = dense ? LAND_KEEP_MAX_DENSE : LAND_KEEP_MAX;
-  if (hs[2] == 0 || (double)hs[3] > keep_max * (double)hs[2]) return done(cudaSuccess);
+  if (hs[0] == 0 || (double)hs[1] > keep_max * (double)hs[0]) return done(cudaSuccess);
 
   g->land_bits = max_d < 0x3fffu ? 16 : 32;  // every sum of two distances below 0x7fff
   g->land_stride = ((uint64_t)n + 7) & ~7ull;
   g->nland = L;
-  g->land_n = g->directed ? g->act_n : (uint32_t)hs[4];
+  g->land_n = g->directed ? g->act_n : (uint32_t)hs[2];
   const uint64_t tab_bytes = g->land_stride * L * (g->land_bits / 8);
   unsigned long long* key = static_cast<unsigned long long*>(alloc(g->nnz * 8));
   if (!key) return done(cudaErrorMemoryAllocation);
@@ -1041,7 +1047,7 @@ void bcgpu::graph_serving_ref(bc_graph* g, int delta) { g->serving_refs += delta
 int bcgpu::serve_plan(bc_graph* g, uint32_t k, uint64_t budget, ServePlan* out) {
   RunCfg r = resolve(g, k);
   out->fixed_bytes = (uint64_t)g->n * 16 + 4096;
-  if (r.algo == ALGO_DELTA && r.algo_auto &&
+  if (r.algo == ALGO_DELTA && r.algo_auto && g->symmetric &&
       make_layout(g->n, g->dist_bits, slab_kind(r)).stride + out->fixed_bytes > budget)
     r = resolve(g, k, BC_ALGO_STRICT);
   r.mode = BC_MODE_BATCHED;
@@ -1312,7 +1318,7 @@ int bc_graph_create(const uint64_t* row_ptr, const uint32_t* col_idx, const uint
     if (e == cudaSuccess) e = cudaMalloc(&g->dnode2, (size_t)n * 4);
     if (e == cudaSuccess) e = cudaMalloc(&g->dnode_arg, (size_t)n * 4);
   }
-  if (e == cudaSuccess) e = cudaMalloc(&d_col, std::max<size_t>(nnz, 1) * 4);
+  if (e == cudaSuccess) e = cudaMalloc(&d_col, std::max<size_t>(nnz, 4) * 4);
   if (e == cudaSuccess) e = cudaMalloc(&d_w, std::max<size_t>(nnz, 1) * 4);
   if (e == cudaSuccess) e = cudaMemcpyAsync(g->row_ptr, row_ptr, ((size_t)n + 1) * 8, cudaMemcpyHostToDevice, g->stream);
   if (e == cudaSuccess && nnz) e = cudaMemcpyAsync(d_col, col_idx, nnz * 4, cudaMemcpyHostToDevice, g->stream);
@@ -1330,6 +1336,14 @@ int bc_graph_create(const uint64_t* row_ptr, const uint32_t* col_idx, const uint
   if (e == cudaSuccess)
     e = launch_prep(n, nnz, g->row_ptr, d_col, d_w, g->adj, g->dnode, g->dnode2, g->dnode_arg, g->stream);
   if (e == cudaSuccess && packed) e = launch_pack32(nnz, d_col, d_w, col_bits, g->adjp, g->stream);
+  unsigned long long sums[2] = {0, 0};
+  if (!directed && e == cudaSuccess) {
+    // the schedules rely on undirected rows being symmetric: known once, by hash
+    unsigned long long* d_sums = reinterpret_cast<unsigned long long*>(d_col);  // both temporaries are free again
+    e = cudaMemsetAsync(d_sums, 0, sizeof sums, g->stream);
+    if (e == cudaSuccess) e = land_symmetry(view(g.get()), d_sums, g->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(sums, d_sums, sizeof sums, cudaMemcpyDeviceToHost, g->stream);
+  }
   if (directed && e == cudaSuccess) {
     // same entry form for the in-edge CSR; d_col / d_w are reused for it
     g->directed = true;
@@ -1348,6 +1362,7 @@ int bc_graph_create(const uint64_t* row_ptr, const uint32_t* col_idx, const uint
     if (e == cudaSuccess && packed) e = launch_pack32(nnz, d_col, d_w, col_bits, g->in_adjp, g->stream);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+  g->symmetric = sums[0] == sums[1];
   cudaFree(d_col);
   cudaFree(d_w);
   if (e == cudaSuccess) e = build_landmarks(g.get(), row_ptr, tdeg);
@@ -1720,8 +1735,9 @@ int autotune(bc_graph* g, const uint32_t* sources, uint32_t k_probe) {
   // a pinned schedule, or a knob that only the strict one has, leaves one schedule
   const bool strict_knob = user.settle_in || user.warp_degree || user.team_degree || user.hot_vertices ||
                            (user.bucket_width && user.algorithm != BC_ALGO_DELTA);
-  const bool try_sweep = user.algorithm == BC_ALGO_DELTA || (user.algorithm == BC_ALGO_AUTO && !strict_knob);
-  const bool try_strict = user.algorithm != BC_ALGO_DELTA;
+  const bool try_sweep =
+      user.algorithm == BC_ALGO_DELTA || (user.algorithm == BC_ALGO_AUTO && (!strict_knob || !g->symmetric));
+  const bool try_strict = user.algorithm == BC_ALGO_STRICT || (user.algorithm == BC_ALGO_AUTO && g->symmetric);
   // sweep schedule: team size x bucket width (one bucket under landmark
   // bounds), then sources in flight
   double sweep_ms = 1e300;

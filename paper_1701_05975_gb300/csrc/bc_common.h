@@ -167,7 +167,8 @@ struct SweepPlan {
   int dist_bits = 32;
   int team = 256;
   bool prune = false;   // rows in landmark order (kadj)
-  int mem = 0;          // 0: slab, 1: slab with the vertex bits in shared memory, 2: all in shared memory
+  int mem = 0;          // 0: slab, 1: slab with the vertex bits in shared memory, 2: all in shared memory,
+                        // 3: slab, every source's rows checked against their reverses
   int group = 1;        // threads per row: 1 or 8
   uint32_t smem_bytes = 0;
 };
@@ -186,6 +187,8 @@ cudaError_t sweep64_full1_global(const SweepPlan& p, const BatchArgs* a, int gri
 cudaError_t sweep64_full8_global(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
 cudaError_t sweep64_full1_bits(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
 cudaError_t sweep64_full8_bits(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep32_check(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
+cudaError_t sweep64_check(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
 cudaError_t sweep64_full1_all(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ);
 
 // Settings of one batched run.

@@ -13,7 +13,8 @@ cudaError_t dispatch(const SweepPlan& p, const BatchArgs* a, int grid, cudaStrea
   static const Fn wide32[3] = {sweep32_full8_global, sweep32_full8_bits, sweep32_full1_all};
   static const Fn full64[3] = {sweep64_full1_global, sweep64_full1_bits, sweep64_full1_all};
   static const Fn wide64[3] = {sweep64_full8_global, sweep64_full8_bits, sweep64_full1_all};
-  if (p.mem < 0 || p.mem > 2) return cudaErrorInvalidValue;
+  if (p.mem == 3) return p.dist_bits == 32 ? sweep32_check(p, a, grid, st, occ) : sweep64_check(p, a, grid, st, occ);
+  if (p.mem < 0 || p.mem > 3) return cudaErrorInvalidValue;
   const Fn* row = p.dist_bits == 32 ? (p.prune ? prune32 : (p.group == 8 ? wide32 : full32))
                                     : (p.group == 8 ? wide64 : full64);
   return row[p.mem](p, a, grid, st, occ);

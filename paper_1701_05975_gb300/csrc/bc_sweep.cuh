@@ -86,6 +86,7 @@ enum : int {
   MEM_GLOBAL = 0,  // the slab
   MEM_BITS = 1,    // the slab, the two bits per vertex in shared memory
   MEM_ALL = 2,     // shared memory
+  MEM_CHECK = 3,   // the slab; an undirected graph whose rows are not symmetric: every source is checked
 };
 
 // Per-vertex record, one 32-byte sector holds two.  Sigma pass: aux's low
@@ -117,6 +118,7 @@ template <typename D, int TEAM, bool PRUNE, int MEM, int G>
 struct SweepTeam {
   using Sh = SweepShared<D, TEAM>;
   static constexpr bool SM = MEM == MEM_ALL;
+  static constexpr bool CHECK = MEM == MEM_CHECK;
   using Idx = typename std::conditional<SM, uint16_t, uint32_t>::type;
   static constexpr int NW = TEAM / 32;
   static constexpr uint32_t FIRST = 4;  // entries that one thread walks before its warp helps
@@ -162,7 +164,7 @@ struct SweepTeam {
   static __device__ __forceinline__ uint32_t* count_of(SweepNode* p) { return reinterpret_cast<uint32_t*>(p) + 2; }
 
   static __device__ __forceinline__ uint32_t ld_bits(const uint32_t* p) {
-    if constexpr (MEM == MEM_GLOBAL) return ldcg(p);
+    if constexpr (MEM == MEM_GLOBAL || CHECK) return ldcg(p);
     else return *reinterpret_cast<const volatile uint32_t*>(p);
   }
   static __device__ __forceinline__ bool test_bit(const uint32_t* b, uint32_t v) {
@@ -878,6 +880,45 @@ struct SweepTeam {
     return total ? start : 0u;
   }
 
+  // 32-bit finaliser of MurmurHash3 (A. Appleby, public domain).
+  static __device__ __forceinline__ uint32_t hash(uint32_t x) {
+    x = (x ^ (x >> 16)) * 0x85ebca6bu;
+    x = (x ^ (x >> 13)) * 0xc2b2ae35u;
+    return x ^ (x >> 16);
+  }
+  // Whether every reached vertex has as many predecessors by its own row
+  // (d(u) + w = d(v)) as by theirs (the DAG): the sums of a hash of each DAG edge's
+  // target, taken both ways.  An entry on a shortest path without a reverse
+  // entry makes them differ.  Ends synchronised.
+  __device__ bool rows_agree() {
+    const D INF = dinf<D>();
+    if (t == 0) sh.tpos = 0;
+    team_sync<TEAM>();
+    uint32_t sum = 0;
+    walk(reached_count(),
+         [&](uint32_t i) {
+           const uint32_t v = reached_vertex(i);
+           return ld(&d[v]) == INF ? NONE : v;
+         },
+         [&](uint32_t v, const Row& r, auto& ok, auto& x, auto& du, uint32_t, uint32_t) {
+           constexpr int N = sizeof(ok) / sizeof(ok[0]);
+#pragma unroll
+           for (int q = 0; q < N; ++q) {
+             if (!ok[q] || du[q] == INF) continue;
+             if (du[q] == r.dv + (D)x[q].y) sum += hash(x[q].x);
+             if (du[q] + (D)x[q].y == r.dv) sum -= hash(v);
+           }
+         });
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(FULL, sum, o);
+    if ((t & 31) == 0) atomicAdd(&sh.tpos, sum);
+    team_sync<TEAM>();
+    const bool agree = sh.tpos == 0;
+    team_sync<TEAM>();
+    return agree;
+  }
+
   // Replace the listed successors that have no successor themselves and one
   // predecessor by a count; then fold, a few times over: a vertex with one
   // predecessor whose successors are all counted has its dependency (the
@@ -1470,16 +1511,19 @@ struct SweepTeam {
       build_dag();
       team_sync<TEAM>();
       over = sh.dag_over != 0;
+      if constexpr (CHECK) {
+        if (!rows_agree()) err = DEV_ERR_INTERNAL;
+      }
       const bool all = over || (a.flags & RUN_FORWARD_ONLY);
-      const bool drop = !all;
-      every = all;
+      const bool drop = !all && (!CHECK || err == DEV_OK);
+      every = !drop;
       if (drop) {
         drop_leaves(rounds < SW_DEEP ? SW_FOLDS : 0);
       } else {
         clear_bits0();
       }
       lap(0);
-      nlev = sigma_levels(qa, qb, over, all, drop, rounds < SW_DEEP);
+      if (!CHECK || err == DEV_OK) nlev = sigma_levels(qa, qb, over, all, drop, rounds < SW_DEEP);
       lap(2);
       if (a.phase_cap < (uint64_t)rounds + advances + nlev) err = DEV_ERR_TIMEOUT;
       if (a.flags & RUN_FORWARD_ONLY) {
@@ -1555,8 +1599,8 @@ __host__ __device__ constexpr int sweep_min_blocks() {
 template <typename D, int TEAM, int BLOCK, bool PRUNE, int MEM, int G>
 __global__ void __launch_bounds__(BLOCK, (sweep_min_blocks<D, TEAM, BLOCK>())) bc_sweep_kernel(const BatchArgs a) {
   static_assert(TEAM == 32 || TEAM == BLOCK, "a CTA holds either warp teams or one team");
-  static_assert(MEM == MEM_GLOBAL || TEAM == BLOCK, "the shared-memory forms hold one team per CTA");
-  constexpr bool SM = MEM == MEM_ALL;
+  constexpr bool SM = MEM == MEM_ALL, SMEM = SM || MEM == MEM_BITS;
+  static_assert(!SMEM || TEAM == BLOCK, "the shared-memory forms hold one team per CTA");
   constexpr int NTEAMS = BLOCK / TEAM;
   __shared__ SweepShared<D, TEAM> shared_teams[NTEAMS];
   extern __shared__ __align__(16) unsigned char sweep_arrays[];
@@ -1592,7 +1636,7 @@ __global__ void __launch_bounds__(BLOCK, (sweep_min_blocks<D, TEAM, BLOCK>())) b
     for (uint32_t v = t; v < a.g.n; v += TEAM) w.node[v] = zero;
     w.fill_distances();
   }
-  if constexpr (MEM != MEM_GLOBAL)
+  if constexpr (SMEM)
     for (uint32_t i = t; i < 2 * words; i += TEAM) w.bits0[i] = 0;
   team_sync<TEAM>();
   for (;;) {
@@ -1622,7 +1666,7 @@ cudaError_t sweep_one(const SweepPlan& p, const BatchArgs* a, int grid, cudaStre
     k<<<grid, BLOCK, p.smem_bytes, st>>>(*a);
     return cudaGetLastError();
   }
-  if (MEM != MEM_GLOBAL) {
+  if (MEM == MEM_ALL || MEM == MEM_BITS) {
     // always the device's limit, so plans of different sizes (and threads) do not disturb each other
     int dev = 0, optin = 0;
     cudaFuncAttributes fa{};
@@ -1640,7 +1684,7 @@ template <typename D, bool PRUNE, int MEM, int G>
 cudaError_t sweep_team(const SweepPlan& p, const BatchArgs* a, int grid, cudaStream_t st, int* occ) {
   switch (p.team) {
     case 32:
-      if constexpr (MEM == MEM_GLOBAL) return sweep_one<D, 32, 256, PRUNE, MEM, G>(p, a, grid, st, occ);
+      if constexpr (MEM == MEM_GLOBAL || MEM == MEM_CHECK) return sweep_one<D, 32, 256, PRUNE, MEM, G>(p, a, grid, st, occ);
       return cudaErrorInvalidValue;
     case 128: return sweep_one<D, 128, 128, PRUNE, MEM, G>(p, a, grid, st, occ);
     case 256: return sweep_one<D, 256, 256, PRUNE, MEM, G>(p, a, grid, st, occ);

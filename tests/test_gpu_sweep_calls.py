@@ -238,3 +238,70 @@ def test_noalloc_schedule_by_the_largest_weight():
         torch.cuda.synchronize()
         assert int(status.item()) == bc.BC_OK, (n, per, wmax, k)
         assert_bc_close(out.cpu().numpy(), oracle.bc(g, src, 0.5, nthreads=8))
+
+
+def csr(n, rows):
+    """CSR from {vertex: [(neighbour, weight), ...]}, as given: nothing is made symmetric."""
+    deg = np.zeros(n + 1, np.uint64)
+    for v, r in rows.items():
+        deg[v + 1] = len(r)
+    ent = [e for v in sorted(rows) for e in rows[v]]
+    return gen.CSRGraph(n=n, row_ptr=np.cumsum(deg).astype(np.uint64), col=np.array([e[0] for e in ent], np.uint32),
+                        w=np.array([e[1] for e in ent], np.uint32), name="csr")
+
+
+def one_way(base, extra, n=None):
+    """The symmetric graph `base` with the one-directional entries (v, u, w) added."""
+    rows = {}
+    for u, v, w in zip(*(x.tolist() for x in base.edges())):
+        rows.setdefault(u, []).append((v, w))
+    for v, u, w in extra:
+        rows[v] = sorted(rows.get(v, []) + [(u, w)])
+    return csr(n or base.n, rows)
+
+
+@pytest.mark.parametrize("team", [0, 32, 128, 512])
+@pytest.mark.parametrize("bits", [32, 64])
+def test_undirected_rows_without_their_reverses_are_an_error(team, bits):
+    """An entry that lies on a shortest path from a source and has no reverse entry: BC_ERR_CUDA on every
+    entry point.  Sources that it does not concern are computed, before and after, as is a graph whose
+    one-directional entries lie on no shortest path."""
+    torch = pytest.importorskip("torch")
+    wmax = 1 << 27 if bits == 64 else 50
+    base = gen.er_graph(300, 1200, 1, wmax, seed=5)
+    whole = gen.csr_from_undirected(420, *(x[base.edges()[0] < base.edges()[1]] for x in base.edges()))
+    free = np.arange(0, 300, 7, dtype=np.uint32)
+    bc.bc_set_config(team_threads=team)
+    # 310 -> 419: a target without a row and with the highest id; 320 -> 321 -> 322, one way each
+    broken = one_way(whole, [(310, 419, 3), (320, 321, 2), (321, 322, 2), (330, 331, 5), (331, 330, 6)])
+    heavy = one_way(whole, [(0, 1, 4_000_000_000 if bits == 64 else 1_000_000)])
+    with bc.Graph(broken) as G, bc.Graph(heavy) as H:
+        assert G.info().dist_bits == bits
+        for pinned in (bc.BC_ALGO_AUTO, bc.BC_ALGO_DELTA):
+            bc.bc_set_config(algorithm=pinned)
+            for bad in (310, 320, 330):
+                src = np.array([5, bad, 9], np.uint32)
+                assert_bc_close(G.compute(free, 0.5), oracle.bc(whole, free, 0.5))
+                calls = [lambda: G.compute(src, 0.5), lambda: G.edge_compute(src, 0.5), lambda: G.submit(src, 0.5).result(60000)]
+                for call in calls:
+                    with pytest.raises(bc.BCError) as ei:
+                        call()
+                    assert ei.value.code == bc.BC_ERR_CUDA
+            d_src, out = torch.tensor([330], dtype=torch.int32, device="cuda"), torch.empty(420, dtype=torch.float64, device="cuda")
+            s = torch.cuda.Stream()
+            s.wait_stream(torch.cuda.current_stream())
+            G.compute_async(d_src, out, 0.5, stream=s)
+            with pytest.raises(bc.BCError) as ei:
+                G.sync(s)
+            assert ei.value.code == bc.BC_ERR_CUDA
+            assert_bc_close(G.compute(free, 0.5), oracle.bc(whole, free, 0.5))
+            assert G.stats().algorithm == bc.BC_ALGO_DELTA
+            ebc, vbc = G.edge_compute(np.array([331 - 300, 6], np.uint32), 0.5)
+            assert_bc_close(vbc, oracle.bc(whole, np.array([31, 6], np.uint32), 0.5))
+            assert_bc_close(H.compute(free, 0.5), oracle.bc(whole, free, 0.5))
+        with pytest.raises(bc.BCError) as ei:
+            G.sssp_debug(320)
+        assert ei.value.code == bc.BC_ERR_CUDA
+        d, sig, _ = G.sssp_debug(8)
+        want = oracle.sssp(whole, 8)
+        assert np.array_equal(d, want[0]) and np.array_equal(sig, want[1])
