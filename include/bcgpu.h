@@ -304,7 +304,7 @@ typedef struct bc_run_stats {
   uint32_t team_threads;
   uint32_t slots;
   uint64_t bucket_width;
-  uint64_t dag_edges;       /* shortest-path DAG edges recorded by the forward pass (BC_ALGO_DELTA: list words) */
+  uint64_t dag_edges;       /* shortest-path DAG edges recorded by the forward pass */
   uint64_t pair_overflows;  /* sources whose DAG edge list overflowed (backward fell back to a CSR scan) */
   uint64_t cycles_expand;   /* SM cycles summed over sources: frontier expansion (sigma pull + relax) */
   uint64_t cycles_refill;   /* near-queue refills from the far queue (BC_ALGO_DELTA: landmark bounds, DAG lists) */

@@ -104,7 +104,7 @@ struct SweepShared {
   uint32_t nwide[3];  // rows left to whole warps
   uint32_t nteam[3];  // rows left to the whole team
   uint32_t tpos;
-  uint32_t S_len, def_len, ndef, dag_len, dag_over, nkeep, nfold;
+  uint32_t S_len, def_len, ndef, dag_len, dag_lists, dag_over, nkeep, nfold;
   unsigned long long cyc[4];
   long long tmark;
   uint32_t team_v[SW_TEAM_CAP], team_e[SW_TEAM_CAP];
@@ -751,7 +751,11 @@ struct SweepTeam {
       const uint32_t inc = warp_incl_scan(c + head);
       uint32_t start = 0;
       const uint32_t wsum = __shfl_sync(FULL, inc, 31);
-      if (lane == 31 && wsum) start = atomicAdd(&sh.dag_len, wsum);
+      const uint32_t has = __ballot_sync(FULL, head != 0);
+      if (lane == 31 && wsum) {
+        start = atomicAdd(&sh.dag_len, wsum);
+        atomicAdd(&sh.dag_lists, __popc(has));
+      }
       start = __shfl_sync(FULL, start, 31);
       const bool fits = start + wsum <= succ_cap;
       if (!fits && lane == 0 && wsum) sh.dag_over = 1;
@@ -761,10 +765,7 @@ struct SweepTeam {
         succ[pos] = total;
         succ[pos + 1] = 0;
       }
-      if (G == 1 && stream) {
-        const uint32_t has = __ballot_sync(FULL, head != 0);
-        if (lane == 0 && i < len) bits2[i >> 5] = has;
-      }
+      if (G == 1 && stream && lane == 0 && i < len) bits2[i >> 5] = has;
       pos += head;
       while (__any_sync(FULL, mask != 0)) {
         uint32_t e[SW_UNR], u[SW_UNR];
@@ -867,6 +868,7 @@ struct SweepTeam {
   }
   // One thread: v's list of `total` successors at `start`; 0 when it has none or does not fit.
   __device__ __forceinline__ uint32_t list_head(uint32_t v, uint32_t start, uint32_t total) {
+    if (total) atomicAdd(&sh.dag_lists, 1u);
     if (total && start + total + SW_HEAD > succ_cap) {
       sh.dag_over = 1;
       total = 0;
@@ -1487,6 +1489,7 @@ struct SweepTeam {
       sh.S_len = seeded ? 0u : 1u;
       sh.def_len = 0;
       sh.dag_len = 1;  // offset 0 means no list
+      sh.dag_lists = 0;
       sh.dag_over = 0;
       sh.cyc[0] = sh.cyc[1] = sh.cyc[2] = sh.cyc[3] = 0;
       sh.tmark = clock64();
@@ -1575,7 +1578,7 @@ struct SweepTeam {
         atomicAdd(&a.stats[STAT_SOURCES], 1ull);
         atomicAdd(&a.stats[STAT_PHASES], (unsigned long long)rounds);
         atomicAdd(&a.stats[STAT_REFILLS], (unsigned long long)advances);
-        atomicAdd(&a.stats[STAT_DAG_EDGES], (unsigned long long)(sh.dag_len - 1));
+        atomicAdd(&a.stats[STAT_DAG_EDGES], (unsigned long long)(sh.dag_len - 1 - SW_HEAD * sh.dag_lists));
         atomicAdd(&a.stats[STAT_LEVELS], (unsigned long long)nlev);
         atomicAdd(&a.stats[STAT_PAIR_OVERFLOW], (unsigned long long)(over ? 1 : 0));
         atomicAdd(&a.stats[STAT_CYC_EXPAND], sh.cyc[1]);

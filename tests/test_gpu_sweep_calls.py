@@ -305,3 +305,28 @@ def test_undirected_rows_without_their_reverses_are_an_error(team, bits):
         d, sig, _ = G.sssp_debug(8)
         want = oracle.sssp(whole, 8)
         assert np.array_equal(d, want[0]) and np.array_equal(sig, want[1])
+
+
+@pytest.mark.parametrize("graph", [
+    lambda: gen.er_graph(700, 5600, 1, 60, seed=1),
+    lambda: gen.er_graph(700, 5600, 1, 1, seed=2),  # lists outgrow shared memory
+    lambda: gen.er_graph(2000, 30000, 1, 40, seed=3),  # eight threads to a row
+    lambda: gen.ba_graph(4000, 4, 1, 100, seed=4),
+    lambda: gen.er_graph(3000, 1700, 1, 9, seed=5),  # most sources reach a few vertices
+    lambda: gen.rmat_graph(12, 16, wmin=1, wmax=3, seed=6),
+    lambda: gen.grid_graph(30, 30, wmin=1, wmax=1 << 27, seed=7),
+], ids=str)
+@pytest.mark.parametrize("team", [0, 32, 512])
+def test_dag_edges_counts_the_edges(graph, team):
+    """stats().dag_edges: the entries on shortest paths, in every form of the DAG build."""
+    g = graph()
+    src = np.arange(0, g.n, max(1, g.n // 60), dtype=np.uint32)
+    rows, cols, ws = g.edges()
+    edges = 0
+    for s in src:
+        d = oracle.sssp(g, int(s))[0]
+        edges += int(np.sum((d[rows] != np.iinfo(np.uint64).max) & (d[rows] + ws.astype(np.uint64) == d[cols])))
+    bc.bc_set_config(algorithm=bc.BC_ALGO_DELTA, team_threads=team)
+    with bc.Graph(g) as G:
+        G.compute(src, 0.5)
+        assert G.stats().dag_edges == edges
