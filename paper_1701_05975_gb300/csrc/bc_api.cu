@@ -773,24 +773,14 @@ int compute_plain(bc_graph* g, const uint32_t* sources, uint32_t k, double scale
   return status_from_dev(dev);
 }
 
-// 64-bit finaliser of SplitMix64 (Steele, Lea and Flood, OOPSLA 2014).
-uint64_t mix64(uint64_t z) {
-  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
-  z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-  return z ^ (z >> 31);
-}
-
 // True when the multiset of entries (v -> u, w) equals that of their reverses
-// (u -> v, w), compared through a sum mod 2^64 of a hash of each entry: exact
-// for a symmetric CSR, and an asymmetric one passes only with probability about
-// 2^-64.  O(nnz).
+// (u -> v, w), by entry_hash.  O(nnz).
 bool symmetric_by_hash(uint32_t n, const uint64_t* rp, const uint32_t* col, const uint32_t* w) {
   uint64_t fwd = 0, rev = 0;
   for (uint32_t v = 0; v < n; ++v)
     for (uint64_t e = rp[v]; e < rp[v + 1]; ++e) {
-      const uint64_t hw = mix64((uint64_t)w[e] + 0x9e3779b97f4a7c15ull);
-      fwd += mix64((((uint64_t)v << 32) | col[e]) ^ hw);
-      rev += mix64((((uint64_t)col[e] << 32) | v) ^ hw);
+      fwd += entry_hash(v, col[e], w[e]);
+      rev += entry_hash(col[e], v, w[e]);
     }
   return fwd == rev;
 }

@@ -8,6 +8,20 @@
 
 namespace bcgpu {
 
+// 64-bit finaliser of SplitMix64 (Steele, Lea and Flood, "Fast splittable
+// pseudorandom number generators", OOPSLA 2014).
+__host__ __device__ inline uint64_t mix64(uint64_t z) {
+  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+  z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+  return z ^ (z >> 31);
+}
+// Hash of one directed entry (a -> b, weight w).  The sums mod 2^64 over all
+// entries and over their reverses are equal for a symmetric CSR, and for
+// another only with probability about 2^-64.
+__host__ __device__ inline uint64_t entry_hash(uint32_t a, uint32_t b, uint32_t w) {
+  return mix64((((uint64_t)a << 32) | b) ^ mix64((uint64_t)w + 0x9e3779b97f4a7c15ull));
+}
+
 // Graph as the kernels see it (Sec. 3.1: CSR plus a parallel weight array,
 // here interleaved as one 8-byte {col, w} record per entry).
 struct GraphDev {

@@ -12,13 +12,6 @@
 namespace bcgpu {
 namespace {
 
-// 64-bit finaliser of SplitMix64 (Steele, Lea and Flood, OOPSLA 2014).
-__device__ __forceinline__ unsigned long long land_mix(unsigned long long z) {
-  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
-  z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-  return z ^ (z >> 31);
-}
-
 // f(v, e) for every entry e of every row v, `chunk` consecutive entries to a
 // warp (32 to 256: few enough that small graphs fill the GPU).  A warp per row
 // left one warp with a hub's whole row.  With a hub of 4 million neighbours and 8
@@ -51,17 +44,14 @@ __device__ __forceinline__ void land_entries(uint32_t n, uint64_t nnz, const uin
   }
 }
 
-// out[0] - out[1] = sum over entries of hash(v, u, w) - hash(u, v, w), mod
-// 2^64: zero for a symmetric CSR, and for another only with probability about
-// 2^-64.
+// out[0], out[1]: sums of entry_hash over the entries and over their reverses.
 __global__ void land_symmetry_kernel(uint32_t n, uint64_t nnz, uint32_t chunk, const uint64_t* __restrict__ row_ptr,
                                      const uint2* __restrict__ adj, unsigned long long* out) {
   unsigned long long fwd = 0, rev = 0;
   land_entries(n, nnz, row_ptr, chunk, [&](uint32_t v, uint64_t e) {
     const uint2 x = adj[e];
-    const unsigned long long hw = land_mix((unsigned long long)x.y + 0x9e3779b97f4a7c15ull);
-    fwd += land_mix((((unsigned long long)v << 32) | x.x) ^ hw);
-    rev += land_mix((((unsigned long long)x.x << 32) | v) ^ hw);
+    fwd += entry_hash(v, x.x, x.y);
+    rev += entry_hash(x.x, v, x.y);
   });
   __syncwarp();
   for (int o = 16; o > 0; o >>= 1) {

@@ -107,19 +107,6 @@ static_assert(DEV_OK == BC_OK && DEV_ERR_INVALID == BC_ERR_INVALID && DEV_ERR_TI
 constexpr uint64_t kCtlBytes = 256;
 static_assert(sizeof(NaCtl) <= kCtlBytes, "control block must fit its reserved bytes");
 
-// 64-bit finaliser of SplitMix64 (Steele, Lea and Flood, "Fast splittable
-// pseudorandom number generators", OOPSLA 2014).
-__device__ __forceinline__ uint64_t mix64(uint64_t z) {
-  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
-  z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
-  return z ^ (z >> 31);
-}
-
-// Hash of one directed entry (a -> b, weight w).
-__device__ __forceinline__ uint64_t entry_hash(uint32_t a, uint32_t b, uint32_t w) {
-  return mix64((((uint64_t)a << 32) | b) ^ mix64((uint64_t)w + 0x9e3779b97f4a7c15ull));
-}
-
 // Strict slabs that the validation kernel initialises on the side (slots 0: none).
 struct NaFill {
   char* slabs;

@@ -1097,8 +1097,7 @@ struct SweepTeam {
   // Levels of the DAG from the source; order holds them back to back, lvl
   // their bounds.  A vertex without successors needs no level of its own
   // unless `all` asks for it.  Returns the number of levels.
-  __device__ __forceinline__ uint32_t sigma_levels(Idx* order, Idx* lvl, bool rows, bool all, bool dropped,
-                                                   bool shallow) {
+  __device__ __forceinline__ uint32_t sigma_levels(Idx* order, Idx* lvl, bool rows, bool all, bool shallow) {
     if (t == 0) {
       node[s].sig = 1.0;
       order[0] = (Idx)s;
@@ -1118,8 +1117,9 @@ struct SweepTeam {
 #pragma unroll
         for (int q = 0; q < N; ++q) {
           const bool multi = on[q] && test_bit(bits1, u[q]);
-          // a listed successor with one predecessor has successors itself; of the others, look
-          look[q] = !all && (multi || !dropped);
+          // after drop_leaves a listed successor with one predecessor has successors itself; of the
+          // others, look
+          look[q] = !all && multi;
           if (on[q]) on[q] = release(u[q], sv, multi);
         }
 #pragma unroll
@@ -1526,7 +1526,7 @@ struct SweepTeam {
         clear_bits0();
       }
       lap(0);
-      if (!CHECK || err == DEV_OK) nlev = sigma_levels(qa, qb, over, all, drop, rounds < SW_DEEP);
+      if (!CHECK || err == DEV_OK) nlev = sigma_levels(qa, qb, over, all, rounds < SW_DEEP);
       lap(2);
       if (a.phase_cap < (uint64_t)rounds + advances + nlev) err = DEV_ERR_TIMEOUT;
       if (a.flags & RUN_FORWARD_ONLY) {
