@@ -78,7 +78,9 @@ extern "C" {
                              bucket_width), started from landmark bounds on graphs where those help; then the
                              shortest-path DAG as compact lists, sigma pushed down it in hop-depth levels, and
                              the dependency pull of Algorithm 3 over those levels in reverse.  Same results; far
-                             fewer synchronised steps, and only the entries that the landmark bounds leave. */
+                             fewer synchronised steps, and only the entries that the landmark bounds leave.
+                             Graphs of 2^31 vertices, or whose entries plus twice the vertices reach
+                             2^32 - 2^16, run BC_ALGO_STRICT instead. */
 
 /* ---- request states (bc_request_poll) ---------------------------------- */
 #define BC_REQ_QUEUED 0

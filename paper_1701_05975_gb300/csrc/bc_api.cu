@@ -350,11 +350,13 @@ RunCfg resolve(const bc_graph* g, uint32_t k, uint32_t force_algo = BC_ALGO_AUTO
   // the sweep schedule unless the configuration asks for the strict one, sets a
   // knob that only that one has, or it is the faster one
   const bool strict_knob = c.settle_in || c.bucket_width || c.warp_degree || c.team_degree || c.hot_vertices;
-  const uint32_t al = c.algorithm ? c.algorithm
-                                  : (strict_knob || g->n >= 0x80000000u || g->nnz + g->n >= (1ull << 32)
-                                     ? (uint32_t)BC_ALGO_STRICT
-                                     : (g->tuned.algo ? g->tuned.algo
-                                                    : (uint32_t)(!edges && strict_is_faster(g, k) ? BC_ALGO_STRICT : BC_ALGO_DELTA)));
+  uint32_t al = c.algorithm;
+  if (!al) {
+    if (strict_knob) al = BC_ALGO_STRICT;
+    else if (g->tuned.algo) al = g->tuned.algo;
+    else al = !edges && strict_is_faster(g, k) ? BC_ALGO_STRICT : BC_ALGO_DELTA;
+  }
+  if (!sweep_counts_fit(g->n, g->nnz)) al = BC_ALGO_STRICT;
   r.algo = (al == BC_ALGO_DELTA) ? ALGO_DELTA : ALGO_STRICT;
   r.algo_auto = c.algorithm == BC_ALGO_AUTO;
   const bool sweep = r.algo == ALGO_DELTA;
@@ -881,7 +883,8 @@ constexpr uint32_t LAND_MAX_N_FLAT = 32768;
 
 cudaError_t build_landmarks(bc_graph* g, const uint64_t* rp, const std::vector<uint64_t>& tdeg) {
   const uint32_t n = g->n;
-  if (g->dist_bits != 32 || n < LAND_MIN_N || g->nnz == 0 || !g->symmetric) return cudaSuccess;
+  if (g->dist_bits != 32 || n < LAND_MIN_N || g->nnz == 0 || !g->symmetric || !sweep_counts_fit(n, g->nnz))
+    return cudaSuccess;
   // without hubs the bounds only help small graphs (the prefix test keeps 28% of
   // the entries of a degree-16 random graph at n = 1024, 62% at 262144, all of a
   // grid's): do not pay for 68 searches to find that out
@@ -1592,8 +1595,8 @@ int bc_sssp_debug(bc_graph_t g, uint32_t s, uint64_t* out_dist, double* out_sigm
   if (s >= g->n) return fail(BC_ERR_INVALID, "source out of range");
   CK(cudaSetDevice(g->device));
   // the strict schedule's levels unless the sweep schedule is asked for by name
-  const bool sweep = config_snapshot().algorithm == BC_ALGO_DELTA;
-  RunCfg r = resolve(g, 1, sweep ? BC_ALGO_DELTA : BC_ALGO_STRICT);
+  RunCfg r = resolve(g, 1, config_snapshot().algorithm == BC_ALGO_DELTA ? BC_ALGO_DELTA : BC_ALGO_STRICT);
+  const bool sweep = r.algo == ALGO_DELTA;
   plan_sweep(g, r, 1, false);  // the arrays are read back from a slab
   // no plan_slots here, so the kernel's shared memory limit is raised by this query alone
   int bps = 0;
@@ -1725,9 +1728,11 @@ int autotune(bc_graph* g, const uint32_t* sources, uint32_t k_probe) {
   // a pinned schedule, or a knob that only the strict one has, leaves one schedule
   const bool strict_knob = user.settle_in || user.warp_degree || user.team_degree || user.hot_vertices ||
                            (user.bucket_width && user.algorithm != BC_ALGO_DELTA);
-  const bool try_sweep =
-      user.algorithm == BC_ALGO_DELTA || (user.algorithm == BC_ALGO_AUTO && (!strict_knob || !g->symmetric));
-  const bool try_strict = user.algorithm == BC_ALGO_STRICT || (user.algorithm == BC_ALGO_AUTO && g->symmetric);
+  const bool fits_sweep = sweep_counts_fit(g->n, g->nnz);
+  const bool try_sweep = fits_sweep && (user.algorithm == BC_ALGO_DELTA ||
+                                        (user.algorithm == BC_ALGO_AUTO && (!strict_knob || !g->symmetric)));
+  const bool try_strict = !fits_sweep || user.algorithm == BC_ALGO_STRICT ||
+                          (user.algorithm == BC_ALGO_AUTO && g->symmetric);
   // sweep schedule: team size x bucket width (one bucket under landmark
   // bounds), then sources in flight
   double sweep_ms = 1e300;

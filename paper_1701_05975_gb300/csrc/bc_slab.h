@@ -33,6 +33,13 @@ inline uint32_t active_vertices(uint32_t n, const uint64_t* row_ptr, const uint3
   return last;
 }
 
+// Whether the sweep schedule's 32-bit counts hold: vertex ids in signed words,
+// DAG lists of every entry plus two words per vertex, and room for a walk's last
+// stride.  Larger graphs run the strict schedule.
+inline bool sweep_counts_fit(uint32_t n, uint64_t nnz) {
+  return n < 0x80000000u && nnz + 2ull * n < (1ull << 32) - (1u << 16);
+}
+
 // What a workspace's slabs hold: the layouts and the values their arrays keep
 // between sources differ by schedule.
 enum SlabKind : int { SLAB_STRICT = 0, SLAB_SWEEP = 1, SLAB_NONE = 2 };

@@ -74,3 +74,12 @@ def test_teams_per_sm_by_registers_and_shared_memory(tmp_path):
     std::cout << sweep_teams_per_sm(32, 256, make_layout(n, 32, SLAB_NONE).smem) << " "
               << sweep_teams_per_sm(32, 128, make_layout(n, 32, SLAB_NONE).smem) << " ";""")
     assert [int(x) for x in got] == [8, 7, 4, 3, 2, 2, 1, 1, 4, 8, 4, 4, 3, 3]
+
+
+def test_sweep_counts_stay_in_32_bits(tmp_path):
+    """A DAG of every entry with a list per vertex must not wrap the list counter."""
+    sizes = [(1 << 20, 1 << 25), (1 << 31, 10), ((1 << 31) - 1, 0), (10**9, 2 * 10**9), (10**9, 23 * 10**8),
+             (2, (1 << 32) - 65541), (2, (1 << 32) - 65540)]
+    got = run_cpp(tmp_path, "".join(f'  std::cout << sweep_counts_fit({n}u, {m}ull) << " ";\n' for n, m in sizes))
+    assert [x == "1" for x in got] == [n < 1 << 31 and m + 2 * n < (1 << 32) - (1 << 16) for n, m in sizes]
+    assert got == ["1", "0", "0", "1", "0", "1", "0"]
