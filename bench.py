@@ -105,8 +105,10 @@ def edge_units(g, opts):
 # per reached vertex 80 B.
 BYTES_PER_ENTRY = 64
 BYTES_PER_VERTEX = 80
-# the kernel the benchmark workloads run and the primitives it is built from
-KERNEL_SRC = [os.path.join(ROOT, "paper_1701_05975_gb300", "csrc", f) for f in ("bc_sweep.cuh", "bc_team.cuh")]
+# the kernel the benchmark workloads run, the primitives it is built from, and what else sets its
+# traffic: the landmarks, the slabs and the limits shared with them
+KERNEL_SRC = [os.path.join(ROOT, "paper_1701_05975_gb300", "csrc", f)
+              for f in ("bc_sweep.cuh", "bc_team.cuh", "bc_land.cu", "bc_slab.h", "bc_common.h")]
 
 
 def reach_model(g, sources, directed=False, sample=32):
@@ -141,9 +143,11 @@ def kernel_digest():
     return hashlib.sha256(b"".join(open(f, "rb").read() for f in KERNEL_SRC)).hexdigest()[:16]
 
 
-def load_traffic(workload):
-    """DRAM bytes per launch of the batched kernel from the committed ncu
-    summary, or None when the summary is missing or the kernel changed since."""
+def load_traffic(workload, run=None):
+    """DRAM bytes per launch of the sweep kernel from the committed ncu
+    summary, or None when the summary is missing, the kernel changed since, or
+    `run` (algorithm, sources, team_threads and slots of the launch to be
+    described) is not the run that was captured."""
     path = os.path.join(ROOT, "profiles", f"bc_batched_{workload}.md")
     if not os.path.exists(path):
         return None
@@ -152,6 +156,10 @@ def load_traffic(workload):
     t = re.search(r"traffic_bytes_per_launch:\s*([0-9.eE+]+)", text)
     if not m or not t or m.group(1) != kernel_digest():
         return None
+    for key, value in (run or {}).items():
+        c = re.search(rf"^captured_{key}:\s*(\S+)", text, re.M)
+        if not c or c.group(1) != str(value):
+            return None
     return float(t.group(1))
 
 
@@ -709,7 +717,9 @@ def main():
     launch_avg_s = statistics.mean(launch_ms) * 1e-3
     achieved = alg_bytes / launch_avg_s / 1e9
     peak, peak_kind = peaks()
-    traffic = load_traffic(args.workload)
+    algorithm = "sweep" if int(st.algorithm) == 2 else "strict"
+    traffic = load_traffic(args.workload, dict(algorithm=algorithm, sources=k, team_threads=int(st.team_threads),
+                                               slots=int(st.slots)))
 
     line = {
         "metric": metric_name(opts),
@@ -729,7 +739,7 @@ def main():
                    "graph_prep_s": round(prep_s, 3),
                    "launch": "CUDA graph (bc_step_launch)" if use_graph else (
                        "bc_edge_compute_async per step" if edge else "bc_compute_async per step"),
-                   "algorithm": "sweep" if int(st.algorithm) == 2 else "strict",
+                   "algorithm": algorithm,
                    "relabeled_by_degree": bool(G.info().relabeled), "dist_bits": int(G.info().dist_bits)},
         "e2e": {"value": whole_job_gteps(ws, k, m, e2e_s), "unit": "GTEPS", "h2d_bytes_per_step": 4 * k,
                 "d2h_bytes_per_step": 8 * g.n + (8 * g.nnz if edge else 0)},
@@ -744,7 +754,8 @@ def main():
                      "model_frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
                      # ncu-measured DRAM bytes per launch over the same launch time
                      "frac_measured": (traffic / launch_avg_s / 1e9 / peak) if traffic else None,
-                     "alg_bytes_per_launch": alg_bytes, "kernel": "bc_sweep_kernel" if int(st.algorithm) == 2 else "bc_batched_kernel"},
+                     "alg_bytes_per_launch": alg_bytes,
+                     "kernel": "bc_sweep_kernel" if algorithm == "sweep" else "bc_batched_kernel"},
         "clocks": clk,
         "run_stats": {"phases_per_source": st.phases / max(st.sources, 1),
                       "refills_per_source": st.refills / max(st.sources, 1),
