@@ -330,3 +330,18 @@ def test_dag_edges_counts_the_edges(graph, team):
     with bc.Graph(g) as G:
         G.compute(src, 0.5)
         assert G.stats().dag_edges == edges
+
+
+@pytest.mark.parametrize("graph", [lambda: gen.er_graph(1024, 8192, 1, 3, seed=1), lambda: gen.ba_graph(3000, 4, 1, 50, seed=6)],
+                         ids=["small-weights", "landmarks"])
+def test_plain_form_keeps_its_split_width(graph):
+    """The automatic schedule of the batched mode does not change the plain form's settings."""
+    g = graph()
+    src = np.arange(200, dtype=np.uint32)
+    with bc.Graph(g) as G:
+        bc.bc_set_config(algorithm=bc.BC_ALGO_DELTA)
+        G.compute(src, 0.5)
+        width = G.stats().bucket_width
+        bc.bc_set_config(mode=bc.BC_MODE_PLAIN, algorithm=bc.BC_ALGO_AUTO)
+        assert_bc_close(G.compute(src, 0.5), oracle.bc(g, src, 0.5))
+        assert G.stats().bucket_width == width
