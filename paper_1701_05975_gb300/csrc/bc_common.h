@@ -28,8 +28,8 @@ struct GraphDev {
   uint32_t n;
   uint64_t nnz;
   const uint64_t* row_ptr;  // [n + 1]
-  const uint2* adj;         // [nnz] {neighbour, weight}, or nullptr when adjp is used
-  const uint32_t* adjp;     // [nnz] neighbour | weight << col_bits (graphs where both fit 32 bits)
+  const uint2* adj;         // [nnz] {neighbour, weight}; nullptr where adjp and kadj serve both schedules
+  const uint32_t* adjp;     // [nnz] neighbour | weight << col_bits (where both fit 32 bits): the strict schedule's
   uint32_t col_bits;        // bits of the neighbour id in an adjp word
   const uint32_t* dnode;    // [n] Delta_node(v) = min incident (directed: outgoing) weight, UINT32_MAX if none
   // Undirected graphs (nullptr otherwise): the second smallest incident weight
