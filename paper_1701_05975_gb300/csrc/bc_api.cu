@@ -315,17 +315,22 @@ uint32_t strict_team_default(const bc_graph* g) {
 //   (1.22), 0.92 to 64 (1.06), 1.13 to 128;
 //   a list of DAG edges that outgrows the strict slabs (ties above 2) costs a second scan:
 //   1.0 at weights to 3, and hubs make it worse (R-MAT 2^12 at unit weights 1.34);
-//   its teams are narrow, so few sources favour the sweep's wide ones from 1536 vertices
-//   on (Erdos-Renyi n = 8192, weights to 4: 1.65 at 40 sources, 1.04 at 304, 0.68 at
-//   608); 20 and more entries walked per vertex make the strict teams wide: then only few
-//   sources of a small graph (Erdos-Renyi of degree 32, n = 700, weights to 4: 0.66 at 40,
-//   1.28 at 700);
+//   its teams are narrow, so from 1536 vertices on sources that leave the sweep wider ones
+//   favour it (Erdos-Renyi n = 6315, degree 16, weights to 4: 1.54 at 152 sources, 1.04 at
+//   304, 0.71 from 305 on, where the sweep's teams are as narrow); 20 and more entries
+//   walked per vertex make the strict teams wide: then only few sources of a small graph
+//   (Erdos-Renyi of degree 32, n = 700, weights to 4: 0.66 at 40, 1.28 at 700);
+//   with landmarks only dense rows in shared memory, one thread to a row (Erdos-Renyi of
+//   degree 32, n = 1400: weights to 8, ties 1.89, 0.26 at 40 sources, 0.68 at 1216; to 16,
+//   ties 1.47, 0.70 and 1.8);
 //   sparse graphs, not probed: grids 0.71 and 0.96 at weights to 1 and 2 (n = 900), 0.76 / 0.83
 //   / 0.90 / 1.01 at weights to 1 / 2 / 3 / 5 (n = 40,000, 1216 sources), 1.5 and more at 304.
 bool strict_is_faster(const bc_graph* g, uint32_t k) {
-  if (g->kadj || !g->symmetric) return false;
+  if (!g->symmetric) return false;
   const double walked = (double)g->nnz * (g->directed ? 2.0 : 1.0) / g->n;
   const bool few = k && k <= (uint32_t)g->sm_count;
+  if (g->kadj)
+    return !g->relabeled && g->n >= 1000 && g->n <= SWEEP_SMEM_N && walked >= 24.0 && g->ties > (few ? 1.4 : 1.8);
   if (g->ties < 0.0) {
     if (g->n < LAND_MIN_N) return !g->directed && walked >= 6.0 && walked < 20.0 && g->max_w < 0.5 * walked;
     if (sweep_sparse(g) && !g->relabeled)
@@ -334,7 +339,7 @@ bool strict_is_faster(const bc_graph* g, uint32_t k) {
   }
   if (walked >= 20.0) return g->n <= SWEEP_SMEM_N && few && g->ties > 1.2;
   if (g->n <= SWEEP_SMEM_N) return few ? walked >= 6.0 && g->ties > 1.5 : g->ties > 1.25;
-  if (g->n >= 32768 || (k && k < (uint64_t)g->sm_count * (1024 / strict_team_default(g)))) return false;
+  if (g->n >= 32768 || (k && k <= (uint64_t)g->sm_count * (512 / strict_team_default(g)))) return false;
   return g->ties > 1.1 && (g->ties < 2.0 || !g->relabeled) && (walked >= 6.0 || g->n < 16000);
 }
 

@@ -191,8 +191,10 @@ def test_dense_rows_without_landmarks_run_in_slabs(n, m):
     (lambda: gen.er_graph(1024, 8192, 1, 3, seed=1), 1024, True),
     (lambda: gen.er_graph(1024, 8192, 1, 3, seed=1), 100, True),
     (lambda: gen.er_graph(1024, 8192, 1, 100, seed=1), 1024, False),
-    (lambda: gen.er_graph(9000, 72000, 1, 8, seed=2), 608, True),
-    (lambda: gen.er_graph(9000, 72000, 1, 8, seed=2), 607, False),
+    (lambda: gen.er_graph(9000, 72000, 1, 8, seed=2), 305, True),
+    (lambda: gen.er_graph(9000, 72000, 1, 8, seed=2), 304, False),
+    (lambda: gen.er_graph(1400, 22400, 1, 16, seed=7), 100, True),  # landmarks
+    (lambda: gen.er_graph(1400, 22400, 1, 16, seed=7), 1400, False),
     (lambda: gen.er_graph(2000, 32000, 1, 4, seed=3), 2000, False),
     (lambda: gen.er_graph(200, 1600, 1, 2, seed=4), 200, True),
     (lambda: gen.grid_graph(40, 40, wmin=1, wmax=2, seed=5), 1000, True),
