@@ -312,7 +312,7 @@ uint32_t strict_team_default(const bc_graph* g) {
 // graphs and 5007 runs, strict / sweep time:
 //   Erdos-Renyi of degree 16, all sources, n = 1024: 0.61 at weights to 3 (ties 2.1), 0.93
 //   to 16 (1.22), 1.45 to 64 (1.06); n = 8192, 1216 sources: 0.73 to 6 (1.6), 0.78 to 16
-//   (1.22), 0.92 to 64 (1.06), 1.13 to 128;
+//   (1.22), 0.92 to 64 (1.06), 1.13 to 128; n = 1400, 608 sources 0.59 to 16 (1.24);
 //   a list of DAG edges that outgrows the strict slabs (ties above 2) costs a second scan:
 //   1.0 at weights to 3, and hubs make it worse (R-MAT 2^12 at unit weights 1.34);
 //   its teams are narrow, so from 1536 vertices on sources that leave the sweep wider ones
@@ -338,7 +338,11 @@ bool strict_is_faster(const bc_graph* g, uint32_t k) {
     return false;
   }
   if (walked >= 20.0) return g->n <= SWEEP_SMEM_N && few && g->ties > 1.2;
-  if (g->n <= SWEEP_SMEM_N) return few ? walked >= 6.0 && g->ties > 1.5 : g->ties > 1.25;
+  if (g->n <= SWEEP_SMEM_N) {
+    if (few || (k && walked < 6.0 && k <= 2ull * g->sm_count)) return walked >= 6.0 && g->ties > 1.5;
+    // above 1150 vertices shared memory holds three teams to an SM: the sweep's second wave comes sooner
+    return g->ties > (g->n > 1150 && (!k || k > 3ull * g->sm_count) ? 1.15 : 1.25);
+  }
   if (g->n >= 32768 || (k && k <= (uint64_t)g->sm_count * (512 / strict_team_default(g)))) return false;
   return g->ties > 1.1 && (g->ties < 2.0 || !g->relabeled) && (walked >= 6.0 || g->n < 16000);
 }
