@@ -174,10 +174,13 @@ __global__ void na_validate_prep(uint32_t n, uint64_t nnz, const uint64_t* __res
       atomicExch(&ctl->counter[1], PARKED);
     }
   } else {
-    for (uint32_t slot = blockIdx.x - rows; slot < fill.slots; slot += gridDim.x - rows) {
-      uint64_t* d = reinterpret_cast<uint64_t*>(fill.slabs + slot * fill.stride);
-      uint64_t* acc = reinterpret_cast<uint64_t*>(fill.slabs + slot * fill.stride + fill.off_acc);
-      for (uint32_t v = threadIdx.x; v < n; v += blockDim.x) {
+    // few slabs: several blocks to each
+    const uint32_t blocks = gridDim.x - rows, parts = max(1u, blocks / fill.slots);
+    for (uint64_t j = blockIdx.x - rows; j < (uint64_t)fill.slots * parts; j += blocks) {
+      char* slab = fill.slabs + j / parts * fill.stride;
+      uint64_t* d = reinterpret_cast<uint64_t*>(slab);
+      uint64_t* acc = reinterpret_cast<uint64_t*>(slab + fill.off_acc);
+      for (uint64_t v = j % parts * blockDim.x + threadIdx.x; v < n; v += (uint64_t)parts * blockDim.x) {
         d[v] = ~0ull;
         acc[v] = 0;
       }
@@ -319,7 +322,7 @@ extern "C" int bc_compute_noalloc(const uint64_t* d_row_ptr, const uint32_t* d_c
     const uint64_t work = std::max<uint64_t>(n, k);
     const uint32_t rows = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((work + 255) / 256, (uint64_t)sms * 8));
     const NaFill fill{slabs, strict_lay.stride, strict_lay.off_acc, fill_early ? strict_slots : 0u};
-    na_validate_prep<<<rows + std::min<uint32_t>(fill.slots, 4u * sms), 256, 0, st>>>(
+    na_validate_prep<<<rows + (fill.slots ? 4u * sms : 0u), 256, 0, st>>>(
         n, nnz, d_row_ptr, d_col_idx, d_w, d_sources, k, adj, dnode, ctl, strict_from, strict_to, rows, fill);
     e = cudaGetLastError();
   }

@@ -242,6 +242,26 @@ def test_noalloc_schedule_by_the_largest_weight():
         assert_bc_close(out.cpu().numpy(), oracle.bc(g, src, 0.5, nthreads=8))
 
 
+@pytest.mark.parametrize("n,k", [(700, 700), (40000, 9), (250000, 2)])
+def test_noalloc_pinned_strict_fills_its_slabs(n, k):
+    """Many slabs with a block each, and few that several blocks share; the second call finds the first one's."""
+    torch = pytest.importorskip("torch")
+    g = gen.grid_graph(n // 50, 50, wmin=1, wmax=20, seed=n)
+    src = np.arange(k, dtype=np.uint32)
+    dev = lambda x, t: torch.from_numpy(np.ascontiguousarray(x).view(t)).cuda()  # noqa: E731
+    rp, col, w, d_src = dev(g.row_ptr, np.int64), dev(g.col, np.int32), dev(g.w, np.int32), dev(src, np.int32)
+    out, status = torch.empty(g.n, dtype=torch.float64, device="cuda"), torch.full((1,), 9, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    bc.bc_set_config(algorithm=bc.BC_ALGO_STRICT)
+    want = oracle.bc(g, src, 0.5, nthreads=8)
+    for _ in range(2):
+        bc.bc_compute_noalloc(rp.data_ptr(), col.data_ptr(), w.data_ptr(), g.n, g.nnz, d_src.data_ptr(), k, 0.5,
+                              out.data_ptr(), status.data_ptr(), 0)
+        torch.cuda.synchronize()
+        assert int(status.item()) == bc.BC_OK
+        assert_bc_close(out.cpu().numpy(), want)
+
+
 def csr(n, rows):
     """CSR from {vertex: [(neighbour, weight), ...]}, as given: nothing is made symmetric."""
     deg = np.zeros(n + 1, np.uint64)
